@@ -163,13 +163,15 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
 
 /* Context options (dof_ctx_set_option). */
 #define DOF_OPT_BVH_BUILDER 1
-#define DOF_BVH_PLOC 0   /* default: PLOC clustering over the Morton order (higher tree quality) */
+#define DOF_BVH_PLOC 0   /* default: a round of PLOC clustering over the Morton order, then top-down splits by a
+                          * binned surface-area heuristic (higher tree quality) */
 #define DOF_BVH_LBVH 1   /* Karras 2012 radix tree (faster build) */
 /* launch shape and scheduling of the persistent ray tracer (results do not depend on them) */
 #define DOF_OPT_TRACE_BLOCKS_PER_SM 2   /* 128-thread blocks per SM, 1..32 (default 8) */
 #define DOF_OPT_TRACE_REFILL_IDLE   3   /* refill a warp when this many lanes are idle, 1..32 (default 16) */
 #define DOF_OPT_TRACE_STEPS         4   /* traversal steps between refill checks, 1..256 (default 64) */
-#define DOF_OPT_PLOC_RADIUS         5   /* PLOC nearest-neighbour search radius, 1..256 (default 48) */
+#define DOF_OPT_PLOC_RADIUS         5   /* nearest-neighbour search radius of the clustering round, 1..256
+                                         * (default 48) */
 #define DOF_OPT_BVH_WIDTH           6   /* tree the rays traverse: 4 (default) = the binary tree collapsed
                                          * to 4-wide nodes, 2 = the binary tree; same hits either way */
 #define DOF_OPT_RAY_ORDER_GRID      7   /* order in which the tracer takes a block's rays: grouped by the
@@ -215,8 +217,8 @@ const char *dof_last_error(void);
 /* ---- scene (Section 4.2: the acceleration structure) ------------------------- */
 
 /* Upload a triangle scene and build its BVH on the device from 63-bit Morton codes of
- * the triangle centroids: PLOC agglomerative clustering (Meister and Bittner 2018)
- * by default, or the LBVH radix tree of Karras 2012 (DOF_OPT_BVH_BUILDER); two child
+ * the triangle centroids: by default one round of PLOC clustering (Meister and Bittner
+ * 2018), then top-down splits by a binned surface-area heuristic (Wald 2007); or the LBVH radix tree of Karras 2012 (DOF_OPT_BVH_BUILDER); two child
  * boxes per node.  The binary tree is then collapsed top-down into nodes of four child
  * boxes (the largest-area child is opened until four remain).  Up to 64
  * "large" triangles (box extent above 1/16 of the scene's centroid extent, e.g. a

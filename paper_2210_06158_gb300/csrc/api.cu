@@ -43,6 +43,12 @@ int dof_alloc(DofCtx *ctx, size_t bytes, void **ptr, size_t *acc) {
         return dof_set_error(DOF_ERR_BUDGET, "allocation of %zu bytes exceeds the budget (%zu of %zu in use)", bytes,
                              (size_t)ctx->in_use, ctx->budget);
     cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e == cudaErrorMemoryAllocation && ctx->pool) {
+        // the scratch that the pool keeps between calls goes back to the device first
+        cudaGetLastError();
+        cudaMemPoolTrimTo(ctx->pool, 0);
+        e = cudaMalloc(ptr, bytes);
+    }
     if (e != cudaSuccess) {
         *ptr = nullptr;
         return dof_cuda_check(e, "cudaMalloc");
@@ -371,6 +377,8 @@ extern "C" size_t dof_ctx_bytes_in_use(const DofCtx *ctx) { return ctx ? (size_t
 // scene
 // ---------------------------------------------------------------------------
 
+constexpr size_t kPoolKeep = (size_t)256 << 20;
+
 extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts, const uint32_t *tri_idx,
                                 const uint32_t *tri_mat, uint32_t n_tris, void *stream, DofScene **out) {
     if (!ctx || !out || (n_tris && (!xyz || !tri_idx || !n_verts)))
@@ -405,6 +413,8 @@ extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts,
         rc = dof_cuda_check(cudaStreamSynchronize(st), "scene triangle index");
     }
     cudaFree(d_xyz); cudaFree(d_idx); cudaFree(d_mat);
+    // the pool keeps at most kPoolKeep of the build's scratch for the next call
+    if (ctx->pool) cudaMemPoolTrimTo(ctx->pool, kPoolKeep);
     if (rc != DOF_OK) {
         dof_free(ctx, s->tris, s->tris_bytes);
         dof_free(ctx, s->prim_k, 4 * (size_t)n_tris);

@@ -1,17 +1,21 @@
 // Device-built BVH of libdof (the acceleration structure whose build the paper
 // counts in its ray-trace time, Section 4.2).
 //
-// LBVH after Karras, "Maximizing Parallelism in the Construction of BVHs, Octrees,
-// and k-d Trees" (HPG 2012): 63-bit Morton codes of triangle centroids (21 bits per
-// axis: scenes with a ground plane hundreds of metres wide still resolve centimetre
-// detail), a stable LSD radix sort written here (8-bit digits, warp-matched ranks), one
-// thread per internal node to find its key range and
-// split (ties between equal codes broken by the sorted index), then a
-// bottom-up box refit in which the second thread to reach a node merges its two
-// children (atomic arrival counter, no waiting).  Nodes hold both child boxes so that
-// traversal fetches one node per step.
+// Both builders start from the triangles sorted by the 63-bit Morton codes of their
+// centroids (21 bits per axis: scenes with a ground plane hundreds of metres wide still
+// resolve centimetre detail; a stable LSD radix sort written here, 8-bit digits,
+// warp-matched ranks).  The default one joins neighbours in one round of PLOC clustering
+// and splits the clusters top-down by a binned surface-area heuristic.  The other is the
+// LBVH after Karras, "Maximizing Parallelism in the Construction of BVHs, Octrees, and
+// k-d Trees" (HPG 2012): one thread per internal node finds its key range and split
+// (ties between equal codes broken by the sorted index), then a bottom-up box refit in
+// which the second thread to reach a node merges its two children (atomic arrival
+// counter, no waiting).  Nodes hold both child boxes so that traversal fetches one node
+// per step.
 
 #include "dof_internal.cuh"
+
+#include <algorithm>
 
 namespace {
 
@@ -25,13 +29,33 @@ __device__ __forceinline__ float3 vtx(const float *xyz, uint32_t i) {
     return make_float3(xyz[3 * (size_t)i], xyz[3 * (size_t)i + 1], xyz[3 * (size_t)i + 2]);
 }
 
+// min (c < 3) and max (c >= 3) of v over the block, then one global atomic per component.
+// The kernels that call it stride over their elements with a few blocks per SM: one set of
+// atomics per warp of the whole input kept the six words' lines busy (64 us at 496k
+// triangles; 8 us this way)
+__device__ __forceinline__ void block_bounds(const float *v, int *out) {
+    __shared__ int s[6];
+    if (threadIdx.x < 6) s[threadIdx.x] = threadIdx.x < 3 ? 0x7FFFFFFF : (int)0x80000000;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int o = ord_of(v[k]);
+        const int w = k < 3 ? __reduce_min_sync(0xffffffffu, o) : __reduce_max_sync(0xffffffffu, o);
+        if ((threadIdx.x & 31) == 0) {
+            if (k < 3) atomicMin(&s[k], w);
+            else atomicMax(&s[k], w);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) atomicMin(&out[threadIdx.x], s[threadIdx.x]);
+    else if (threadIdx.x < 6) atomicMax(&out[threadIdx.x], s[threadIdx.x]);
+}
+
 // centroids and their bounds (order-preserving int atomics); flags bad indices
-__global__ void k_centroids(const float *xyz, uint32_t n_verts, const uint32_t *idx, uint32_t n,
-                            float4 *cen, int *bounds, int *bad) {
-    uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    float3 c = make_float3(0.f, 0.f, 0.f);
-    bool ok = t < n;
-    if (ok) {
+__global__ void __launch_bounds__(256) k_centroids(const float *xyz, uint32_t n_verts, const uint32_t *idx, uint32_t n,
+                                                   float4 *cen, int *bounds, int *bad) {
+    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         uint32_t i0 = idx[3 * (size_t)t], i1 = idx[3 * (size_t)t + 1], i2 = idx[3 * (size_t)t + 2];
         if (i0 >= n_verts || i1 >= n_verts || i2 >= n_verts) {
             atomicExch(bad, 1);
@@ -40,21 +64,12 @@ __global__ void k_centroids(const float *xyz, uint32_t n_verts, const uint32_t *
         float3 a = vtx(xyz, i0), b = vtx(xyz, i1), d = vtx(xyz, i2);
         float3 lo = make_float3(fminf(a.x, fminf(b.x, d.x)), fminf(a.y, fminf(b.y, d.y)), fminf(a.z, fminf(b.z, d.z)));
         float3 hi = make_float3(fmaxf(a.x, fmaxf(b.x, d.x)), fmaxf(a.y, fmaxf(b.y, d.y)), fmaxf(a.z, fmaxf(b.z, d.z)));
-        c = make_float3(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z));
-        cen[t] = make_float4(c.x, c.y, c.z, fmaxf(hi.x - lo.x, fmaxf(hi.y - lo.y, hi.z - lo.z)));
+        const float c[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
+        cen[t] = make_float4(c[0], c[1], c[2], fmaxf(hi.x - lo.x, fmaxf(hi.y - lo.y, hi.z - lo.z)));
+#pragma unroll
+        for (int k = 0; k < 3; k++) { v[k] = fminf(v[k], c[k]); v[3 + k] = fmaxf(v[3 + k], c[k]); }
     }
-    // block reduction of min/max through warp shuffles
-    float v[6] = {c.x, c.y, c.z, c.x, c.y, c.z};
-    if (!ok) { v[0] = v[1] = v[2] = INFINITY; v[3] = v[4] = v[5] = -INFINITY; }
-    for (int o = 16; o > 0; o >>= 1)
-        for (int k = 0; k < 6; k++) {
-            float w = __shfl_xor_sync(0xffffffffu, v[k], o);
-            v[k] = k < 3 ? fminf(v[k], w) : fmaxf(v[k], w);
-        }
-    if ((threadIdx.x & 31) == 0) {
-        for (int k = 0; k < 3; k++) atomicMin(&bounds[k], ord_of(v[k]));
-        for (int k = 3; k < 6; k++) atomicMax(&bounds[k], ord_of(v[k]));
-    }
+    block_bounds(v, bounds);
 }
 
 // threshold of a "large" triangle: its largest box extent above 1/16 of the largest
@@ -66,26 +81,24 @@ __device__ __forceinline__ float big_threshold(const int *bounds) {
 }
 
 // count the large triangles and the centroid bounds of the others
-__global__ void k_classify(const float4 *cen, uint32_t n, const int *bounds, int *n_big, int *small_bounds) {
-    uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    float thr = big_threshold(bounds);
-    bool ok = t < n;
-    float4 c = ok ? cen[t] : make_float4(0.f, 0.f, 0.f, 0.f);
-    bool big = ok && c.w > thr;
-    bool small = ok && !big;
-    unsigned nb = __popc(__ballot_sync(0xffffffffu, big));
-    float v[6] = {c.x, c.y, c.z, c.x, c.y, c.z};
-    if (!small) { v[0] = v[1] = v[2] = INFINITY; v[3] = v[4] = v[5] = -INFINITY; }
-    for (int o = 16; o > 0; o >>= 1)
-        for (int k = 0; k < 6; k++) {
-            float w = __shfl_xor_sync(0xffffffffu, v[k], o);
-            v[k] = k < 3 ? fminf(v[k], w) : fmaxf(v[k], w);
+__global__ void __launch_bounds__(256) k_classify(const float4 *cen, uint32_t n, const int *bounds, int *n_big,
+                                                  int *small_bounds) {
+    const float thr = big_threshold(bounds);
+    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    int nb = 0;
+    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+        const float4 q = cen[t];
+        if (q.w > thr) {
+            nb++;
+            continue;
         }
-    if ((threadIdx.x & 31) == 0) {
-        if (nb) atomicAdd(n_big, (int)nb);
-        for (int k = 0; k < 3; k++) atomicMin(&small_bounds[k], ord_of(v[k]));
-        for (int k = 3; k < 6; k++) atomicMax(&small_bounds[k], ord_of(v[k]));
+        const float c[3] = {q.x, q.y, q.z};
+#pragma unroll
+        for (int k = 0; k < 3; k++) { v[k] = fminf(v[k], c[k]); v[3 + k] = fmaxf(v[3 + k], c[k]); }
     }
+    nb = __reduce_add_sync(0xffffffffu, nb);
+    if ((threadIdx.x & 31) == 0 && nb) atomicAdd(n_big, nb);
+    block_bounds(v, small_bounds);
 }
 
 // spread the low 21 bits of v to every third bit
@@ -383,8 +396,10 @@ __global__ void k_tree_refs(const BvhNode *nodes, int n_nodes, int n_tree, int *
         else parent_leaf[~c[e]] = i;
     }
 }
-__global__ void k_tree_counts(int n_nodes, int n_tree, int root, const int *ref_node, const int *ref_leaf, int *bad) {
+__global__ void k_tree_counts(int n_nodes, int n_tree, const int *root_p, const int *ref_node, const int *ref_leaf,
+                              int *bad) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int root = *root_p;
     if (i == 0 && (root < 0 || root >= n_nodes)) atomicExch(bad, 9);
     if (i < n_nodes && ref_node[i] != (i == root ? 0 : 1)) atomicExch(bad, 9);
     if (i < n_tree && ref_leaf[i] != 1) atomicExch(bad, 9);
@@ -401,79 +416,723 @@ __global__ void k_depth(int n, const int *parent_node, const int *parent_leaf, i
 
 
 // ---------------------------------------------------------------------------
-// PLOC (Meister and Bittner, "Parallel Locally-Ordered Clustering for Bounding
-// Volume Hierarchy Construction", TVCG 2018): clusters start as the Morton-sorted
-// leaves; each finds its nearest neighbour within +-kPlocRadius positions by the
-// surface area of the merged box; mutual nearest neighbours merge into a new node;
-// the cluster array is compacted (order preserved) and the steps repeat.
+// One round of PLOC (Meister and Bittner, "Parallel Locally-Ordered Clustering for
+// Bounding Volume Hierarchy Construction", TVCG 2018) over the Morton-sorted leaves: each
+// finds its nearest neighbour within +-radius positions by the surface area of the merged
+// box; mutual nearest neighbours merge into a new node; the clusters are compacted, in
+// order.  A cluster is its box, with its reference (leaf ~k or node) in lo.w.
 // ---------------------------------------------------------------------------
-
-__global__ void k_ploc_init(const float4 *tris, int m, int *cid, float4 *clo, float4 *chi) {
+__global__ void k_ploc_init(const float4 *tris, int m, float4 *clo, float4 *chi) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= m) return;
     float3 lo, hi;
     tri_box(tris, k, lo, hi);
-    cid[k] = ~k;
-    clo[k] = make_float4(lo.x, lo.y, lo.z, 0.f);
+    clo[k] = make_float4(lo.x, lo.y, lo.z, __int_as_float(~k));
     chi[k] = make_float4(hi.x, hi.y, hi.z, 0.f);
 }
 
 // nearest neighbour by merged area; ties to the smaller index (symmetric cost, so the
-// globally cheapest pair is always mutual and every round merges at least once)
-__global__ void k_ploc_nn(int count, int radius, const float4 *clo, const float4 *chi, int *nn) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+// globally cheapest pair is always mutual).  The block's clusters and a halo of `radius` on
+// either side are staged in shared memory.
+constexpr int kNnThreads = 256, kNnMaxRadius = 256;
+__global__ void __launch_bounds__(kNnThreads) k_ploc_nn(int count, int radius, const float4 *clo, const float4 *chi, int *nn) {
+    extern __shared__ float4 sm_nn[];
+    const int base = blockIdx.x * kNnThreads - radius, tile = kNnThreads + 2 * radius;
+    float4 *sl = sm_nn, *sh = sm_nn + tile;
+    for (int e = threadIdx.x; e < tile; e += kNnThreads) {
+        const int j = min(max(base + e, 0), count - 1);
+        sl[e] = clo[j];
+        sh[e] = chi[j];
+    }
+    __syncthreads();
+    const int i = blockIdx.x * kNnThreads + threadIdx.x;
     if (i >= count) return;
-    float4 lo = clo[i], hi = chi[i];
+    const float4 lo = sl[i - base], hi = sh[i - base];
     float best = INFINITY;
     int bj = -1;
-    int j0 = max(0, i - radius), j1 = min(count - 1, i + radius);
+    const int j0 = max(0, i - radius), j1 = min(count - 1, i + radius);
     for (int j = j0; j <= j1; j++) {
         if (j == i) continue;
-        float4 l2 = clo[j], h2 = chi[j];
-        float a = half_area(make_float4(fminf(lo.x, l2.x), fminf(lo.y, l2.y), fminf(lo.z, l2.z), 0.f),
-                            make_float4(fmaxf(hi.x, h2.x), fmaxf(hi.y, h2.y), fmaxf(hi.z, h2.z), 0.f));
+        const float a = union_area(lo, hi, sl[j - base], sh[j - base]);
         if (a < best) { best = a; bj = j; }
     }
     nn[i] = bj;
 }
 
-// mutual pairs merge: the lower position creates the node and keeps the merged
-// cluster, the higher one drops out
-__global__ void k_ploc_merge(int count, int *cid, float4 *clo, float4 *chi, const int *nn, int *keep,
-                             int *node_count, BvhNode *nodes, int *parent_node, int *parent_leaf, int n_nodes,
-                             int *bad) {
+// mutual pairs merge: the lower position creates the node and keeps the merged cluster, the
+// higher one drops out
+__global__ void k_ploc_merge(int count, float4 *clo, float4 *chi, const int *nn, int *keep, int *node_count, BvhNode *nodes,
+                             int n_nodes, int *bad) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = i < count ? nn[i] : -1;
+    const bool mutual = j >= 0 && nn[j] == i, make = mutual && i < j;
+    // one atomic per warp for its new nodes
+    const unsigned lane = threadIdx.x & 31, b = __ballot_sync(0xffffffffu, make);
+    int id = 0;
+    if (lane == 0 && b) id = atomicAdd(node_count, __popc(b));
+    id = __shfl_sync(0xffffffffu, id, 0) + __popc(b & ((1u << lane) - 1u));
     if (i >= count) return;
-    int j = nn[i];
-    bool mutual = j >= 0 && nn[j] == i;
-    if (!mutual) { keep[i] = 1; return; }
-    if (i > j) { keep[i] = 0; return; }
-    int id = atomicAdd(node_count, 1);
-    if (id >= n_nodes) { atomicExch(bad, 4); keep[i] = 1; return; }
-    int a = cid[i], b = cid[j];
-    float4 l0 = clo[i], h0 = chi[i], l1 = clo[j], h1 = chi[j];
-    BvhNode nd;
-    nd.a = make_float4(l0.x, l0.y, l0.z, h0.x);
-    nd.b = make_float4(h0.y, h0.z, l1.x, l1.y);
-    nd.c = make_float4(l1.z, h1.x, h1.y, h1.z);
-    nd.r = make_int4(a, b, 0, 0);
-    nodes[id] = nd;
-    if (a < 0) parent_leaf[~a] = id; else parent_node[a] = id;
-    if (b < 0) parent_leaf[~b] = id; else parent_node[b] = id;
-    cid[i] = id;
-    clo[i] = make_float4(fminf(l0.x, l1.x), fminf(l0.y, l1.y), fminf(l0.z, l1.z), 0.f);
-    chi[i] = make_float4(fmaxf(h0.x, h1.x), fmaxf(h0.y, h1.y), fmaxf(h0.z, h1.z), 0.f);
+    if (!make) {
+        keep[i] = mutual ? 0 : 1;
+        return;
+    }
     keep[i] = 1;
+    if (id >= n_nodes) { atomicExch(bad, 4); return; }
+    const float4 l0 = clo[i], h0 = chi[i], l1 = clo[j], h1 = chi[j];
+    nodes[id] = make_node(l0, h0, __float_as_int(l0.w), l1, h1, __float_as_int(l1.w));
+    clo[i] = make_float4(fminf(l0.x, l1.x), fminf(l0.y, l1.y), fminf(l0.z, l1.z), __int_as_float(id));
+    chi[i] = make_float4(fmaxf(h0.x, h1.x), fmaxf(h0.y, h1.y), fmaxf(h0.z, h1.z), 0.f);
 }
 
-__global__ void k_ploc_scatter(int count, const int *keep, const int *pos, const int *cid, const float4 *clo,
-                               const float4 *chi, int *cid2, float4 *clo2, float4 *chi2) {
+__global__ void k_ploc_scatter(int count, const int *keep, const int *pos, const float4 *clo, const float4 *chi, float4 *clo2,
+                               float4 *chi2) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count || !keep[i]) return;
-    int o = pos[i];
-    cid2[o] = cid[i];
+    const int o = pos[i];
     clo2[o] = clo[i];
     chi2[o] = chi[i];
+}
+
+// ---------------------------------------------------------------------------
+// Top-down binned SAH (Wald, "On fast Construction of SAH-based Bounding Volume
+// Hierarchies", 2007) over the clusters that one PLOC round leaves.
+//
+// A segment is a contiguous range of the cluster array that becomes one subtree.  While
+// a segment holds more than kSahSmall clusters it is split by whole launches, one level at
+// a time: its chunks fill 16 bins per axis over the centroids' bounds (k_sah_bin), a warp
+// picks the cheapest of the 45 planes, writes the node and makes the two children
+// (k_sah_split), and the chunks move their clusters to the side they belong to, gathering
+// the children's centroid bounds (k_sah_part).  A segment of at most kSahSmall clusters is
+// finished by one warp in shared memory (k_sah_small).
+//
+// Why: the rays of the packet tracer step this tree.  PLOC alone left its large structure
+// to chance (97 to 150 node tests per packet at 496k triangles, by search radius); with the
+// planes of the surface-area heuristic at the top it takes ~70, whatever the radius.  One
+// PLOC round first halves the clusters to split and costs no quality: it pairs the
+// triangles that share a box.  Two or three rounds are worse by 3-6% at 496k triangles.
+// Measured against PLOC alone (radius 48): the 1080p tracer 0.440 -> 0.237 ms one ray per
+// lane, 0.194 -> 0.161 ms as packets, ten rays per pixel 1.239 -> 0.895 ms; the ray-cast
+// G-buffer 0.917 -> 0.615 ms; the 4K tracer (2M triangles) is even.
+//
+// The build itself is bound by latency at the top (a level of few segments cannot fill the
+// chip: 14 levels x 4 launches, 0.4 ms) and by the warps' serial splits at the bottom
+// (k_sah_small 0.67 ms).  Scratch comes from one pool block and the host reads back three
+// times, where every PLOC round used to end in a synchronisation (65 of them): upload and
+// first view of 496k triangles 7.1 -> 2.9 ms.
+// ---------------------------------------------------------------------------
+constexpr int kSahBins = 16;             // per axis
+constexpr int kSahSmall = 256;           // clusters a warp finishes alone (uint8 indices)
+constexpr int kSahChunk = 1024;          // clusters of one work item of a large segment
+constexpr int kSahThreads = 256;
+constexpr int kSahSlotInts = 3 * 7 * kSahBins;   // [axis][count, lo.xyz, hi.xyz][bin]
+constexpr int kSahMaxLevel = 48;         // from here on segments are halved by position, so that
+                                         // the tree is at most 48 + 31 + 1 levels deep
+
+struct SahSeg {
+    int begin, count, node, level;
+    int clo[3], chi[3];                  // bounds of the centroids (ordered ints)
+    int axis, bin, nl;                   // the plane: axis (-1: by position), last bin of the left side
+    int cur_l, cur_r;                    // clusters placed so far on either side
+    int child_l, child_r;                // their segments in the next level's table, -1 if small
+    int refs;                            // left/right child is a single cluster: bits 0 / 1
+};
+
+struct SahState {
+    int n_seg[2], n_item[2];             // per level parity
+    int n_small, small_next;             // small segments, and the next one to take
+    int count;                           // clusters
+};
+
+// the bin of a centroid: every kernel computes it here, with each rounding written out, so
+// that the counts of the bins and the sides of the partition agree
+__device__ __forceinline__ int sah_bin(float c, float lo, float ext) {
+    const float u = __fmul_rn(__fdiv_rn(__fsub_rn(c, lo), ext), (float)kSahBins);
+    return min(max((int)u, 0), kSahBins - 1);
+}
+__device__ __forceinline__ float sah_centre(float lo, float hi) { return __fmul_rn(0.5f, __fadd_rn(lo, hi)); }
+
+struct SahPlane {
+    int axis, bin, nl;                   // axis -1: no plane separates the clusters
+    float lo[2][3], hi[2][3];            // boxes of the two sides
+};
+
+// The cheapest plane of 3 x 15, by a full warp; bins[axis][component][bin] with ordered-int
+// bounds.  Lanes 0-15 take axes 0 then 2, lanes 16-31 axis 1.  cost = area x clusters on
+// either side; ties to the smaller (axis, bin).
+__device__ __forceinline__ SahPlane sah_select(const int *bins, unsigned lane) {
+    float best = INFINITY;
+    int best_id = 0x7FFFFFFF;
+    float bl[2][3], bh[2][3];
+    int bn = 0;
+#pragma unroll
+    for (int k = 0; k < 3; k++) bl[0][k] = bl[1][k] = bh[0][k] = bh[1][k] = 0.f;
+#pragma unroll
+    for (int round = 0; round < 2; round++) {
+        const int axis = round == 0 ? (int)(lane >> 4) : 2;
+        const int q = (int)(lane & 15u);
+        const int *b = bins + axis * 7 * kSahBins + q;
+        int n = b[0];
+        float lo[3], hi[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            lo[k] = n ? float_of(b[(1 + k) * kSahBins]) : INFINITY;
+            hi[k] = n ? float_of(b[(4 + k) * kSahBins]) : -INFINITY;
+        }
+        // inclusive prefix and suffix over the 16 bins
+        int np = n, ns = n;
+        float pl[3], ph[3], sl[3], sh[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) { pl[k] = sl[k] = lo[k]; ph[k] = sh[k] = hi[k]; }
+#pragma unroll
+        for (int o = 1; o < kSahBins; o <<= 1) {
+            const int tn = __shfl_up_sync(0xffffffffu, np, o, 16), un = __shfl_down_sync(0xffffffffu, ns, o, 16);
+            const bool up = q >= o, dn = q + o < kSahBins;
+            if (up) np += tn;
+            if (dn) ns += un;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const float a = __shfl_up_sync(0xffffffffu, pl[k], o, 16), c = __shfl_up_sync(0xffffffffu, ph[k], o, 16);
+                const float d = __shfl_down_sync(0xffffffffu, sl[k], o, 16), e = __shfl_down_sync(0xffffffffu, sh[k], o, 16);
+                if (up) { pl[k] = fminf(pl[k], a); ph[k] = fmaxf(ph[k], c); }
+                if (dn) { sl[k] = fminf(sl[k], d); sh[k] = fmaxf(sh[k], e); }
+            }
+        }
+        // the plane after bin q: bins 0 .. q against q + 1 .. 15
+        const int nr = __shfl_down_sync(0xffffffffu, ns, 1, 16);
+        float rl[3], rh[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            rl[k] = __shfl_down_sync(0xffffffffu, sl[k], 1, 16);
+            rh[k] = __shfl_down_sync(0xffffffffu, sh[k], 1, 16);
+        }
+        if (q < kSahBins - 1 && np > 0 && nr > 0) {
+            const float cost = half_area(make_float4(pl[0], pl[1], pl[2], 0.f), make_float4(ph[0], ph[1], ph[2], 0.f)) * (float)np +
+                               half_area(make_float4(rl[0], rl[1], rl[2], 0.f), make_float4(rh[0], rh[1], rh[2], 0.f)) * (float)nr;
+            if (cost < best && !(round == 1 && lane >= 16)) {
+                best = cost;
+                best_id = axis * kSahBins + q;
+                bn = np;
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    bl[0][k] = pl[k]; bh[0][k] = ph[k];
+                    bl[1][k] = rl[k]; bh[1][k] = rh[k];
+                }
+            }
+        }
+    }
+    float m = best;
+    int id = best_id;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float c = __shfl_xor_sync(0xffffffffu, m, o);
+        const int i = __shfl_xor_sync(0xffffffffu, id, o);
+        if (c < m || (c == m && i < id)) { m = c; id = i; }
+    }
+    SahPlane p;
+    if (id == 0x7FFFFFFF) {
+        p.axis = -1; p.bin = 0; p.nl = 0;
+#pragma unroll
+        for (int s = 0; s < 2; s++)
+#pragma unroll
+            for (int k = 0; k < 3; k++) p.lo[s][k] = p.hi[s][k] = 0.f;
+        return p;
+    }
+    const int win = __ffs(__ballot_sync(0xffffffffu, best_id == id)) - 1;
+    p.axis = id / kSahBins;
+    p.bin = id % kSahBins;
+    p.nl = __shfl_sync(0xffffffffu, bn, win);
+#pragma unroll
+    for (int s = 0; s < 2; s++)
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            p.lo[s][k] = __shfl_sync(0xffffffffu, bl[s][k], win);
+            p.hi[s][k] = __shfl_sync(0xffffffffu, bh[s][k], win);
+        }
+    return p;
+}
+
+__device__ __forceinline__ void sah_bins_clear(int *b, int tid, int threads) {
+    for (int e = tid; e < kSahSlotInts; e += threads) {
+        const int c = (e / kSahBins) % 7;
+        b[e] = c == 0 ? 0 : (c <= 3 ? 0x7FFFFFFF : (int)0x80000000);
+    }
+}
+
+// add a cluster's box to its bin of each axis (shared memory)
+__device__ __forceinline__ void sah_bins_add(int *b, const int *bin, float4 lo, float4 hi) {
+    const int l[3] = {ord_of(lo.x), ord_of(lo.y), ord_of(lo.z)}, h[3] = {ord_of(hi.x), ord_of(hi.y), ord_of(hi.z)};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        int *p = b + a * 7 * kSahBins + bin[a];
+        atomicAdd(p, 1);
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            atomicMin(p + (1 + k) * kSahBins, l[k]);
+            atomicMax(p + (4 + k) * kSahBins, h[k]);
+        }
+    }
+}
+
+// the table's segment `s` of parity `par` for clusters [begin, begin + count), with its bins
+// cleared and its chunks listed; the calling warp does it together
+__device__ __forceinline__ void sah_make_seg(SahSeg *segs, int *bins, int2 *items, int *n_item, int s, int max_items, int begin,
+                                             int count, int node, int level, unsigned lane, int *bad) {
+    if (lane == 0) {
+        SahSeg g;
+        g.begin = begin; g.count = count; g.node = node; g.level = level;
+        for (int k = 0; k < 3; k++) { g.clo[k] = 0x7FFFFFFF; g.chi[k] = (int)0x80000000; }
+        g.axis = -1; g.bin = 0; g.nl = 0;
+        g.cur_l = g.cur_r = 0;
+        g.child_l = g.child_r = -1;
+        g.refs = 0;
+        segs[s] = g;
+    }
+    sah_bins_clear(bins + (size_t)s * kSahSlotInts, (int)lane, 32);
+    const int n = (count + kSahChunk - 1) / kSahChunk;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(n_item, n);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (at + n > max_items) {
+        if (lane == 0) atomicExch(bad, 10);
+        return;
+    }
+    for (int k = (int)lane; k < n; k += 32) items[at + k] = make_int2(s, k);
+}
+
+// the clusters' first segment (one warp), or the small list, or nothing to split
+__global__ void k_sah_root(SahState *st, const int *pos, const int *keep, int m, const float4 *lo, SahSeg *segs, int *bins,
+                           int2 *items, int max_items, int4 *small, int *node_count, int *root, int *bad) {
+    const unsigned lane = threadIdx.x;
+    const int c = pos[m - 1] + keep[m - 1];
+    int node = -1;
+    if (lane == 0) {
+        st->count = c;
+        if (c == 1) {
+            *root = __float_as_int(lo[0].w);
+        } else {
+            node = atomicAdd(node_count, 1);
+            *root = node;
+            if (c <= kSahSmall) {
+                small[0] = make_int4(0, c, node, 0);
+                st->n_small = 1;
+            } else {
+                st->n_seg[0] = 1;
+            }
+        }
+    }
+    node = __shfl_sync(0xffffffffu, node, 0);
+    if (c > kSahSmall) sah_make_seg(segs, bins, items, &st->n_item[0], 0, max_items, 0, c, node, 0, lane, bad);
+}
+
+__device__ __forceinline__ int warp_min(int v) { return __reduce_min_sync(0xffffffffu, v); }
+__device__ __forceinline__ int warp_max(int v) { return __reduce_max_sync(0xffffffffu, v); }
+
+// the root segment's centroid bounds (the children's come with the partition)
+__global__ void __launch_bounds__(kSahThreads) k_sah_root_bounds(const SahState *st, const float4 *lo, const float4 *hi,
+                                                                 SahSeg *segs) {
+    const int c = st->count;
+    if (c <= kSahSmall) return;
+    int l[3] = {0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF}, h[3] = {(int)0x80000000, (int)0x80000000, (int)0x80000000};
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c; i += gridDim.x * blockDim.x) {
+        const float4 a = lo[i], b = hi[i];
+        const int e[3] = {ord_of(sah_centre(a.x, b.x)), ord_of(sah_centre(a.y, b.y)), ord_of(sah_centre(a.z, b.z))};
+#pragma unroll
+        for (int k = 0; k < 3; k++) { l[k] = min(l[k], e[k]); h[k] = max(h[k], e[k]); }
+    }
+    __shared__ int s[6];
+    if (threadIdx.x < 6) s[threadIdx.x] = threadIdx.x < 3 ? 0x7FFFFFFF : (int)0x80000000;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int a = warp_min(l[k]), b = warp_max(h[k]);
+        if ((threadIdx.x & 31) == 0) { atomicMin(&s[k], a); atomicMax(&s[3 + k], b); }
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) atomicMin(&segs[0].clo[threadIdx.x], s[threadIdx.x]);
+    else if (threadIdx.x < 6) atomicMax(&segs[0].chi[threadIdx.x - 3], s[threadIdx.x]);
+}
+
+// one level, step 1: the chunks of the large segments fill their bins (in shared memory, then
+// one global atomic per non-empty bin and component)
+__global__ void __launch_bounds__(kSahThreads) k_sah_bin(const SahState *st, int par, const SahSeg *segs, const int2 *items,
+                                                         const float4 *lo, const float4 *hi, int *bins) {
+    __shared__ int sb[kSahSlotInts];
+    const int n = st->n_item[par];
+    for (int it = blockIdx.x; it < n; it += gridDim.x) {
+        const int2 w = items[it];
+        const SahSeg &g = segs[w.x];
+        const int b0 = g.begin + w.y * kSahChunk, b1 = min(g.begin + g.count, b0 + kSahChunk);
+        float cl[3], ext[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            cl[k] = float_of(g.clo[k]);
+            ext[k] = __fsub_rn(float_of(g.chi[k]), cl[k]);
+        }
+        sah_bins_clear(sb, threadIdx.x, kSahThreads);
+        __syncthreads();
+        for (int i = b0 + (int)threadIdx.x; i < b1; i += kSahThreads) {
+            const float4 a = lo[i], b = hi[i];
+            const int bin[3] = {sah_bin(sah_centre(a.x, b.x), cl[0], ext[0]), sah_bin(sah_centre(a.y, b.y), cl[1], ext[1]),
+                                sah_bin(sah_centre(a.z, b.z), cl[2], ext[2])};
+            sah_bins_add(sb, bin, a, b);
+        }
+        __syncthreads();
+        int *gb = bins + (size_t)w.x * kSahSlotInts;
+        for (int e = threadIdx.x; e < kSahSlotInts; e += kSahThreads) {
+            const int c = (e / kSahBins) % 7, v = sb[e];
+            if (sb[e - c * kSahBins] == 0) continue;
+            if (c == 0) atomicAdd(&gb[e], v);
+            else if (c <= 3) atomicMin(&gb[e], v);
+            else atomicMax(&gb[e], v);
+        }
+        __syncthreads();
+    }
+}
+
+// step 2: a warp per large segment picks its plane, writes its node and makes its children
+__global__ void __launch_bounds__(128) k_sah_split(SahState *st, int par, SahSeg *segs, const int *bins, SahSeg *next,
+                                                   int *next_bins, int2 *next_items, int max_segs, int max_items, int4 *small,
+                                                   int max_small, BvhNode *nodes, int n_nodes, int *node_count, int *bad) {
+    const unsigned lane = threadIdx.x & 31;
+    const int n = st->n_seg[par];
+    const int warps = gridDim.x * (blockDim.x >> 5);
+    for (int s = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); s < n; s += warps) {
+        SahSeg &g = segs[s];
+        const int begin = g.begin, count = g.count, level = g.level, node = g.node;
+        SahPlane p = sah_select(bins + (size_t)s * kSahSlotInts, lane);
+        if (level >= kSahMaxLevel || p.nl <= 0 || p.nl >= count) p.axis = -1;
+        if (p.axis < 0) {
+            // by position: both sides take the whole segment's box (a superset is as safe)
+            p.nl = count / 2;
+            const int *b = bins + (size_t)s * kSahSlotInts;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int q = (int)(lane & 15u);
+                const float l = float_of(warp_min(b[(1 + k) * kSahBins + q])), h = float_of(warp_max(b[(4 + k) * kSahBins + q]));
+                p.lo[0][k] = p.lo[1][k] = l;
+                p.hi[0][k] = p.hi[1][k] = h;
+            }
+        }
+        const int nc[2] = {p.nl, count - p.nl};
+        int ref[2] = {0, 0}, child[2] = {-1, -1}, single = 0;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const int at = c ? begin + p.nl : begin;
+            if (nc[c] == 1) {                       // the partition fills in the cluster's own reference
+                single |= 1 << c;
+                continue;
+            }
+            int id = 0;
+            if (lane == 0) id = atomicAdd(node_count, 1);
+            id = __shfl_sync(0xffffffffu, id, 0);
+            ref[c] = id;
+            int slot = 0;
+            if (nc[c] <= kSahSmall) {
+                if (lane == 0) {
+                    slot = atomicAdd(&st->n_small, 1);
+                    if (slot < max_small) small[slot] = make_int4(at, nc[c], id, level + 1);
+                    else atomicExch(bad, 10);
+                }
+            } else {
+                if (lane == 0) slot = atomicAdd(&st->n_seg[par ^ 1], 1);
+                slot = __shfl_sync(0xffffffffu, slot, 0);
+                if (slot < max_segs) {
+                    sah_make_seg(next, next_bins, next_items, &st->n_item[par ^ 1], slot, max_items, at, nc[c], id, level + 1,
+                                 lane, bad);
+                    child[c] = slot;
+                } else if (lane == 0) {
+                    atomicExch(bad, 10);
+                }
+            }
+        }
+        if (lane == 0) {
+            g.axis = p.axis; g.bin = p.bin; g.nl = p.nl;
+            g.child_l = child[0]; g.child_r = child[1];
+            g.refs = single;
+            if (node >= 0 && node < n_nodes)
+                nodes[node] = make_node(make_float4(p.lo[0][0], p.lo[0][1], p.lo[0][2], 0.f),
+                                        make_float4(p.hi[0][0], p.hi[0][1], p.hi[0][2], 0.f), ref[0],
+                                        make_float4(p.lo[1][0], p.lo[1][1], p.lo[1][2], 0.f),
+                                        make_float4(p.hi[1][0], p.hi[1][1], p.hi[1][2], 0.f), ref[1]);
+            else
+                atomicExch(bad, 10);
+        }
+    }
+}
+
+// step 3: the chunks move their clusters to either side of the plane (places reserved with one
+// atomic per chunk and side) and gather the large children's centroid bounds
+__global__ void __launch_bounds__(kSahThreads) k_sah_part(const SahState *st, int par, SahSeg *segs, const int2 *items,
+                                                          const float4 *lo, const float4 *hi, float4 *lo2, float4 *hi2,
+                                                          SahSeg *next, BvhNode *nodes, int *bad) {
+    __shared__ int base[2], cb[12];
+    __shared__ int wl[kSahThreads / 32], wr[kSahThreads / 32];
+    const int n = st->n_item[par];
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kPer = kSahChunk / kSahThreads;
+    for (int it = blockIdx.x; it < n; it += gridDim.x) {
+        const int2 w = items[it];
+        SahSeg &g = segs[w.x];
+        const int begin = g.begin, count = g.count, nl = g.nl, axis = g.axis, bin = g.bin;
+        const int b0 = begin + w.y * kSahChunk, b1 = min(begin + count, b0 + kSahChunk);
+        const float cl = axis >= 0 ? float_of(g.clo[axis]) : 0.f;
+        const float ext = axis >= 0 ? __fsub_rn(float_of(g.chi[axis]), cl) : 0.f;
+        if (threadIdx.x < 12) cb[threadIdx.x] = threadIdx.x % 6 < 3 ? 0x7FFFFFFF : (int)0x80000000;
+        float4 a[kPer], b[kPer];
+        bool in[kPer], left[kPer];
+        int nleft = 0, nright = 0;
+        unsigned ml[kPer], mr[kPer];
+#pragma unroll
+        for (int r = 0; r < kPer; r++) {
+            const int i = b0 + r * kSahThreads + (int)threadIdx.x;
+            in[r] = i < b1;
+            left[r] = false;
+            if (in[r]) {
+                a[r] = lo[i];
+                b[r] = hi[i];
+                const float c = axis == 0 ? sah_centre(a[r].x, b[r].x) : (axis == 1 ? sah_centre(a[r].y, b[r].y) : sah_centre(a[r].z, b[r].z));
+                left[r] = axis >= 0 ? sah_bin(c, cl, ext) <= bin : i - begin < nl;
+            }
+            ml[r] = __ballot_sync(0xffffffffu, in[r] && left[r]);
+            mr[r] = __ballot_sync(0xffffffffu, in[r] && !left[r]);
+            nleft += __popc(ml[r]);
+            nright += __popc(mr[r]);
+        }
+        if (lane == 0) { wl[warp] = nleft; wr[warp] = nright; }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int tl = 0, tr = 0;
+#pragma unroll
+            for (int k = 0; k < kSahThreads / 32; k++) {
+                const int x = wl[k], y = wr[k];
+                wl[k] = tl; wr[k] = tr;
+                tl += x; tr += y;
+            }
+            base[0] = begin + atomicAdd(&g.cur_l, tl);
+            base[1] = begin + nl + atomicAdd(&g.cur_r, tr);
+        }
+        __syncthreads();
+        int pl = base[0] + wl[warp], pr = base[1] + wr[warp];
+        const unsigned lt = (1u << lane) - 1u;
+        int cmin[2][3], cmax[2][3];
+#pragma unroll
+        for (int s = 0; s < 2; s++)
+#pragma unroll
+            for (int k = 0; k < 3; k++) { cmin[s][k] = 0x7FFFFFFF; cmax[s][k] = (int)0x80000000; }
+#pragma unroll
+        for (int r = 0; r < kPer; r++) {
+            if (in[r]) {
+                const int o = left[r] ? pl + __popc(ml[r] & lt) : pr + __popc(mr[r] & lt);
+                if (o >= (left[r] ? begin : begin + nl) && o < (left[r] ? begin + nl : begin + count)) {
+                    lo2[o] = a[r];
+                    hi2[o] = b[r];
+                } else {
+                    atomicExch(bad, 11);
+                }
+                const int e[3] = {ord_of(sah_centre(a[r].x, b[r].x)), ord_of(sah_centre(a[r].y, b[r].y)),
+                                  ord_of(sah_centre(a[r].z, b[r].z))};
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    if (left[r]) { cmin[0][k] = min(cmin[0][k], e[k]); cmax[0][k] = max(cmax[0][k], e[k]); }
+                    else { cmin[1][k] = min(cmin[1][k], e[k]); cmax[1][k] = max(cmax[1][k], e[k]); }
+                }
+                if (g.refs & (left[r] ? 1 : 2)) {       // a child that is this one cluster
+                    int4 *ref = &nodes[g.node].r;
+                    if (left[r]) ref->x = __float_as_int(a[r].w);
+                    else ref->y = __float_as_int(a[r].w);
+                }
+            }
+            pl += __popc(ml[r]);
+            pr += __popc(mr[r]);
+        }
+        const int child[2] = {g.child_l, g.child_r};
+#pragma unroll
+        for (int s = 0; s < 2; s++)
+            if (child[s] >= 0) {
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const int x = warp_min(cmin[s][k]), y = warp_max(cmax[s][k]);
+                    if (lane == 0) { atomicMin(&cb[6 * s + k], x); atomicMax(&cb[6 * s + 3 + k], y); }
+                }
+            }
+        __syncthreads();
+        if (threadIdx.x < 12) {
+            const int s = threadIdx.x / 6, k = threadIdx.x % 6;
+            if (child[s] >= 0) {
+                if (k < 3) atomicMin(&next[child[s]].clo[k], cb[threadIdx.x]);
+                else atomicMax(&next[child[s]].chi[k - 3], cb[threadIdx.x]);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// the finished level's counters are cleared for the level after next
+__global__ void k_sah_next(SahState *st, int par) { st->n_seg[par] = st->n_item[par] = 0; }
+
+// Small segments, one warp each (taken from a counter): the clusters' boxes are loaded into
+// shared memory once, and the warp splits index ranges depth-first, the larger side pushed
+// (at most 8 pending), with the same bins and costs as the large segments.  A segment of n
+// clusters reserves its n - 1 nodes with one atomic.
+constexpr int kSmallWarps = 4;
+struct SahSmallWarp {
+    float4 lo[kSahSmall], hi[kSahSmall];
+    int bins[kSahSlotInts];
+    uint8_t idx[kSahSmall];
+    int4 stack[12];                      // (first, count, node, level)
+};
+
+__global__ void __launch_bounds__(kSmallWarps * 32) k_sah_small(SahState *st, int max_small, const int4 *small,
+                                                                const float4 *lo0, const float4 *hi0, const float4 *lo1,
+                                                                const float4 *hi1, BvhNode *nodes, int n_nodes,
+                                                                int *node_count, int *bad) {
+    extern __shared__ unsigned char sm_small[];
+    SahSmallWarp &S = reinterpret_cast<SahSmallWarp *>(sm_small)[threadIdx.x >> 5];
+    const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+    const int n = min(st->n_small, max_small);
+    while (true) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(&st->small_next, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= n) return;
+        const int4 seg = small[t];
+        const int begin = seg.x, count = seg.y;
+        // the level a segment was made at tells which copy of the clusters holds it
+        const float4 *lo = (seg.w & 1) ? lo1 : lo0, *hi = (seg.w & 1) ? hi1 : hi0;
+        for (int k = (int)lane; k < count; k += 32) {
+            S.lo[k] = lo[begin + k];
+            S.hi[k] = hi[begin + k];
+            S.idx[k] = (uint8_t)k;
+        }
+        int fresh = 0;                   // the next of the reserved nodes
+        if (lane == 0 && count > 2) fresh = atomicAdd(node_count, count - 2);
+        fresh = __shfl_sync(0xffffffffu, fresh, 0);
+        if (fresh + max(count - 2, 0) > n_nodes || seg.z < 0 || seg.z >= n_nodes) {
+            if (lane == 0) atomicExch(bad, 10);
+            return;
+        }
+        __syncwarp();
+        int first = 0, cnt = count, node = seg.z, level = seg.w, sp = 0;
+        while (true) {
+            int nl = 1;
+            float bl[2][3], bh[2][3];
+            if (cnt == 2) {
+#pragma unroll
+                for (int s = 0; s < 2; s++) {
+                    const float4 a = S.lo[S.idx[first + s]], b = S.hi[S.idx[first + s]];
+                    bl[s][0] = a.x; bl[s][1] = a.y; bl[s][2] = a.z;
+                    bh[s][0] = b.x; bh[s][1] = b.y; bh[s][2] = b.z;
+                }
+            } else {
+                // the centroids' bounds, then the bins
+                int l[3] = {0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF}, h[3] = {(int)0x80000000, (int)0x80000000, (int)0x80000000};
+                for (int k = (int)lane; k < cnt; k += 32) {
+                    const float4 a = S.lo[S.idx[first + k]], b = S.hi[S.idx[first + k]];
+                    const int e[3] = {ord_of(sah_centre(a.x, b.x)), ord_of(sah_centre(a.y, b.y)), ord_of(sah_centre(a.z, b.z))};
+#pragma unroll
+                    for (int q = 0; q < 3; q++) { l[q] = min(l[q], e[q]); h[q] = max(h[q], e[q]); }
+                }
+                float cl[3], ext[3];
+#pragma unroll
+                for (int q = 0; q < 3; q++) {
+                    cl[q] = float_of(warp_min(l[q]));
+                    ext[q] = __fsub_rn(float_of(warp_max(h[q])), cl[q]);
+                }
+                sah_bins_clear(S.bins, (int)lane, 32);
+                __syncwarp();
+                for (int k = (int)lane; k < cnt; k += 32) {
+                    const float4 a = S.lo[S.idx[first + k]], b = S.hi[S.idx[first + k]];
+                    const int bin[3] = {sah_bin(sah_centre(a.x, b.x), cl[0], ext[0]), sah_bin(sah_centre(a.y, b.y), cl[1], ext[1]),
+                                        sah_bin(sah_centre(a.z, b.z), cl[2], ext[2])};
+                    sah_bins_add(S.bins, bin, a, b);
+                }
+                __syncwarp();
+                SahPlane p = sah_select(S.bins, lane);
+                if (level >= kSahMaxLevel || p.nl <= 0 || p.nl >= cnt) p.axis = -1;
+                if (p.axis < 0) {
+                    p.nl = cnt / 2;
+#pragma unroll
+                    for (int q = 0; q < 3; q++) {
+                        const int *b = S.bins + (lane & 15u);
+                        p.lo[0][q] = p.lo[1][q] = float_of(warp_min(b[(1 + q) * kSahBins]));
+                        p.hi[0][q] = p.hi[1][q] = float_of(warp_max(b[(4 + q) * kSahBins]));
+                    }
+                } else {
+                    // stable partition of the index range (all of it read before any is written)
+                    uint8_t v[kSahSmall / 32];
+                    unsigned m[kSahSmall / 32];
+                    const float pcl = p.axis == 0 ? cl[0] : (p.axis == 1 ? cl[1] : cl[2]);
+                    const float pex = p.axis == 0 ? ext[0] : (p.axis == 1 ? ext[1] : ext[2]);
+#pragma unroll
+                    for (int r = 0; r < kSahSmall / 32; r++) {
+                        m[r] = 0u;
+                        v[r] = 0;
+                        if (r * 32 < cnt) {
+                            const int k = r * 32 + (int)lane;
+                            bool left = false;
+                            if (k < cnt) {
+                                v[r] = S.idx[first + k];
+                                const float4 a = S.lo[v[r]], b = S.hi[v[r]];
+                                const float c = p.axis == 0 ? sah_centre(a.x, b.x) : (p.axis == 1 ? sah_centre(a.y, b.y) : sah_centre(a.z, b.z));
+                                left = sah_bin(c, pcl, pex) <= p.bin;
+                            }
+                            m[r] = __ballot_sync(0xffffffffu, left);
+                        }
+                    }
+                    __syncwarp();
+                    int ol = first, orr = first + p.nl;
+#pragma unroll
+                    for (int r = 0; r < kSahSmall / 32; r++) {
+                        if (r * 32 < cnt) {
+                            const int k = r * 32 + (int)lane;
+                            const unsigned in = cnt - r * 32 >= 32 ? 0xffffffffu : (1u << (cnt - r * 32)) - 1u;
+                            if (k < cnt) {
+                                const int o = ((m[r] >> lane) & 1u) ? ol + __popc(m[r] & lt) : orr + __popc(~m[r] & in & lt);
+                                if (o < first + cnt) S.idx[o] = v[r];
+                                else atomicExch(bad, 11);
+                            }
+                            ol += __popc(m[r]);
+                            orr += __popc(~m[r] & in);
+                        }
+                    }
+                }
+                nl = p.nl;
+#pragma unroll
+                for (int s = 0; s < 2; s++)
+#pragma unroll
+                    for (int q = 0; q < 3; q++) { bl[s][q] = p.lo[s][q]; bh[s][q] = p.hi[s][q]; }
+                __syncwarp();
+            }
+            const int nr = cnt - nl;
+            int ref[2];
+            ref[0] = nl == 1 ? __float_as_int(S.lo[S.idx[first]].w) : fresh++;
+            ref[1] = nr == 1 ? __float_as_int(S.lo[S.idx[first + nl]].w) : fresh++;
+            if (lane == 0)
+                nodes[node] = make_node(make_float4(bl[0][0], bl[0][1], bl[0][2], 0.f), make_float4(bh[0][0], bh[0][1], bh[0][2], 0.f),
+                                        ref[0], make_float4(bl[1][0], bl[1][1], bl[1][2], 0.f),
+                                        make_float4(bh[1][0], bh[1][1], bh[1][2], 0.f), ref[1]);
+            level++;
+            if (nl > 1 && nr > 1) {
+                const bool big_left = nl >= nr;
+                if (lane == 0)
+                    S.stack[sp] = big_left ? make_int4(first, nl, ref[0], level) : make_int4(first + nl, nr, ref[1], level);
+                sp++;
+                if (big_left) { first += nl; cnt = nr; node = ref[1]; }
+                else { cnt = nl; node = ref[0]; }
+            } else if (nl > 1) {
+                cnt = nl; node = ref[0];
+            } else if (nr > 1) {
+                first += nl; cnt = nr; node = ref[1];
+            } else {
+                if (sp == 0) break;
+                __syncwarp();
+                const int4 e = S.stack[--sp];
+                first = e.x; cnt = e.y; node = e.z; level = e.w;
+            }
+            __syncwarp();
+        }
+        __syncwarp();
+    }
 }
 
 
@@ -491,10 +1150,17 @@ __device__ __forceinline__ void bin_child(const BvhNode &nd, int c, float3 &lo, 
     }
 }
 
-__global__ void k_collapse(const BvhNode *nodes, int n_bin, const int2 *fin, int n_in, Bvh4Node *out4, int max4,
-                           int *n4, int2 *fout, int *n_out, int *bad) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_in) return;
+// frontier counters: n4[0] 4-wide nodes made, n4[1 + level] the frontier of each level
+constexpr int kCollapseLevels = 200;
+__global__ void k_collapse_root(const int *root, int2 *f, int *n4) {
+    n4[0] = n4[1] = 1;
+    f[0] = make_int2(0, *root);
+}
+
+__global__ void __launch_bounds__(128) k_collapse(const BvhNode *nodes, int n_bin, const int2 *fin, const int *n_in, Bvh4Node *out4,
+                                                  int max4, int *n4, int2 *fout, int *n_out, int *bad) {
+  const int n = *n_in;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     int w4 = fin[t].x, b = fin[t].y;
     if (b < 0 || b >= n_bin || w4 < 0 || w4 >= max4) { atomicExch(bad, 5); return; }
     float3 lo[4], hi[4];
@@ -558,6 +1224,26 @@ __global__ void k_collapse(const BvhNode *nodes, int n_bin, const int2 *fin, int
     o.ref = make_int4(R[0], R[1], R[2], R[3]);
     o.pad = make_int4(0, 0, 0, 0);
     out4[w4] = o;
+  }
+}
+
+// what the host needs to know of the finished tree
+struct TreeSummary {
+    int bad, depth, root, clusters, n_seg[2];
+    float lo[3], hi[3];                  // the root's box
+};
+__global__ void k_summary(const int *ibuf, const SahState *st, const int *root, const BvhNode *nodes, int n_nodes, TreeSummary *o) {
+    o->bad = ibuf[6];
+    o->depth = ibuf[7];
+    o->root = *root;
+    o->clusters = st->count;
+    o->n_seg[0] = st->n_seg[0];
+    o->n_seg[1] = st->n_seg[1];
+    if (*root >= 0 && *root < n_nodes) {
+        const BvhNode nd = nodes[*root];
+        o->lo[0] = fminf(nd.a.x, nd.b.z); o->lo[1] = fminf(nd.a.y, nd.b.w); o->lo[2] = fminf(nd.a.z, nd.c.x);
+        o->hi[0] = fmaxf(nd.a.w, nd.c.y); o->hi[1] = fmaxf(nd.b.x, nd.c.z); o->hi[2] = fmaxf(nd.b.y, nd.c.w);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -738,147 +1424,168 @@ void sort_pairs_by_low_bits(unsigned long long *keys, uint32_t *vals, unsigned l
 
 static inline unsigned blocks_for(size_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
-// PLOC hierarchy over the m sorted tree triangles; writes nodes, parents, *root
-static int ploc_build(DofScene *s, int m, int radius, int *pnode, int *pleaf, int *ibuf, int *root, cudaStream_t st) {
-    const int B = 256;
-    int rc = DOF_OK;
-    int *cid[2] = {nullptr, nullptr}, *nn = nullptr, *keep = nullptr, *pos = nullptr, *cnt = nullptr;
-    float4 *clo[2] = {nullptr, nullptr}, *chi[2] = {nullptr, nullptr};
-    void *tmp = nullptr;
-    size_t tmp_bytes = 0;
-    auto ck = [&](cudaError_t e, const char *w) { if (rc == DOF_OK && e != cudaSuccess) rc = dof_cuda_check(e, w); };
-    for (int k = 0; k < 2; k++) {
-        ck(cudaMalloc(&cid[k], sizeof(int) * m), "ploc");
-        ck(cudaMalloc(&clo[k], sizeof(float4) * m), "ploc");
-        ck(cudaMalloc(&chi[k], sizeof(float4) * m), "ploc");
+namespace {
+// One block of scratch, handed out in 256-byte aligned pieces (sized first, then taken).
+struct Arena {
+    char *base = nullptr;
+    size_t used = 0;
+    template <class T> T *take(size_t n) {
+        T *p = base ? reinterpret_cast<T *>(base + used) : nullptr;
+        used += (n * sizeof(T) + 255) & ~(size_t)255;
+        return p;
     }
-    ck(cudaMalloc(&nn, sizeof(int) * m), "ploc");
-    ck(cudaMalloc(&keep, sizeof(int) * m), "ploc");
-    ck(cudaMalloc(&pos, sizeof(int) * m), "ploc");
-    ck(cudaMalloc(&cnt, sizeof(int)), "ploc");
-    tmp_bytes = sizeof(int) * (size_t)((m + kScanTile - 1) / kScanTile + 1);
-    ck(cudaMalloc(&tmp, tmp_bytes), "ploc scan temp");
-    if (rc == DOF_OK) {
-        ck(cudaMemsetAsync(cnt, 0, sizeof(int), st), "ploc");
-        k_ploc_init<<<blocks_for(m, B), B, 0, st>>>(s->tris, m, cid[0], clo[0], chi[0]);
-        int count = m, cur = 0;
-        for (int round = 0; count > 1 && rc == DOF_OK; round++) {
-            if (round > 100000) { rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "PLOC made no progress"); break; }
-            k_ploc_nn<<<blocks_for(count, B), B, 0, st>>>(count, radius, clo[cur], chi[cur], nn);
-            k_ploc_merge<<<blocks_for(count, B), B, 0, st>>>(count, cid[cur], clo[cur], chi[cur], nn, keep, cnt,
-                                                            s->nodes, pnode, pleaf, m - 1, ibuf + 6);
-            device_exclusive_scan(keep, pos, count, static_cast<int *>(tmp), st);
-            k_ploc_scatter<<<blocks_for(count, B), B, 0, st>>>(count, keep, pos, cid[cur], clo[cur], chi[cur],
-                                                              cid[cur ^ 1], clo[cur ^ 1], chi[cur ^ 1]);
-            int last[2];
-            ck(cudaMemcpyAsync(&last[0], pos + count - 1, sizeof(int), cudaMemcpyDeviceToHost, st), "ploc count");
-            ck(cudaMemcpyAsync(&last[1], keep + count - 1, sizeof(int), cudaMemcpyDeviceToHost, st), "ploc count");
-            ck(cudaStreamSynchronize(st), "ploc round");
-            int next = last[0] + last[1];
-            if (rc == DOF_OK && next >= count) { rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "PLOC round merged nothing"); break; }
-            count = next;
-            cur ^= 1;
-        }
-        if (rc == DOF_OK) {
-            ck(cudaMemcpyAsync(root, cid[cur], sizeof(int), cudaMemcpyDeviceToHost, st), "ploc root");
-            ck(cudaStreamSynchronize(st), "ploc root");
-            if (rc == DOF_OK && *root >= 0) {
-                int minus1 = -1;
-                ck(cudaMemcpy(pnode + *root, &minus1, sizeof(int), cudaMemcpyHostToDevice), "ploc root parent");
+};
+
+struct BuildScratch {
+    float4 *cen;
+    int *ibuf;                           // [0..5] centroid bounds, [6] bad, [7] depth, [8] large count, [9..14] small
+                                         // bounds, [15] nodes made
+    int *root;
+    unsigned long long *keys, *keys2;
+    uint32_t *vals, *vals2;
+    int *hist, *sums;                    // radix sort and scan
+    int *pnode, *pleaf, *arr;
+    TreeSummary *summary;
+    SahState *state;
+    // Karras
+    int4 *child;
+    float4 *blo, *bhi;
+    // PLOC and SAH
+    float4 *clo[2], *chi[2];
+    int *nn, *keep, *pos;
+    SahSeg *segs[2];
+    int *bins[2];
+    int2 *items[2];
+    int4 *small;
+    int max_segs, max_items, max_small;
+    // collapse
+    Bvh4Node *wide;
+    int2 *front[2];
+    int *n4;
+
+    void lay_out(Arena &A, int n, bool ploc) {
+        const size_t nn1 = (size_t)std::max(n - 1, 1);
+        const size_t nbk = (size_t)(n + kSortTile - 1) / kSortTile, nh = (size_t)kSortBins * nbk;
+        cen = A.take<float4>(n);
+        ibuf = A.take<int>(16);
+        root = A.take<int>(1);
+        keys = A.take<unsigned long long>(n);
+        keys2 = A.take<unsigned long long>(n);
+        vals = A.take<uint32_t>(n);
+        vals2 = A.take<uint32_t>(n);
+        hist = A.take<int>(nh);
+        sums = A.take<int>(std::max((nh + kScanTile - 1) / kScanTile, (size_t)(n + kScanTile - 1) / kScanTile) + 1);
+        pnode = A.take<int>(nn1);
+        pleaf = A.take<int>(n);
+        arr = A.take<int>(nn1);
+        summary = A.take<TreeSummary>(1);
+        state = A.take<SahState>(1);
+        max_segs = n / (kSahSmall + 1) + 2;
+        max_items = n / kSahChunk + max_segs + 2;
+        max_small = n / 2 + 2;
+        if (ploc) {
+            for (int k = 0; k < 2; k++) {
+                clo[k] = A.take<float4>(n);
+                chi[k] = A.take<float4>(n);
+                segs[k] = A.take<SahSeg>(max_segs);
+                bins[k] = A.take<int>((size_t)max_segs * kSahSlotInts);
+                items[k] = A.take<int2>(max_items);
             }
+            nn = A.take<int>(n);
+            keep = A.take<int>(n);
+            pos = A.take<int>(n);
+            small = A.take<int4>(max_small);
+        } else {
+            child = A.take<int4>(nn1);
+            blo = A.take<float4>(2 * (size_t)n);
+            bhi = A.take<float4>(2 * (size_t)n);
         }
+        wide = A.take<Bvh4Node>(nn1);
+        for (int k = 0; k < 2; k++) front[k] = A.take<int2>(nn1);
+        n4 = A.take<int>(kCollapseLevels + 2);
     }
-    for (int k = 0; k < 2; k++) { cudaFree(cid[k]); cudaFree(clo[k]); cudaFree(chi[k]); }
-    cudaFree(nn); cudaFree(keep); cudaFree(pos); cudaFree(cnt); cudaFree(tmp);
-    return rc;
+};
+
+// levels [from, from + count) of the large segments
+void sah_levels(const BuildScratch &b, DofScene *s, int m, int from, int count, int sms, cudaStream_t st) {
+    for (int l = from; l < from + count; l++) {
+        const int p = l & 1;
+        k_sah_bin<<<4 * sms, kSahThreads, 0, st>>>(b.state, p, b.segs[p], b.items[p], b.clo[p], b.chi[p], b.bins[p]);
+        k_sah_split<<<sms, 128, 0, st>>>(b.state, p, b.segs[p], b.bins[p], b.segs[p ^ 1], b.bins[p ^ 1], b.items[p ^ 1],
+                                         b.max_segs, b.max_items, b.small, b.max_small, s->nodes, m - 1, b.ibuf + 15,
+                                         b.ibuf + 6);
+        k_sah_part<<<4 * sms, kSahThreads, 0, st>>>(b.state, p, b.segs[p], b.items[p], b.clo[p], b.chi[p], b.clo[p ^ 1],
+                                                    b.chi[p ^ 1], b.segs[p ^ 1], s->nodes, b.ibuf + 6);
+        k_sah_next<<<1, 1, 0, st>>>(b.state, p);
+    }
 }
 
-// 4-wide tree from the binary one (root `root`, n_bin internal nodes); sets
-// s->nodes4 / root4 / n_nodes4 / depth4 (nodes4 stays null for a one-leaf tree)
-static int collapse4(DofScene *s, int root, int n_bin, int *ibuf, cudaStream_t st) {
+// The hierarchy over the m >= 2 sorted tree triangles: one PLOC round, then SAH.
+int ploc_sah_build(const BuildScratch &b, DofScene *s, int m, int radius, int sms, cudaStream_t st) {
     const int B = 256;
     int rc = DOF_OK;
-    s->root4 = root;
-    s->n_nodes4 = 0;
-    s->depth4 = 0;
-    if (root < 0 || n_bin < 1) return DOF_OK;
-    Bvh4Node *big = nullptr;
-    int2 *fr[2] = {nullptr, nullptr};
-    int *cnt = nullptr;
     auto ck = [&](cudaError_t e, const char *w) { if (rc == DOF_OK && e != cudaSuccess) rc = dof_cuda_check(e, w); };
-    ck(cudaMalloc(&big, sizeof(Bvh4Node) * n_bin), "collapse");
-    ck(cudaMalloc(&fr[0], sizeof(int2) * n_bin), "collapse");
-    ck(cudaMalloc(&fr[1], sizeof(int2) * n_bin), "collapse");
-    ck(cudaMalloc(&cnt, sizeof(int) * 2), "collapse");
-    if (rc == DOF_OK) {
-        int2 first = make_int2(0, root);
-        int init[2] = {1, 0};   // [0] 4-wide nodes allocated (the root), [1] next frontier size
-        ck(cudaMemcpy(fr[0], &first, sizeof(int2), cudaMemcpyHostToDevice), "collapse");
-        ck(cudaMemcpy(cnt, init, sizeof(init), cudaMemcpyHostToDevice), "collapse");
-        int n_in = 1, cur = 0, level = 0;
-        while (n_in > 0 && rc == DOF_OK) {
-            if (++level > 200) { rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "BVH collapse did not terminate"); break; }
-            ck(cudaMemsetAsync(cnt + 1, 0, sizeof(int), st), "collapse");
-            k_collapse<<<blocks_for(n_in, B), B, 0, st>>>(s->nodes, n_bin, fr[cur], n_in, big, n_bin, cnt, fr[cur ^ 1],
-                                                         cnt + 1, ibuf + 6);
-            int h[2];
-            ck(cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, st), "collapse");
-            ck(cudaStreamSynchronize(st), "collapse");
-            n_in = h[1];
-            s->n_nodes4 = h[0];
-            cur ^= 1;
+    // the clusters are compacted into copy 0 from copy 1
+    k_ploc_init<<<blocks_for(m, B), B, 0, st>>>(s->tris, m, b.clo[1], b.chi[1]);
+    radius = std::min(std::max(radius, 1), kNnMaxRadius);
+    k_ploc_nn<<<blocks_for(m, kNnThreads), kNnThreads, (kNnThreads + 2 * radius) * 2 * sizeof(float4), st>>>(
+        m, radius, b.clo[1], b.chi[1], b.nn);
+    k_ploc_merge<<<blocks_for(m, B), B, 0, st>>>(m, b.clo[1], b.chi[1], b.nn, b.keep, b.ibuf + 15, s->nodes, m - 1, b.ibuf + 6);
+    device_exclusive_scan(b.keep, b.pos, m, b.sums, st);
+    k_ploc_scatter<<<blocks_for(m, B), B, 0, st>>>(m, b.keep, b.pos, b.clo[1], b.chi[1], b.clo[0], b.chi[0]);
+    k_sah_root<<<1, 32, 0, st>>>(b.state, b.pos, b.keep, m, b.clo[0], b.segs[0], b.bins[0], b.items[0], b.max_items, b.small,
+                                 b.ibuf + 15, b.root, b.ibuf + 6);
+    if (m > kSahSmall) {
+        k_sah_root_bounds<<<2 * sms, kSahThreads, 0, st>>>(b.state, b.clo[0], b.chi[0], b.segs[0]);
+        // as many levels as balanced halving of the clusters (at most m) and a few uneven planes
+        // take, then more while segments are left
+        int levels = 4;
+        while ((m >> 1 >> (levels - 4)) > kSahSmall) levels++;
+        sah_levels(b, s, m, 0, levels, sms, st);
+        for (int from = levels;; from += 4) {
+            int left[2] = {0, 0};
+            ck(cudaMemcpyAsync(left, b.state->n_seg, sizeof(left), cudaMemcpyDeviceToHost, st), "bvh levels");
+            ck(cudaStreamSynchronize(st), "bvh levels");
+            if (rc != DOF_OK || left[from & 1] == 0) break;
+            if (from > 100) return dof_set_error(DOF_ERR_DEVICE_CHECK, "BVH splits did not end");
+            sah_levels(b, s, m, from, 4, sms, st);
         }
-        s->depth4 = level;
     }
-    if (rc == DOF_OK) {
-        s->nodes4_bytes = sizeof(Bvh4Node) * (size_t)s->n_nodes4;
-        rc = dof_alloc(s->ctx, s->nodes4_bytes, (void **)&s->nodes4, &s->bytes);
-        if (rc == DOF_OK)
-            ck(cudaMemcpy(s->nodes4, big, s->nodes4_bytes, cudaMemcpyDeviceToDevice), "collapse copy");
-        s->root4 = 0;
-    }
-    cudaFree(big); cudaFree(fr[0]); cudaFree(fr[1]); cudaFree(cnt);
+    const int shm = kSmallWarps * (int)sizeof(SahSmallWarp);
+    k_sah_small<<<(int)std::min<size_t>(blocks_for(b.max_small, kSmallWarps), 5 * (size_t)sms), kSmallWarps * 32, shm, st>>>(
+        b.state, b.max_small, b.small, b.clo[0], b.chi[0], b.clo[1], b.chi[1], s->nodes, m - 1, b.ibuf + 15, b.ibuf + 6);
+    ck(cudaGetLastError(), "bvh kernels");
     return rc;
 }
+}  // namespace
 
 int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const uint32_t *d_idx,
                      const uint32_t *d_mat, int builder, int ploc_radius, int rotations, cudaStream_t st) {
     const int n = (int)s->n_tris;
-    const int B = 256;
+    const int B = 256, sms = s->ctx->sm_count;
+    const bool ploc = builder == DOF_BVH_PLOC;
     int rc = DOF_OK;
-    float4 *cen = nullptr;
-    int *ibuf = nullptr;                    // bounds[6], bad, depth
-    unsigned long long *keys = nullptr, *keys2 = nullptr;
-    uint32_t *vals = nullptr, *vals2 = nullptr;
-    int4 *child = nullptr;
-    int *pnode = nullptr, *pleaf = nullptr, *arr = nullptr;
-    float4 *blo = nullptr, *bhi = nullptr;
-    void *tmp = nullptr;
-    size_t tmp_bytes = 0;
+    auto ck = [&](cudaError_t e, const char *w) { if (rc == DOF_OK && e != cudaSuccess) rc = dof_cuda_check(e, w); };
+    // all scratch in one stream-ordered block
+    Arena arena;
+    BuildScratch b{};
+    b.lay_out(arena, n, ploc);
+    if (s->ctx->pool) ck(cudaMallocFromPoolAsync((void **)&arena.base, arena.used, s->ctx->pool, st), "bvh scratch");
+    else ck(cudaMallocAsync((void **)&arena.base, arena.used, st), "bvh scratch");
+    if (rc != DOF_OK) return rc;
+    arena.used = 0;
+    b.lay_out(arena, n, ploc);
     int hbuf[16];
     int n_small = n, n_big = 0;
-    auto ck = [&](cudaError_t e, const char *w) { if (rc == DOF_OK && e != cudaSuccess) rc = dof_cuda_check(e, w); };
-    ck(cudaMalloc(&cen, sizeof(float4) * n), "bvh centroids");
-    ck(cudaMalloc(&ibuf, sizeof(int) * 16), "bvh scalars");
-    ck(cudaMalloc(&keys, sizeof(unsigned long long) * n), "bvh keys");
-    ck(cudaMalloc(&vals, sizeof(uint32_t) * n), "bvh vals");
-    ck(cudaMalloc(&keys2, sizeof(unsigned long long) * n), "bvh keys2");
-    ck(cudaMalloc(&vals2, sizeof(uint32_t) * n), "bvh vals2");
-    ck(cudaMalloc(&child, sizeof(int4) * (n > 1 ? n - 1 : 1)), "bvh children");
-    ck(cudaMalloc(&pnode, sizeof(int) * (n > 1 ? n - 1 : 1)), "bvh parents");
-    ck(cudaMalloc(&pleaf, sizeof(int) * n), "bvh leaf parents");
-    ck(cudaMalloc(&arr, sizeof(int) * (n > 1 ? n - 1 : 1)), "bvh flags");
-    ck(cudaMalloc(&blo, sizeof(float4) * (2 * n)), "bvh boxes");
-    ck(cudaMalloc(&bhi, sizeof(float4) * (2 * n)), "bvh boxes");
-    if (rc != DOF_OK) goto done;
     {
-        // ibuf: [0..5] centroid bounds, [6] bad, [7] depth, [8] large count, [9..14] small bounds
         const int lo_i = 0x7FFFFFFF, hi_i = (int)0x80000000;
-        int init[16] = {lo_i, lo_i, lo_i, hi_i, hi_i, hi_i, 0, 0, 0, lo_i, lo_i, lo_i, hi_i, hi_i, hi_i, 0};
-        ck(cudaMemcpyAsync(ibuf, init, sizeof(init), cudaMemcpyHostToDevice, st), "bvh init");
-        k_centroids<<<blocks_for(n, B), B, 0, st>>>(d_xyz, n_verts, d_idx, (uint32_t)n, cen, ibuf, ibuf + 6);
-        k_classify<<<blocks_for(n, B), B, 0, st>>>(cen, (uint32_t)n, ibuf, ibuf + 8, ibuf + 9);
-        ck(cudaMemcpyAsync(hbuf, ibuf, sizeof(hbuf), cudaMemcpyDeviceToHost, st), "bvh readback");
+        const int init[16] = {lo_i, lo_i, lo_i, hi_i, hi_i, hi_i, 0, 0, 0, lo_i, lo_i, lo_i, hi_i, hi_i, hi_i, 0};
+        ck(cudaMemcpyAsync(b.ibuf, init, sizeof(init), cudaMemcpyHostToDevice, st), "bvh init");
+        ck(cudaMemsetAsync(b.state, 0, sizeof(SahState), st), "bvh init");
+        const unsigned gb = std::min(blocks_for(n, B), (unsigned)(4 * sms));
+        k_centroids<<<gb, B, 0, st>>>(d_xyz, n_verts, d_idx, (uint32_t)n, b.cen, b.ibuf, b.ibuf + 6);
+        k_classify<<<gb, B, 0, st>>>(b.cen, (uint32_t)n, b.ibuf, b.ibuf + 8, b.ibuf + 9);
+        ck(cudaMemcpyAsync(hbuf, b.ibuf, sizeof(hbuf), cudaMemcpyDeviceToHost, st), "bvh readback");
         ck(cudaStreamSynchronize(st), "bvh classify");
         if (rc != DOF_OK) goto done;
         // large triangles stay out of the tree (tested directly by every ray) when there
@@ -886,83 +1593,100 @@ int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const ui
         int separate = hbuf[8] > 0 && hbuf[8] <= kMaxLargeTris && hbuf[8] < n;
         n_big = separate ? hbuf[8] : 0;
         n_small = n - n_big;
-        k_morton<<<blocks_for(n, B), B, 0, st>>>(cen, (uint32_t)n, separate ? ibuf + 9 : ibuf, ibuf, separate, keys,
-                                                 vals);
-        {
-            // scratch of the sort: the digit histograms and the scan's tile sums
-            const size_t nbk = (size_t)(n + kSortTile - 1) / kSortTile;
-            const size_t nh = (size_t)kSortBins * nbk, ns = (nh + kScanTile - 1) / kScanTile + 1;
-            tmp_bytes = sizeof(int) * (nh + ns);
-            ck(cudaMalloc(&tmp, tmp_bytes), "sort temp");
-            if (rc != DOF_OK) goto done;
-            int *hist = static_cast<int *>(tmp);
-            device_radix_sort_pairs(keys, vals, keys2, vals2, n, hist, hist + nh, st);
-            ck(cudaGetLastError(), "sort");
-        }
+        k_morton<<<blocks_for(n, B), B, 0, st>>>(b.cen, (uint32_t)n, separate ? b.ibuf + 9 : b.ibuf, b.ibuf, separate, b.keys,
+                                                 b.vals);
+        device_radix_sort_pairs(b.keys, b.vals, b.keys2, b.vals2, n, b.hist, b.sums, st);
         // sorted (key, triangle) pairs are in (keys, vals)
-        k_sorted_tris<<<blocks_for(n, B), B, 0, st>>>(d_xyz, d_idx, d_mat, (uint32_t)n, n_verts, vals, s->tris);
+        k_sorted_tris<<<blocks_for(n, B), B, 0, st>>>(d_xyz, d_idx, d_mat, (uint32_t)n, n_verts, b.vals, s->tris);
         const int m = n_small;
-        int root = m >= 2 ? 0 : ~0;
+        int levels4 = 0, n_front[kCollapseLevels + 2];
+        TreeSummary sum{};
         if (m >= 2) {
-            ck(cudaMemsetAsync(pleaf, 0xFF, sizeof(int) * m, st), "memset");
-            ck(cudaMemsetAsync(arr, 0, sizeof(int) * (m - 1), st), "memset");
             ck(cudaMemsetAsync(s->nodes, 0xFF, sizeof(BvhNode) * (m - 1), st), "memset");
-            if (builder == DOF_BVH_PLOC) {
-                if (rc == DOF_OK) rc = ploc_build(s, m, ploc_radius, pnode, pleaf, ibuf, &root, st);
+            if (ploc) {
+                if (rc == DOF_OK) rc = ploc_sah_build(b, s, m, ploc_radius, sms, st);
                 if (rc != DOF_OK) goto done;
             } else {
-                k_karras<<<blocks_for(m - 1, B), B, 0, st>>>(keys, m, child, pnode, pleaf, ibuf + 6);
-                k_refit<<<blocks_for(m, B), B, 0, st>>>(s->tris, m, child, pnode, pleaf, blo, bhi, arr, s->nodes,
-                                                        ibuf + 6);
+                ck(cudaMemsetAsync(b.arr, 0, sizeof(int) * (m - 1), st), "memset");
+                ck(cudaMemsetAsync(b.root, 0, sizeof(int), st), "memset");
+                k_karras<<<blocks_for(m - 1, B), B, 0, st>>>(b.keys, m, b.child, b.pnode, b.pleaf, b.ibuf + 6);
+                k_refit<<<blocks_for(m, B), B, 0, st>>>(s->tris, m, b.child, b.pnode, b.pleaf, b.blo, b.bhi, b.arr, s->nodes,
+                                                        b.ibuf + 6);
+            }
+            int *ref_leaf = reinterpret_cast<int *>(b.vals2);
+            if (rotations > 0) {
+                // the parents the passes walk up
+                ck(cudaMemsetAsync(b.pnode, 0xFF, sizeof(int) * (m - 1), st), "memset");
+                k_tree_refs<<<blocks_for(m - 1, B), B, 0, st>>>(s->nodes, m - 1, m, b.arr, ref_leaf, b.pnode, b.pleaf, b.ibuf + 6);
             }
             for (int pass = 0; pass < rotations; pass++) {
-                ck(cudaMemsetAsync(arr, 0, sizeof(int) * (m - 1), st), "memset");
-                k_rotate<<<blocks_for(m, B), B, 0, st>>>(m, s->nodes, pnode, pleaf, arr, ibuf + 6);
+                ck(cudaMemsetAsync(b.arr, 0, sizeof(int) * (m - 1), st), "memset");
+                k_rotate<<<blocks_for(m, B), B, 0, st>>>(m, s->nodes, b.pnode, b.pleaf, b.arr, b.ibuf + 6);
             }
             // the structure the packet tracer relies on (k_tree_refs), then the depth of
             // that structure; the sort's second buffers count the leaves' references
-            ck(cudaMemsetAsync(arr, 0, sizeof(int) * (m - 1), st), "memset");
-            ck(cudaMemsetAsync(vals2, 0, sizeof(int) * m, st), "memset");
-            ck(cudaMemsetAsync(pnode, 0xFF, sizeof(int) * (m - 1), st), "memset");
-            ck(cudaMemsetAsync(pleaf, 0xFF, sizeof(int) * m, st), "memset");
-            int *ref_leaf = reinterpret_cast<int *>(vals2);
-            k_tree_refs<<<blocks_for(m - 1, B), B, 0, st>>>(s->nodes, m - 1, m, arr, ref_leaf, pnode, pleaf, ibuf + 6);
-            k_tree_counts<<<blocks_for(m, B), B, 0, st>>>(m - 1, m, root, arr, ref_leaf, ibuf + 6);
-            k_depth<<<blocks_for(m, B), B, 0, st>>>(m, pnode, pleaf, ibuf + 7);
+            ck(cudaMemsetAsync(b.arr, 0, sizeof(int) * (m - 1), st), "memset");
+            ck(cudaMemsetAsync(b.vals2, 0, sizeof(int) * m, st), "memset");
+            ck(cudaMemsetAsync(b.pnode, 0xFF, sizeof(int) * (m - 1), st), "memset");
+            ck(cudaMemsetAsync(b.pleaf, 0xFF, sizeof(int) * m, st), "memset");
+            k_tree_refs<<<blocks_for(m - 1, B), B, 0, st>>>(s->nodes, m - 1, m, b.arr, ref_leaf, b.pnode, b.pleaf, b.ibuf + 6);
+            k_tree_counts<<<blocks_for(m, B), B, 0, st>>>(m - 1, m, b.root, b.arr, ref_leaf, b.ibuf + 6);
+            k_depth<<<blocks_for(m, B), B, 0, st>>>(m, b.pnode, b.pleaf, b.ibuf + 7);
+            // the 4-wide tree, level by level (a level past the deepest finds an empty frontier)
+            ck(cudaMemsetAsync(b.n4, 0, sizeof(int) * (kCollapseLevels + 2), st), "memset");
+            k_collapse_root<<<1, 1, 0, st>>>(b.root, b.front[0], b.n4);
+            for (bool more = true; more && rc == DOF_OK;) {
+                for (int k = 0; k < 20 && levels4 < kCollapseLevels; k++, levels4++)
+                    k_collapse<<<2 * sms, 128, 0, st>>>(s->nodes, m - 1, b.front[levels4 & 1], b.n4 + 1 + levels4, b.wide, m - 1,
+                                                       b.n4, b.front[(levels4 + 1) & 1], b.n4 + 2 + levels4, b.ibuf + 6);
+                k_summary<<<1, 1, 0, st>>>(b.ibuf, b.state, b.root, s->nodes, m - 1, b.summary);
+                ck(cudaMemcpyAsync(n_front, b.n4, sizeof(n_front), cudaMemcpyDeviceToHost, st), "bvh readback");
+                ck(cudaMemcpyAsync(&sum, b.summary, sizeof(sum), cudaMemcpyDeviceToHost, st), "bvh readback");
+                ck(cudaGetLastError(), "bvh kernels");
+                ck(cudaStreamSynchronize(st), "bvh build");
+                more = rc == DOF_OK && !sum.bad && n_front[1 + levels4] > 0 && levels4 < kCollapseLevels;
+            }
+        } else {
+            ck(cudaMemcpyAsync(&sum.bad, b.ibuf + 6, sizeof(int), cudaMemcpyDeviceToHost, st), "bvh readback");
+            ck(cudaGetLastError(), "bvh kernels");
+            ck(cudaStreamSynchronize(st), "bvh build");
         }
-        s->root = root;
-        ck(cudaGetLastError(), "bvh kernels");
-        ck(cudaMemcpyAsync(hbuf, ibuf, sizeof(hbuf), cudaMemcpyDeviceToHost, st), "bvh readback");
-        ck(cudaStreamSynchronize(st), "bvh build");
         if (rc != DOF_OK) goto done;
-        if (hbuf[6] == 1) { rc = dof_set_error(DOF_ERR_INVALID_ARG, "dof_scene_upload: vertex index out of range"); goto done; }
-        if (hbuf[6]) { rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "dof_scene_upload: BVH hierarchy check failed (%d)", hbuf[6]); goto done; }
-        s->depth = m >= 2 ? (uint32_t)hbuf[7] : 1;
+        if (sum.bad == 1) { rc = dof_set_error(DOF_ERR_INVALID_ARG, "dof_scene_upload: vertex index out of range"); goto done; }
+        if (sum.bad) { rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "dof_scene_upload: BVH hierarchy check failed (%d)", sum.bad); goto done; }
+        s->root = m >= 2 ? sum.root : ~0;
+        s->depth = m >= 2 ? (uint32_t)sum.depth : 1;
         s->n_tree = (uint32_t)m;
         s->n_large = (uint32_t)n_big;
         s->n_nodes = m >= 2 ? (uint32_t)(m - 1) : 0;
+        s->root4 = s->root;
+        s->n_nodes4 = 0;
+        s->depth4 = 0;
         if (s->depth > kTraversalStack) {
             rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "BVH depth %u exceeds the traversal stack", s->depth);
             goto done;
         }
-        if (m >= 2) {
-            rc = collapse4(s, root, m - 1, ibuf, st);
-            if (rc != DOF_OK) goto done;
-            ck(cudaMemcpyAsync(hbuf, ibuf, sizeof(hbuf), cudaMemcpyDeviceToHost, st), "bvh readback");
-            ck(cudaStreamSynchronize(st), "bvh collapse");
-            if (rc != DOF_OK) goto done;
-            if (hbuf[6]) { rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "dof_scene_upload: BVH collapse check failed (%d)", hbuf[6]); goto done; }
+        if (m >= 2 && ploc) {
+            // boxes whose areas overflow (or are no numbers) cannot be clustered by area
+            const float dx = sum.hi[0] - sum.lo[0], dy = sum.hi[1] - sum.lo[1], dz = sum.hi[2] - sum.lo[2];
+            if (!(dx * dy + dy * dz + dz * dx < INFINITY)) {
+                rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "dof_scene_upload: the triangles' bounds have no finite area");
+                goto done;
+            }
         }
-        // bounds of the tree's triangles: union of the root's child boxes
-        if (m >= 2 && root >= 0) {
-            BvhNode nd;
-            ck(cudaMemcpy(&nd, s->nodes + root, sizeof(BvhNode), cudaMemcpyDeviceToHost), "bounds");
-            s->lo[0] = fminf(nd.a.x, nd.b.z); s->lo[1] = fminf(nd.a.y, nd.b.w); s->lo[2] = fminf(nd.a.z, nd.c.x);
-            s->hi[0] = fmaxf(nd.a.w, nd.c.y); s->hi[1] = fmaxf(nd.b.x, nd.c.z); s->hi[2] = fmaxf(nd.b.y, nd.c.w);
+        if (m >= 2) {
+            if (n_front[1 + levels4] > 0) { rc = dof_set_error(DOF_ERR_DEVICE_CHECK, "BVH collapse did not terminate"); goto done; }
+            while (s->depth4 < levels4 && n_front[1 + s->depth4] > 0) s->depth4++;
+            s->n_nodes4 = n_front[0];
+            s->nodes4_bytes = sizeof(Bvh4Node) * (size_t)s->n_nodes4;
+            rc = dof_alloc(s->ctx, s->nodes4_bytes, (void **)&s->nodes4, &s->bytes);
+            ck(cudaMemcpyAsync(s->nodes4, b.wide, s->nodes4_bytes, cudaMemcpyDeviceToDevice, st), "collapse copy");
+            s->root4 = 0;
+            // bounds of the tree's triangles
+            for (int k = 0; k < 3; k++) { s->lo[k] = sum.lo[k]; s->hi[k] = sum.hi[k]; }
         }
     }
 done:
-    cudaFree(cen); cudaFree(ibuf); cudaFree(keys); cudaFree(vals); cudaFree(keys2); cudaFree(vals2);
-    cudaFree(child); cudaFree(pnode); cudaFree(pleaf); cudaFree(arr); cudaFree(blo); cudaFree(bhi); cudaFree(tmp);
+    cudaFreeAsync(arena.base, st);
     return rc;
 }
