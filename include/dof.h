@@ -218,11 +218,12 @@ const char *dof_last_error(void);
 
 /* Upload a triangle scene and build its BVH on the device from 63-bit Morton codes of
  * the triangle centroids: by default one round of PLOC clustering (Meister and Bittner
- * 2018), then top-down splits by a binned surface-area heuristic (Wald 2007); or the LBVH radix tree of Karras 2012 (DOF_OPT_BVH_BUILDER); two child
- * boxes per node.  The binary tree is then collapsed top-down into nodes of four child
- * boxes (the largest-area child is opened until four remain).  Up to 64
- * "large" triangles (box extent above 1/16 of the scene's centroid extent, e.g. a
- * ground plane) are kept out of the tree and tested directly by every ray.
+ * 2018), then top-down splits by a binned surface-area heuristic (Wald 2007); or the
+ * LBVH radix tree of Karras 2012 (DOF_OPT_BVH_BUILDER); two child boxes per node.  The
+ * binary tree is then collapsed top-down into nodes of four child boxes (the
+ * largest-area child is opened until four remain).  Up to 64 "large" triangles (box
+ * extent above 1/2 of the scene's centroid extent, 1/16 for the LBVH, e.g. a ground
+ * plane) are kept out of the tree and tested directly by every ray.
  *   xyz      host, n_verts * 3 floats
  *   tri_idx  host, n_tris * 3 vertex indices (< n_verts, checked)
  *   tri_mat  host, n_tris material ids (0 diffuse with hash albedo, 1 emitter), or NULL
