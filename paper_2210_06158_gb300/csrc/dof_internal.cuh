@@ -55,12 +55,13 @@ struct DevParams {
 // ---------------------------------------------------------------------------
 
 // BVH node: boxes of both children and their references.  A reference r >= 0 is an
-// internal node, r < 0 the leaf holding sorted triangle ~r.
+// internal node, r < 0 the leaf holding sorted triangle ~r.  Per axis the two planes of a
+// child lie side by side, so the slab test takes both with one packed multiply-add.
 struct __align__(16) BvhNode {
-    float4 a;   // child0 lo.xyz, child0 hi.x
-    float4 b;   // child0 hi.yz, child1 lo.xy
-    float4 c;   // child1 lo.z, child1 hi.xyz
-    int4 r;     // child0 ref, child1 ref, unused, unused
+    float4 a;   // x: child0 lo, child0 hi, child1 lo, child1 hi
+    float4 b;   // y
+    float4 c;   // z
+    int4 r;     // child0 ref, child1 ref, the axis along which child0 comes first, unused
 };
 
 // 4-wide node: the boxes of up to four children (structure of arrays) and their

@@ -44,20 +44,17 @@ __device__ __forceinline__ bool box_hit(const Ray &r, float3 lo, float3 hi, floa
     return tmin <= tmax * 1.0000005f;
 }
 
-// The slab test for a ray of known octant: per axis the near plane is lo where inv >= 0
-// and hi where inv < 0, so the near and far distances need no min/max.  With the
-// offsets of make_ray (off0 for lo, off1 for hi) these are exactly the min and max
-// that box_hit takes, so both tests give the same answer.
+// The slab test for a ray of known octant, on the (lo, hi) planes of one child per axis: the
+// near plane is lo where inv >= 0 and hi where inv < 0, so the near and far distances need
+// no min/max.  With the offsets of make_ray (off0 for lo, off1 for hi) these are exactly the
+// min and max that box_hit takes, so both tests give the same answer.
 template <bool NX, bool NY, bool NZ>
-__device__ __forceinline__ bool box_hit_o(const Ray &r, float3 lo, float3 hi, float tbest, float &tent) {
-    const float nx = NX ? fmaf(hi.x, r.inv.x, -r.off1.x) : fmaf(lo.x, r.inv.x, -r.off0.x);
-    const float fx = NX ? fmaf(lo.x, r.inv.x, -r.off0.x) : fmaf(hi.x, r.inv.x, -r.off1.x);
-    const float ny = NY ? fmaf(hi.y, r.inv.y, -r.off1.y) : fmaf(lo.y, r.inv.y, -r.off0.y);
-    const float fy = NY ? fmaf(lo.y, r.inv.y, -r.off0.y) : fmaf(hi.y, r.inv.y, -r.off1.y);
-    const float nz = NZ ? fmaf(hi.z, r.inv.z, -r.off1.z) : fmaf(lo.z, r.inv.z, -r.off0.z);
-    const float fz = NZ ? fmaf(lo.z, r.inv.z, -r.off0.z) : fmaf(hi.z, r.inv.z, -r.off1.z);
-    const float tmin = fmaxf(fmaxf(nx, ny), fmaxf(nz, 0.f));
-    const float tmax = fminf(fminf(fx, fy), fminf(fz, tbest));
+__device__ __forceinline__ bool box_hit_o(const Ray &r, float2 x, float2 y, float2 z, float tbest, float &tent) {
+    const float x0 = fmaf(x.x, r.inv.x, -r.off0.x), x1 = fmaf(x.y, r.inv.x, -r.off1.x);
+    const float y0 = fmaf(y.x, r.inv.y, -r.off0.y), y1 = fmaf(y.y, r.inv.y, -r.off1.y);
+    const float z0 = fmaf(z.x, r.inv.z, -r.off0.z), z1 = fmaf(z.y, r.inv.z, -r.off1.z);
+    const float tmin = fmaxf(fmaxf(NX ? x1 : x0, NY ? y1 : y0), fmaxf(NZ ? z1 : z0, 0.f));
+    const float tmax = fminf(fminf(NX ? x0 : x1, NY ? y0 : y1), fminf(NZ ? z0 : z1, tbest));
     tent = tmin;
     return tmin <= tmax * 1.0000005f;
 }
@@ -66,12 +63,12 @@ __device__ __forceinline__ bool box_hit_o(const Ray &r, float3 lo, float3 hi, fl
 // branch (uniform across a warp whose rays share the octant)
 __device__ __forceinline__ void box_pair(const Ray &r, const float4 &a, const float4 &b, const float4 &c,
                                          float tbest, bool &h0, float &t0, bool &h1, float &t1) {
-    const float3 lo0 = make_float3(a.x, a.y, a.z), hi0 = make_float3(a.w, b.x, b.y);
-    const float3 lo1 = make_float3(b.z, b.w, c.x), hi1 = make_float3(c.y, c.z, c.w);
-#define DOF_BOX_PAIR(X, Y, Z)                                   \
-    {                                                           \
-        h0 = box_hit_o<X, Y, Z>(r, lo0, hi0, tbest, t0);        \
-        h1 = box_hit_o<X, Y, Z>(r, lo1, hi1, tbest, t1);        \
+    const float2 x0 = make_float2(a.x, a.y), y0 = make_float2(b.x, b.y), z0 = make_float2(c.x, c.y);
+    const float2 x1 = make_float2(a.z, a.w), y1 = make_float2(b.z, b.w), z1 = make_float2(c.z, c.w);
+#define DOF_BOX_PAIR(X, Y, Z)                                  \
+    {                                                          \
+        h0 = box_hit_o<X, Y, Z>(r, x0, y0, z0, tbest, t0);     \
+        h1 = box_hit_o<X, Y, Z>(r, x1, y1, z1, tbest, t1);     \
     }
     switch (r.oct & 7) {
     case 0: DOF_BOX_PAIR(false, false, false) break;
@@ -84,6 +81,63 @@ __device__ __forceinline__ void box_pair(const Ray &r, const float4 &a, const fl
     default: DOF_BOX_PAIR(true, true, true) break;
     }
 #undef DOF_BOX_PAIR
+}
+
+// A packet ray's slab test: per axis one packed multiply-add takes a child's (lo, hi) planes.
+// The multipliers are inv for the near plane and inv (1 + 7e-7) for the far one, with each
+// plane's offset moved outward as make_ray does (from its own multiplier), so the far
+// distances carry the relative slack that box_hit multiplies in, and no distance is scaled at
+// a node.  The bound tbest comes scaled by the same slack.
+struct SlabRay {
+    float2 mx, my, mz, ox, oy, oz;
+};
+constexpr float kSlabSlack = 1.0000007f;
+
+__device__ __forceinline__ SlabRay make_slab_ray(const Ray &r) {
+    SlabRay s;
+    auto axis = [](float o, float inv, float2 &m, float2 &off) {
+        const float far = inv * kSlabSlack;
+        m = inv >= 0.f ? make_float2(inv, far) : make_float2(far, inv);
+        // near: -(o inv) lowered; far: -(o far) raised
+        const float on = o * inv, of = o * far;
+        const float near_off = -(on + fabsf(on) * 2.38418579e-7f), far_off = -(of - fabsf(of) * 2.38418579e-7f);
+        off = inv >= 0.f ? make_float2(near_off, far_off) : make_float2(far_off, near_off);
+    };
+    axis(r.o.x, r.inv.x, s.mx, s.ox);
+    axis(r.o.y, r.inv.y, s.my, s.oy);
+    axis(r.o.z, r.inv.z, s.mz, s.oz);
+    return s;
+}
+
+template <bool NX, bool NY, bool NZ>
+__device__ __forceinline__ bool slab_hit(const SlabRay &r, float2 x, float2 y, float2 z, float tbest) {
+    const float2 tx = __ffma2_rn(x, r.mx, r.ox), ty = __ffma2_rn(y, r.my, r.oy), tz = __ffma2_rn(z, r.mz, r.oz);
+    const float tmin = fmaxf(fmaxf(NX ? tx.y : tx.x, NY ? ty.y : ty.x), fmaxf(NZ ? tz.y : tz.x, 0.f));
+    const float tmax = fminf(fminf(NX ? tx.x : tx.y, NY ? ty.x : ty.y), fminf(NZ ? tz.x : tz.y, tbest));
+    return tmin <= tmax;
+}
+
+// whether the ray enters either child of a node (a, b, c: its planes per axis)
+__device__ __forceinline__ void slab_pair(const SlabRay &r, int oct, const float4 &a, const float4 &b, const float4 &c,
+                                          float tbest, bool &h0, bool &h1) {
+    const float2 x0 = make_float2(a.x, a.y), y0 = make_float2(b.x, b.y), z0 = make_float2(c.x, c.y);
+    const float2 x1 = make_float2(a.z, a.w), y1 = make_float2(b.z, b.w), z1 = make_float2(c.z, c.w);
+#define DOF_SLAB_PAIR(X, Y, Z)                               \
+    {                                                        \
+        h0 = slab_hit<X, Y, Z>(r, x0, y0, z0, tbest);        \
+        h1 = slab_hit<X, Y, Z>(r, x1, y1, z1, tbest);        \
+    }
+    switch (oct & 7) {
+    case 0: DOF_SLAB_PAIR(false, false, false) break;
+    case 1: DOF_SLAB_PAIR(true, false, false) break;
+    case 2: DOF_SLAB_PAIR(false, true, false) break;
+    case 3: DOF_SLAB_PAIR(true, true, false) break;
+    case 4: DOF_SLAB_PAIR(false, false, true) break;
+    case 5: DOF_SLAB_PAIR(true, false, true) break;
+    case 6: DOF_SLAB_PAIR(false, true, true) break;
+    default: DOF_SLAB_PAIR(true, true, true) break;
+    }
+#undef DOF_SLAB_PAIR
 }
 
 // the same slab test on one box of a 4-wide node (boxes stored per axis)
@@ -686,8 +740,8 @@ __global__ void __launch_bounds__(kTraceThreads, 7) k_trace_rays(const __grid_co
 
 // Packet tracer over the binary tree: the 32 rays a warp takes traverse it together,
 // one node sequence for the warp held in a warp-uniform stack.  A child is entered
-// when the ray of any lane enters its box, and the two children go in the order that
-// most of the lanes entering both prefer.  Each lane tests boxes and triangles with
+// when the ray of any lane enters its box, and the two children go in the order the node
+// keeps for the packet's octant (bvh.cu: order_children).  Each lane tests boxes and triangles with
 // its own ray and its own best hit (inclusive cull), so every ray ends with the closest
 // hit that the per-ray traversal finds.  A warp's rays come from a compact patch of
 // pixels (pixel order: with several rays per pixel, the cones of a few pixels through
@@ -695,6 +749,13 @@ __global__ void __launch_bounds__(kTraceThreads, 7) k_trace_rays(const __grid_co
 // frustum): the warp then steps with all its lanes and one broadcast load per node, at
 // the price of the nodes that only some of its rays need.  Lanes of a warp that
 // straddles two sessions of a batch trace one session's packet after the other.
+//
+// Bound (ncu, 4K scene at 1080p): 70% of the issue slots, the ALU pipe (min / max, compares,
+// votes) 53%, and the fixed latency of one dependent chain per warp: 62 registers hold 32
+// warps per SM.  The static order and the folded slack take the entry distances, a vote, two
+// counts and two multiplies out of a step: 1.589 -> 1.552 ms at 4K, 0.162 -> 0.158 ms at
+// 1080p.  Measured and not kept: 10 or 12 blocks per SM (spills, 7-11% slower), the 4-wide
+// tree (half the steps at twice the box tests: 8% slower at 4K).
 template <int kCap, bool kStats, class AS>
 __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_packets(const __grid_constant__ AS as_) {
     const BatchArgs &A = batch_args(as_);
@@ -756,6 +817,7 @@ __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_packets(const __grid
                 pending = true;
             }
         }
+        const SlabRay slab = make_slab_ray(ray);
         while (true) {
             const unsigned pm = __ballot_sync(0xffffffffu, pending);
             if (pm == 0) break;
@@ -768,8 +830,11 @@ __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_packets(const __grid
                 const float4 *__restrict__ tris = S.sc.tris;
                 int node = S.sc.root, sp = 0;
                 // the best distance the lane tests boxes and triangles against: its own
-                // for a lane of this session, -1 (nothing passes) for the others
-                float tb = act ? h.t : -1.f;
+                // for a lane of this session, -1 (nothing passes) for the others; ts is the
+                // same with the slab test's slack
+                float tb = act ? h.t : -1.f, ts = tb * kSlabSlack;
+                // the packet's octant, for the order of the children: its first lane's
+                const int first = __shfl_sync(0xffffffffu, ray.oct, __ffs(pm) - 1);
                 // no per-step guard: the tree passed the structure check at upload (every
                 // reference in range, every node but the root referenced once), so the
                 // packet enters each node at most once and ends within the tree's size;
@@ -780,24 +845,23 @@ __global__ void __launch_bounds__(kTraceThreads, 8) k_trace_packets(const __grid
                         const float4 *np = reinterpret_cast<const float4 *>(nodes + node);
                         const float4 a = __ldg(np), b = __ldg(np + 1), c = __ldg(np + 2);
                         const int4 ref = __ldg(reinterpret_cast<const int4 *>(np + 3));
-                        float t0, t1;
                         bool h0, h1;
-                        box_pair(ray, a, b, c, tb, h0, t0, h1, t1);
+                        slab_pair(slab, ray.oct, a, b, c, ts, h0, h1);
                         if (kStats) n_visit += act ? 1u : 0u;
-                        const unsigned m0 = __ballot_sync(0xffffffffu, h0), m1 = __ballot_sync(0xffffffffu, h1);
-                        if (m0 && m1) {
-                            const unsigned right_first = __ballot_sync(0xffffffffu, h0 && h1 && t1 < t0);
-                            const bool rf = 2 * __popc(right_first) > __popc(m0 & m1);
+                        const bool any0 = __any_sync(0xffffffffu, h0), any1 = __any_sync(0xffffffffu, h1);
+                        if (any0 && any1) {
+                            const bool rf = (first >> ref.z) & 1;     // child 1 first where the packet descends the axis
                             // at most one entry per level above the node: sp < depth <= kCap
                             stack[sp++] = rf ? ref.x : ref.y;
                             node = rf ? ref.y : ref.x;
                             continue;
                         }
-                        if (m0) { node = ref.x; continue; }
-                        if (m1) { node = ref.y; continue; }
+                        if (any0) { node = ref.x; continue; }
+                        if (any1) { node = ref.y; continue; }
                     } else {
                         if (kStats && act) n_tests++;
                         tri_update_bound(ray, tris, ~node, tb, h);
+                        ts = tb * kSlabSlack;
                     }
                     if (sp == 0) break;
                     node = stack[--sp];
