@@ -172,12 +172,12 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
 #define DOF_OPT_TRACE_STEPS         4   /* traversal steps between refill checks, 1..256 (default 64) */
 #define DOF_OPT_PLOC_RADIUS         5   /* nearest-neighbour search radius of the clustering round, 1..256
                                          * (default 48) */
-#define DOF_OPT_BVH_WIDTH           6   /* tree the rays traverse: 4 (default) = the binary tree collapsed
-                                         * to 4-wide nodes, 2 = the binary tree; same hits either way */
+#define DOF_OPT_BVH_WIDTH           6   /* tree that one ray per lane traverses: 4 (default) = the binary tree
+                                         * collapsed to 4-wide nodes, 2 = the binary tree; same hits either way */
 #define DOF_OPT_RAY_ORDER_GRID      7   /* order in which the tracer takes a block's rays: grouped by the
                                          * cell of their lens point on a g x g grid over the aperture,
-                                         * g = 1..16 (default 4), cells in Morton order; 1 = pixel by
-                                         * pixel.  Same hits either way */
+                                         * g = 1..16, cells in Morton order; 1 = pixel by pixel.  Until it is
+                                         * set the library chooses per session.  Same hits either way */
 /* block of the main filter's 81-tap gather in half-resolution pixels: value = width |
  * height << 16, width >= 8, width * height a multiple of 32 in 64..512 (default 32 x 8) */
 #define DOF_OPT_GATHER_BLOCK        8
@@ -193,10 +193,11 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
  * smallest compiled capacity (32, 64, 96) that holds both this and what the batch's trees
  * can need, so a small value never overflows.  Same hits either way */
 #define DOF_OPT_TRACE_STACK         11
-/* how the binary tree is traversed: 0 (default) = one ray per lane, persistent threads with
- * dynamic fetch; 1 = the 32 rays of a warp as one packet (one node sequence per warp, each lane
- * testing with its own ray and best hit); packets always traverse the binary tree, whatever
- * DOF_OPT_BVH_WIDTH says.  Same hits either way */
+/* the tracer: 0 = one ray per lane, persistent threads with dynamic fetch, on the tree of
+ * DOF_OPT_BVH_WIDTH; 1 = the 32 rays of a warp as one packet (one node sequence per warp, each
+ * lane testing with its own ray and best hit), always on the binary tree.  Until this option
+ * or DOF_OPT_BVH_WIDTH (which implies 0) is set the library chooses per step, by the
+ * aperture and the number of rays.  Same hits either way */
 #define DOF_OPT_TRACE_PACKETS       12
 /* passes of tree rotations after the BVH build of scenes uploaded afterwards, 0..16
  * (default 0): each swaps, bottom-up, a child with a grandchild where that shrinks the

@@ -221,8 +221,8 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
     c->trace_blocks_per_sm = 8;
     c->trace_refill_idle = 16;
     c->trace_steps = 64;
-    c->ray_order_grid = 4;
-    c->trace_packets = 0;
+    c->ray_order_grid = 0;
+    c->trace_packets = -1;
     c->trace_stats = 1;
     c->stack_depth = kTraversalStack;
     c->gather_w = 32;
@@ -232,6 +232,7 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
     c->main_form = 0;
     c->ploc_radius = 48;
     c->bvh_width = 4;
+    c->bvh_width_set = 0;
     c->bvh_rotations = 0;
     cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
     preload_trace_kernels();
@@ -301,6 +302,7 @@ extern "C" int dof_ctx_set_option(DofCtx *ctx, int option, int64_t value) {
         case DOF_OPT_BVH_WIDTH:
             if (value != 2 && value != 4) return dof_set_error(DOF_ERR_INVALID_ARG, "BVH width must be 2 or 4");
             ctx->bvh_width = (int)value;
+            ctx->bvh_width_set = 1;
             return DOF_OK;
         case DOF_OPT_TRACE_STEPS:
             if (value < 1 || value > 256) return dof_set_error(DOF_ERR_INVALID_ARG, "steps per round must be 1..256");
@@ -463,14 +465,14 @@ static SceneDev scene_dev(const DofScene *s) {
     d.n_tris = (int)s->n_tree;
     d.n_large = (int)s->n_large;
     d.root = s->root;
-    // the 4-wide tree, when its traversal stack bound (3 per level) fits; warp packets
-    // traverse the binary tree
-    bool wide = s->nodes4 && s->ctx->bvh_width == 4 && !s->ctx->trace_packets && 3 * s->depth4 + 3 <= kTraversalStack;
+    // the 4-wide tree, when its traversal stack bound (3 per level) fits
+    bool wide = s->nodes4 && s->ctx->bvh_width == 4 && 3 * s->depth4 + 3 <= kTraversalStack;
     d.nodes4 = wide ? s->nodes4 : nullptr;
     d.root4 = s->root4;
     d.n_nodes4 = s->n_nodes4;
     // a binary node pushes at most one child per level, a 4-wide node three
     d.stack_need = wide ? 3 * s->depth4 + 3 : (int)s->depth;
+    d.packet_need = (int)s->depth;
     return d;
 }
 
@@ -757,6 +759,36 @@ static void shape_grid(const BatchArgs &A, const SessDesc &d, const DofHistory *
     }
 }
 
+// The tracer of a step whose context leaves it open: warp packets, taken in pixel order, but
+// by lens cells of 1/8 aperture where the blur of the far field (cocK, its asymptotic
+// diameter) spans 11 px and more, so that a packet's rays leave one patch of the lens.  One ray
+// per lane stays where both the aperture is wide (cocK >= 6) and the rays are too few to fill
+// the chip's warps more than twice: the packets' unions are then large and the longest one
+// sets the time.  Measured (tracer + mask kernel, us; packets against one ray per lane at its
+// former default order):
+//   35 mm f/2 (cocK 1.6), 1080p: 1 ray 171 / 277, 2 rays 232 / 491, 4 rays 409 / 919;
+//     768p, up to 4 rays by Eq. 4: 191 / 328
+//   50 mm f/1.4, 256 x 144: 53 / 60; 720p, 4 rays (cocK 4.2): 101 / 189
+//   85 mm f/1.2, 1080p (cocK 16): 1 ray 234 / 239, 4 rays 593 / 736; 4K (cocK 32) 583 / 733;
+//     720p, up to 8 rays (cocK 10.7): 634 in pixel order, 601 by lens cells / 645;
+//     540p, 1 ray (cocK 8): 137 / 110, 4 rays 219 / 227
+static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
+    double rays = 0, wide_rays = 0;
+    for (int s = 0; s < A.ns; s++) {
+        const SessDesc &d = A.s[s];
+        const double r = (double)d.N * (d.p.ray_mode ? 0.5 * d.p.m : (double)d.p.spp);
+        rays += r;
+        if (d.cam.cocK >= 6.f) wide_rays += r;
+    }
+    if (ctx->trace_packets >= 0) A.packets = ctx->trace_packets;
+    else if (ctx->bvh_width_set) A.packets = 0;
+    else A.packets = !(wide_rays > 0.5 * rays && rays < 400e3);
+    for (int s = 0; s < A.ns; s++) {
+        const int g = A.packets ? (A.s[s].cam.cocK >= 11.f ? 8 : 1) : 4;
+        A.s[s].lens_grid = ctx->ray_order_grid ? ctx->ray_order_grid : g;
+    }
+}
+
 // The batch descriptor of one step of `reqs` (validated); *adaptive: a session uses Eq. 4.
 static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchArgs &A, bool &adaptive) {
     if (n > (uint32_t)kMaxBatch) return dof_set_error(DOF_ERR_INVALID_ARG, "dof_batch_frame: %u > %d sessions", n, kMaxBatch);
@@ -787,8 +819,7 @@ static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchAr
     A.cursor = &reqs[0].hist->counters[2];
     A.refill_idle = ctx->trace_refill_idle;
     A.steps_per_round = ctx->trace_steps;
-    A.lens_grid = ctx->ray_order_grid;
-    A.packets = ctx->trace_packets;
+    choose_tracer(ctx, A);
     A.stats = ctx->trace_stats;
     A.stack_depth = ctx->stack_depth;
     return DOF_OK;
@@ -876,7 +907,10 @@ struct DofGraph {
     DofHistory *hist[kMaxBatch];
     int start[SH_COUNT][kMaxBatch + 1];
     bool adaptive, wide;
-    int trace_blocks, refill_idle, steps_per_round, lens_grid, stack_depth, packets, stats;
+    int trace_blocks, refill_idle, steps_per_round, stack_depth, packets, stats;
+    int lens_grid;                // the context's lens-cell grid of that moment (0: chosen per session)
+    int packets_opt, width_set;   // ... and its choice of tracer
+    int packet_need;              // stack entries of the captured packet tracer
     int gather_w, gather_h, main_form, recon_w, recon_h;
     int main_tile;                // the main filter's shared-memory bytes (0: through L1)
     int store_mode;               // image_storage_mode of the captured step
@@ -927,7 +961,10 @@ extern "C" int dof_graph_create(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n
     g->taa = any_taa(A);
     g->refill_idle = A.refill_idle;
     g->steps_per_round = A.steps_per_round;
-    g->lens_grid = A.lens_grid;
+    g->lens_grid = ctx->ray_order_grid;
+    g->packets_opt = ctx->trace_packets;
+    g->width_set = ctx->bvh_width_set;
+    g->packet_need = packet_capacity(A);
     g->packets = A.packets;
     g->stats = A.stats;
     g->stack_depth = A.stack_depth;
@@ -985,6 +1022,12 @@ extern "C" int dof_graph_launch(DofGraph *g, const DofFrameReq *reqs, uint32_t n
     bool adaptive = false;
     int rc = build_batch(ctx, reqs, n, A, adaptive);
     if (rc) return rc;
+    // a tracer that the library chose is the captured one whatever the cameras are now
+    if (ctx->trace_packets == g->packets_opt && ctx->bvh_width_set == g->width_set) A.packets = g->packets;
+    for (int s = 0; s < A.ns; s++)
+        if (g->lens_grid) A.s[s].lens_grid = g->lens_grid;
+    if (A.packets && g->packets && packet_capacity(A) > g->packet_need)
+        return dof_set_error(DOF_ERR_MISMATCH, "dof_graph_launch: a scene's tree is deeper than the captured stack");
     if (memcmp(A.start, g->start, sizeof(A.start)) != 0 || adaptive != g->adaptive || all_wide(A) != g->wide ||
         ctx->sm_count * ctx->trace_blocks_per_sm != g->trace_blocks || main_filter_tile_bytes(A) != g->main_tile ||
         A.gather_w != g->gather_w || A.gather_h != g->gather_h || A.main_form != g->main_form ||
@@ -994,7 +1037,6 @@ extern "C" int dof_graph_launch(DofGraph *g, const DofFrameReq *reqs, uint32_t n
     // the kernels' scheduling knobs come from the staged copy; keep the captured ones
     A.refill_idle = g->refill_idle;
     A.steps_per_round = g->steps_per_round;
-    A.lens_grid = g->lens_grid;
     A.stack_depth = g->stack_depth;
     cudaStream_t st = (cudaStream_t)stream;
     cudaGetLastError();

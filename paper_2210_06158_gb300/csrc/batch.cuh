@@ -25,6 +25,7 @@ struct SessDesc {
     SceneDev sc;
     int gx[SH_COUNT];              // blocks per row of each shape
     int N, max_rays, valid, record_rays;
+    int lens_grid;                 // tracer work order: lens-cell grid of the mask kernel (1 = pixel order)
     // frame inputs and output (caller-owned)
     const float4 *color;
     const float *depth;
@@ -56,7 +57,6 @@ struct SessDesc {
 struct BatchArgs {
     int ns;
     int refill_idle, steps_per_round;   // tracer scheduling
-    int lens_grid;                 // tracer work order: lens-cell grid of the mask kernel (1 = pixel order)
     int packets;                   // 1: the binary tree traversed by warp packets (k_trace_packets)
     int stats;                     // 1: the packet tracer counts node visits and triangle tests
     int stack_depth;               // requested traversal stack entries (the launch takes an instance >= the need)
@@ -75,6 +75,13 @@ inline int image_storage_mode(const BatchArgs &A) {
     int n16 = 0;
     for (int i = 0; i < A.ns; i++) n16 += A.s[i].p.f16 != 0;
     return n16 == 0 ? 0 : (n16 == A.ns ? 1 : 2);
+}
+// The packet tracer's stack entries in this launch: the smallest compiled capacity that holds
+// the requested depth and every session's tree.
+inline int packet_capacity(const BatchArgs &A) {
+    int need = A.stack_depth;
+    for (int i = 0; i < A.ns; i++) need = need > A.s[i].sc.packet_need ? need : A.s[i].sc.packet_need;
+    return need <= 32 ? 32 : (need <= 64 ? 64 : kTraversalStack);
 }
 // whether any session of the launch takes the final TAA pass
 inline bool any_taa(const BatchArgs &A) {

@@ -82,7 +82,8 @@ struct SceneDev {
     const Bvh4Node *nodes4;      // the tree collapsed to 4-wide nodes (traversed when non-null)
     int root4;                   // its root reference
     int n_nodes4;
-    int stack_need;              // traversal stack entries the traversed tree can need
+    int stack_need;              // traversal stack entries one ray per lane can need on the traversed tree
+    int packet_need;             // ... and a packet on the binary tree
 };
 
 // at most this many large triangles are kept out of the tree (see bvh.cu)
@@ -100,12 +101,14 @@ struct DofCtx {
     int sm_count;
     int bvh_builder;               // DOF_BVH_PLOC or DOF_BVH_LBVH
     int bvh_rotations;             // passes of tree rotations after the build
-    int trace_blocks_per_sm, trace_refill_idle, trace_steps, ray_order_grid, trace_packets, trace_stats;
+    int trace_blocks_per_sm, trace_refill_idle, trace_steps, trace_stats;
+    int ray_order_grid, trace_packets;   // 0 / -1: not set, the library chooses (choose_tracer)
     int gather_w, gather_h, main_form;   // main filter launch shape and form
     int recon_w, recon_h;                // reconstruction launch shape
     int stack_depth;                     // requested traversal stack entries (raised to the tree's need)
     int ploc_radius;
     int bvh_width;                 // 4: traverse the collapsed 4-wide tree, 2: the binary tree
+    int bvh_width_set;             // the caller chose it (and with it one ray per lane, unless packets are set)
     uint32_t *d_status;            // device status word of context-level launches
     // A frame's ray path (mask .. reconstruction) runs on ray_stream (highest priority)
     // while its post-process filters run on the caller's stream; ev_fork / ev_join order

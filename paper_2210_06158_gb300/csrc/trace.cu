@@ -432,7 +432,7 @@ __global__ void k_edges(const __grid_constant__ AS as_) {
 // there and the shader reduces them in sample order.  The order in which the tracer
 // takes the rays is a separate list (ray_pix: work items q << 6 | s over the same
 // range): inside the block the rays are grouped by the cell of their lens point on a
-// g x g grid over the aperture's bounding square (g = BatchArgs::lens_grid; 1 keeps
+// g x g grid over the aperture's bounding square (g = SessDesc::lens_grid; 1 keeps
 // pixel order), cells taken in Morton order, so the 32 rays a tracer warp takes leave
 // nearby lens points for nearby pixels and stay close together through the blurred near
 // field.  The grouping changes no result: every ray is traced independently.
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(256) k_mask_compact(const __grid_constant__ AS
         b_ray = (uint32_t)(old >> 32);
     }
     __syncthreads();     // b_pix, b_ray and the warp offsets are read by every thread below
-    const int grid = A.lens_grid;
+    const int grid = S.lens_grid;
     if (grid <= 1) {
         // pixel order: the work items follow the pixels' own slots
         if (n > 0) {
@@ -986,14 +986,17 @@ void launch_trace_b(const BatchArgs &A, const AS &as, int blocks, cudaStream_t s
     // what every session's tree can need
     int need = A.stack_depth;
     for (int i = 0; i < A.ns; i++) need = max(need, A.s[i].sc.stack_need);
-    if (A.packets && !wide && A.stats) {
-        if (need <= 32) k_trace_packets<32, true, AS><<<blocks, kTraceThreads, 0, st>>>(as);
-        else if (need <= 64) k_trace_packets<64, true, AS><<<blocks, kTraceThreads, 0, st>>>(as);
-        else k_trace_packets<kStack, true, AS><<<blocks, kTraceThreads, 0, st>>>(as);
-    } else if (A.packets && !wide) {
-        if (need <= 32) k_trace_packets<32, false, AS><<<blocks, kTraceThreads, 0, st>>>(as);
-        else if (need <= 64) k_trace_packets<64, false, AS><<<blocks, kTraceThreads, 0, st>>>(as);
-        else k_trace_packets<kStack, false, AS><<<blocks, kTraceThreads, 0, st>>>(as);
+    if (A.packets) {
+        const int cap = packet_capacity(A);
+        if (A.stats) {
+            if (cap == 32) k_trace_packets<32, true, AS><<<blocks, kTraceThreads, 0, st>>>(as);
+            else if (cap == 64) k_trace_packets<64, true, AS><<<blocks, kTraceThreads, 0, st>>>(as);
+            else k_trace_packets<kStack, true, AS><<<blocks, kTraceThreads, 0, st>>>(as);
+        } else {
+            if (cap == 32) k_trace_packets<32, false, AS><<<blocks, kTraceThreads, 0, st>>>(as);
+            else if (cap == 64) k_trace_packets<64, false, AS><<<blocks, kTraceThreads, 0, st>>>(as);
+            else k_trace_packets<kStack, false, AS><<<blocks, kTraceThreads, 0, st>>>(as);
+        }
     } else if (wide) {
         if (need <= 32) k_trace_rays<true, 32, AS><<<blocks, kTraceThreads, 0, st>>>(as);
         else if (need <= 64) k_trace_rays<true, 64, AS><<<blocks, kTraceThreads, 0, st>>>(as);
