@@ -109,7 +109,6 @@ struct DofCtx {
     int ploc_radius;
     int bvh_width;                 // 4: traverse the collapsed 4-wide tree, 2: the binary tree
     int bvh_width_set;             // the caller chose it (and with it one ray per lane, unless packets are set)
-    uint32_t *d_status;            // device status word of context-level launches
     // A frame's ray path (mask .. reconstruction) runs on ray_stream (highest priority)
     // while its post-process filters run on the caller's stream; ev_fork / ev_join order
     // them around the shared inputs (tiles) and the composite.
@@ -208,8 +207,8 @@ void dof_free(DofCtx *ctx, void *ptr, size_t bytes);
 // launch wrappers (one per kernel group, defined in the .cu files)
 int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const uint32_t *d_idx,
                      const uint32_t *d_mat, int builder, int ploc_radius, int rotations, cudaStream_t st);
-void launch_primary(const DevCam &cam, const DevParams &p, SceneDev sc, float4 *color, float *depth,
-                    float4 *normal, int32_t *prim, uint32_t *status, cudaStream_t st);
+void launch_primary(const DevCam &cam, const DevParams &p, const SceneDev &sc, float4 *color, float *depth, float4 *normal,
+                    int32_t *prim, cudaStream_t st);
 // host-side tally of this library's kernel launches (dof_launch_count); each launch
 // wrapper adds the launches it enqueued
 void count_launches(long long n);
