@@ -11,27 +11,45 @@
 //
 // Work distribution: triangles whose candidate box holds at most kSmallPx pixels are
 // rasterised by the warp that set them up (the warp's 32 boxes are enumerated as one
-// list, so a warp's lanes stay busy whatever the box sizes); larger ones are queued and
-// cut into chunks of kChunkPx pixels that persistent blocks claim from a counter.
+// list, so a warp's lanes stay busy whatever the box sizes); larger ones are queued, and a
+// warp takes each (or, above kChunkTiles, a stretch of its tiles): its lanes test 32 tiles of
+// 8 x 8 pixels at once, then cover 32 surviving tiles at once, a bit per pixel; the pixels that
+// are left form a list for the check against the closest hits, and those that pass a second
+// one for the ray tests, so that each runs with all its lanes.
 //
-// Occlusion culling: the triangles are taken nearest first, in batches of growing size
-// (sorted by a lower bound of their distance from the lens centre).  After each batch a
-// two-level depth pyramid holds, per 16 x 16 and 128 x 128 pixel tile, the farthest
-// closest hit so far; a triangle whose bound is beyond it on every tile of its candidate
-// box is dropped whole, and a candidate pixel skips the ray test when the bound is beyond
-// the pixel's own closest hit.  Keys only decrease, so a stale read or an older pyramid
-// culls less, never wrongly; see near_bound for the margin.
+// Occlusion culling: the triangles are taken nearest first (sorted by a lower bound of their
+// distance from the lens centre, its top 16 bits) in batches of growing size.  Before each
+// batch, every pixel whose closest hit is nearer than the batch's least bound is marked done:
+// no triangle from here on can win it.  A triangle whose candidate box holds only finished
+// tiles is dropped whole, finished tiles and pixels of a queued triangle are dropped by their
+// bits, and a candidate pixel skips the ray test when the bound is beyond the pixel's own
+// closest hit.  Keys only decrease, so a stale read culls less, never wrongly; see near_bound
+// for the margin.
+//
+// Bound: the workloads' candidate boxes hold 592 times the image's pixels at 1080p (496k
+// triangles, tall blades in front of each other).  Enumerating them pixel by pixel took 6.4 of
+// 8.4 ms; now 1.6 ms, of which the queued triangles 1.2 ms (the longest warps of each batch, and
+// the tests of hits within a batch).  A farthest-hit pyramid over the tiles (4.7 ms) drops
+// little: grass leaves gaps, and one far pixel keeps a tile open; the bits keep only that
+// pixel.  Warps that take up to 1024 tiles set the time of a batch (4.3 ms); 64 tiles 1.9 ms, and
+// with the lists 1.6 ms; 32 tiles 1.65 ms.  4, 6 and 8 batches: 2.0, 1.6 and 1.7 ms.
 #include "geometry.cuh"
 
 #include <algorithm>
 
 namespace {
 
-constexpr int kSmallPx = 4096;       // candidate pixels above which a triangle is queued
-constexpr int kChunkPx = 2048;       // pixels of one chunk of a queued triangle
+constexpr int kSmallPx = 64;         // candidate pixels above which a triangle is queued
+// Tiles of a queued triangle that one warp takes at a time: one per 1024 triangles of the scene,
+// between these.  In a scene of few triangles a few of them cover the image and have to be
+// spread over the chip (256 x 144, 2.8k triangles: 159 us with 64 tiles, 59 us with 8); with
+// many, claiming and looking up the pieces costs more than it spreads (1080p, 60k: 689 us with
+// 64, 844 with 16, 1126 with 8; 640 x 360, 30k: 224, 190, 198).
+constexpr int kChunkTiles = 64, kChunkTilesFew = 8;
 constexpr int kRastThreads = 256;
-constexpr int kHizShift1 = 4, kHizShift2 = 7;   // depth-pyramid tiles: 16 and 128 pixels
-constexpr int kHizMaxTiles1 = 16;               // boxes over more fine tiles use the coarse level
+constexpr int kBigThreads = 128;
+constexpr int kTileShift = 3, kCoarseShift = 6;   // tiles of 8 x 8 and of 64 x 64 pixels
+constexpr int kMaxFineTiles = 16;                 // boxes over more tiles are looked up in the coarse ones
 
 // Edge functions of the image plane, scaled so that |a| + |b| = 1 (values in pixels)
 // and oriented so that a pixel centre (x, y) can see the triangle only where
@@ -44,10 +62,11 @@ struct TriSetup {
 // queued (large) triangle: setup and vertices
 struct BigTri {
     float4 e0, e1, e2;          // (a, b, c, -) per edge
-    int4 box;                   // i0, j0, box width, candidate pixels
+    int4 box;                   // i0, j0, i1, j1
     int k;                      // sorted triangle index
     float tn;                   // its distance bound (near_bound)
-    int pad[2];
+    int tiles;                  // 8 x 8 pixel tiles of the box
+    int pad;
 };
 
 __device__ __forceinline__ float3 xyz(float4 v) { return make_float3(v.x, v.y, v.z); }
@@ -195,7 +214,7 @@ __device__ __forceinline__ void divmod(int idx, int w, float rw, int &q, int &r)
 
 // the ray test of one candidate pixel, written to its closest-hit key
 __device__ __forceinline__ void test_pixel(const DevCam &cam, unsigned long long *keys, int i, int j, float4 v0,
-                                           float4 v1, float4 v2) {
+                                            float4 v1, float4 v2) {
     const float3 d = pixel_dir(cam, i + 0.5f, j + 0.5f);
     const Ray r = make_ray(cam.O, d);
     const float t = tri_hit(r, v0, v1, v2);
@@ -205,6 +224,21 @@ __device__ __forceinline__ void test_pixel(const DevCam &cam, unsigned long long
         atomicMin(&keys[(size_t)j * cam.W + i], key);
     }
 }
+
+// per batch: triangles queued whole; triangles cut into chunks (high word) and their chunks;
+// the next piece of work
+struct BigCounts {
+    unsigned long long cut;
+    uint32_t one, cursor;
+};
+
+// how triangles are cut: chunks of `tiles` tiles, more where a triangle would have over `most`
+// chunks (so that a batch's work items fit 32 bits)
+struct Cut {
+    int tiles;
+    uint32_t most;
+    __device__ __forceinline__ uint32_t per_chunk(int n) const { return max((uint32_t)tiles, ((uint32_t)n + most - 1u) / most); }
+};
 
 struct SmallSlot {               // one triangle of a warp's list (112 bytes)
     float e[9];
@@ -241,80 +275,68 @@ __device__ __forceinline__ float near_bound(const DevCam &cam, float4 v0, float4
     return d >= 0.f ? d : 0.f;
 }
 
-// the pixel's closest hit so far (from L2: the atomics update it there); +inf bits are
-// 0xFFFFFFFF, a NaN, so an untouched pixel never culls
+// distance bits of a pixel's key: +inf while it has no hit
+__device__ __forceinline__ uint32_t key_dist(unsigned long long key) { return min((uint32_t)(key >> 32), 0x7F800000u); }
+
+// whether the pixel's closest hit so far is nearer than tn (from L2: the atomics update it there)
 __device__ __forceinline__ bool occluded(const unsigned long long *keys, size_t q, float tn) {
-    const unsigned long long key = __ldcg(&keys[q]);
-    return tn > __uint_as_float((uint32_t)(key >> 32));
+    return tn > __uint_as_float(key_dist(__ldcg(&keys[q])));
 }
 
-// Depth pyramid: hiz1 per 16 x 16 tile (tw1 x th1), hiz2 per 128 x 128 tile (tw2 x th2),
-// each the largest closest-hit distance of its pixels (+inf while a pixel has none).
-struct Hiz {
-    const float *l1, *l2;
-    int tw1, th1, tw2, th2;
+// Which pixels are done (or outside the image): a bit each per 8 x 8 tile (row-major in the
+// tile, tw x th tiles), and per 64 x 64 tile (tw2 x th2) whether all of them are.
+struct Done {
+    unsigned long long *bits;
+    uint8_t *all;
+    int tw, th, tw2, th2;
 };
 
-// true when every tile of the pixel box [i0, i1] x [j0, j1] has all its pixels' closest
-// hits nearer than tn (fine tiles when the box spans few of them, else coarse ones)
-__device__ bool hiz_occluded(const Hiz &z, int i0, int j0, int i1, int j1, float tn) {
-    if (!(tn > 0.f)) return false;
-    int x0 = i0 >> kHizShift1, x1 = i1 >> kHizShift1, y0 = j0 >> kHizShift1, y1 = j1 >> kHizShift1;
-    const float *lv = z.l1;
-    int tw = z.tw1;
-    if ((x1 - x0 + 1) * (y1 - y0 + 1) > kHizMaxTiles1) {
-        x0 = i0 >> kHizShift2; x1 = i1 >> kHizShift2; y0 = j0 >> kHizShift2; y1 = j1 >> kHizShift2;
-        lv = z.l2;
-        tw = z.tw2;
+// one block per coarse tile, a warp per row of its fine tiles: a pixel is done when its
+// closest hit is nearer than every bound from sorted position `at` on (none when skeys is null)
+__global__ void __launch_bounds__(256) k_done(const unsigned long long *keys, int W, int H, Done done,
+                                              const unsigned long long *skeys, int at) {
+    const uint32_t least = skeys ? (uint32_t)(__ldg(&skeys[at]) << 15) : 0u;
+    const int lane = threadIdx.x & 31, ty = blockIdx.y * 8 + (threadIdx.x >> 5);
+    bool all = true;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const int tx = blockIdx.x * 8 + k;
+        const int i = tx * 8 + (lane & 7), j = ty * 8 + (lane >> 3);
+        const bool d0 = i >= W || j >= H || key_dist(__ldcg(&keys[(size_t)j * W + i])) < least;
+        const bool d1 = i >= W || j + 4 >= H || key_dist(__ldcg(&keys[(size_t)(j + 4) * W + i])) < least;
+        const unsigned m0 = __ballot_sync(0xffffffffu, d0), m1 = __ballot_sync(0xffffffffu, d1);
+        if (lane == 0 && tx < done.tw && ty < done.th) done.bits[ty * done.tw + tx] = m0 | ((unsigned long long)m1 << 32);
+        all = all && (m0 & m1) == 0xffffffffu;
     }
+    const int n = __syncthreads_and(all);
+    if (threadIdx.x == 0) done.all[blockIdx.y * done.tw2 + blockIdx.x] = (uint8_t)(n != 0);
+}
+
+// true when every pixel of the tiles over the box [i0, i1] x [j0, j1] is done (fine tiles when
+// the box spans few of them, else coarse ones)
+__device__ bool box_done(const Done &z, int i0, int j0, int i1, int j1) {
+    int x0 = i0 >> kTileShift, x1 = i1 >> kTileShift, y0 = j0 >> kTileShift, y1 = j1 >> kTileShift;
+    if ((x1 - x0 + 1) * (y1 - y0 + 1) <= kMaxFineTiles) {
+        for (int y = y0; y <= y1; y++)
+            for (int x = x0; x <= x1; x++)
+                if (~__ldg(&z.bits[y * z.tw + x])) return false;
+        return true;
+    }
+    x0 = i0 >> kCoarseShift; x1 = i1 >> kCoarseShift; y0 = j0 >> kCoarseShift; y1 = j1 >> kCoarseShift;
     for (int y = y0; y <= y1; y++)
         for (int x = x0; x <= x1; x++)
-            if (!(tn > __ldcg(&lv[y * tw + x]))) return false;
+            if (!__ldg(&z.all[y * z.tw2 + x])) return false;
     return true;
-}
-
-// one 16 x 16 block per fine tile: the largest closest hit of its pixels
-__global__ void __launch_bounds__(256) k_hiz1(const unsigned long long *keys, int W, int H, float *hiz1, int tw1) {
-    __shared__ float wmax[8];
-    const int i = blockIdx.x * 16 + (threadIdx.x & 15), j = blockIdx.y * 16 + (threadIdx.x >> 4);
-    float t = -INFINITY;
-    if (i < W && j < H) {
-        const float v = __uint_as_float((uint32_t)(__ldcg(&keys[(size_t)j * W + i]) >> 32));
-        t = v == v ? v : INFINITY;       // no hit yet: +inf
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float m = wmax[0];
-#pragma unroll
-        for (int k = 1; k < 8; k++) m = fmaxf(m, wmax[k]);
-        hiz1[blockIdx.y * tw1 + blockIdx.x] = m;
-    }
-}
-
-// coarse tiles: the largest of their 8 x 8 fine tiles
-__global__ void k_hiz2(const float *hiz1, int tw1, int th1, float *hiz2, int tw2, int th2) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= tw2 || y >= th2) return;
-    float m = -INFINITY;
-    for (int b = 0; b < 8; b++)
-        for (int a = 0; a < 8; a++) {
-            const int fx = 8 * x + a, fy = 8 * y + b;
-            if (fx < tw1 && fy < th1) m = fmaxf(m, hiz1[fy * tw1 + fx]);
-        }
-    hiz2[y * tw2 + x] = m;
 }
 
 // Setup of every triangle; the small ones are rasterised here, the others queued.
 // `split` warps serve each group of 32 triangles (each sets the group up and takes every
 // split-th stretch of 32 of its candidate pixels), so that scenes with few triangles
-// still occupy the GPU.
+// still occupy the GPU.  They must agree on the list: nothing writes the done bits meanwhile.
 __global__ void __launch_bounds__(kRastThreads) k_rast_small(DevCam cam, SceneDev sc, const uint32_t *order,
-                                                              int count, int split, const float *tnear, Hiz hiz,
-                                                              bool use_hiz, unsigned long long *keys, BigTri *big,
-                                                              uint32_t *n_big) {
+                                                              int count, int split, const float *tnear, Done done,
+                                                              unsigned long long *keys, BigTri *big, int max_big,
+                                                              Cut cut, uint32_t *chunk_start, BigCounts *counts) {
     __shared__ SmallSlot slot[kRastThreads];
     __shared__ int excl[kRastThreads];
     const int lane = threadIdx.x & 31, wbase = threadIdx.x & ~31;
@@ -328,21 +350,31 @@ __global__ void __launch_bounds__(kRastThreads) k_rast_small(DevCam cam, SceneDe
         const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
         TriSetup S;
         const float tn = __ldg(&tnear[k]);
-        if (tri_setup(cam, v0, v1, v2, S) && !(use_hiz && hiz_occluded(hiz, S.i0, S.j0, S.i1, S.j1, tn))) {
+        if (tri_setup(cam, v0, v1, v2, S) && !box_done(done, S.i0, S.j0, S.i1, S.j1)) {
             const int bw = S.i1 - S.i0 + 1, bh = S.j1 - S.j0 + 1;
             const long long n = (long long)bw * bh;
             if (n > kSmallPx) {
                 if (part == 0) {                     // the group's first warp queues it
-                    const uint32_t b = atomicAdd(n_big, 1u);
                     BigTri B;
                     B.e0 = make_float4(S.e[0], S.e[1], S.e[2], 0.f);
                     B.e1 = make_float4(S.e[3], S.e[4], S.e[5], 0.f);
                     B.e2 = make_float4(S.e[6], S.e[7], S.e[8], 0.f);
-                    B.box = make_int4(S.i0, S.j0, bw, (int)n);
+                    B.box = make_int4(S.i0, S.j0, S.i1, S.j1);
                     B.k = k;
                     B.tn = tn;
-                    B.pad[0] = B.pad[1] = 0;
-                    big[b] = B;
+                    B.tiles = ((S.i1 >> kTileShift) - (S.i0 >> kTileShift) + 1) * ((S.j1 >> kTileShift) - (S.j0 >> kTileShift) + 1);
+                    B.pad = 0;
+                    // one warp's work from the front of the queue; what is cut into chunks from
+                    // its end, its place and its first chunk from one atomic, so that the first
+                    // chunks ascend with the places
+                    if (B.tiles <= cut.tiles) {
+                        big[atomicAdd(&counts->one, 1u)] = B;
+                    } else {
+                        const uint32_t per = cut.per_chunk(B.tiles), n_chunks = ((uint32_t)B.tiles + per - 1u) / per;
+                        const unsigned long long at = atomicAdd(&counts->cut, (1ull << 32) | n_chunks);
+                        big[(uint32_t)max_big - 1u - (uint32_t)(at >> 32)] = B;
+                        chunk_start[at >> 32] = (uint32_t)at;
+                    }
                 }
             } else {
                 npx = (int)n;
@@ -380,98 +412,196 @@ __global__ void __launch_bounds__(kRastThreads) k_rast_small(DevCam cam, SceneDe
     }
 }
 
-// exclusive prefix of the queued triangles' chunk counts (one block)
-__global__ void __launch_bounds__(1024) k_big_chunks(const BigTri *big, const uint32_t *n_big,
-                                                     uint32_t *chunk_start, uint32_t *n_chunks) {
-    __shared__ uint32_t warp_sum[32];
-    __shared__ uint32_t carry;
-    const int n = (int)*n_big;
-    if (threadIdx.x == 0) carry = 0u;
-    __syncthreads();
-    for (int base = 0; base < n; base += 1024) {
-        const int b = base + threadIdx.x;
-        const uint32_t c = b < n ? (uint32_t)((big[b].box.w + kChunkPx - 1) / kChunkPx) : 0u;
-        uint32_t incl = c;
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane == 31) warp_sum[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t s = warp_sum[lane], si = s;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t v = __shfl_up_sync(0xffffffffu, si, o);
-                if (lane >= o) si += v;
-            }
-            warp_sum[lane] = si - s;
-        }
-        __syncthreads();
-        const uint32_t off = carry + warp_sum[warp] + incl - c;
-        if (b < n) chunk_start[b] = off;
-        __syncthreads();
-        if (threadIdx.x == 1023) carry = off + c;
-        __syncthreads();
+// A warp's working lists: tiles to cover (the triangle's place in the queue and the tile), the
+// pixels that 32 tiles leave (lane of the tile << 6 | pixel of the tile), and the pixels whose
+// closest hit so far the triangle may beat.
+struct RastWarp {
+    uint32_t tri[64];
+    int tile[64];
+    uint16_t px[32 * 64];
+    uint32_t test_tri[64];
+    int2 test_ij[64];
+};
+
+// the ray tests of the last n (<= 32) listed pixels, one per lane
+__device__ __forceinline__ void test_listed(const DevCam &cam, const SceneDev &sc, unsigned long long *keys,
+                                            const BigTri *__restrict__ big, const RastWarp &Q, int first, int n, int lane) {
+    if (lane < n) {
+        const int2 ij = Q.test_ij[first + lane];
+        const float4 *tp = sc.tris + 3 * (size_t)__ldg(&big[Q.test_tri[first + lane]].k);
+        test_pixel(cam, keys, ij.x, ij.y, __ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
     }
-    if (threadIdx.x == 0) {
-        chunk_start[n] = carry;
-        *n_chunks = carry;
+    __syncwarp();
+}
+
+// Up to 32 queued tiles, one per lane: the pixels that pass the three edges (edges_pass,
+// evaluated for all 64 pixels of the tile), lie in the triangle's box and are not done.  They
+// form one list, which the lanes check against the pixels' closest hits 32 at a time; what is
+// left is listed again (`tests` entries wait on entry and exit) and gets its ray tests 32 at a
+// time, so that the long test runs with all its lanes.
+__device__ __forceinline__ void cover_tiles(const DevCam &cam, const SceneDev &sc, unsigned long long *keys, const Done &done,
+                                            const BigTri *__restrict__ big, RastWarp &Q, int first, int n, int lane, int &tests) {
+    unsigned long long mask = 0ull;
+    uint32_t tri = 0;
+    int tx = 0, ty = 0;
+    float tn = 0.f;
+    if (lane < n) {
+        tri = Q.tri[first + lane];
+        const int tile = Q.tile[first + lane];
+        ty = tile / done.tw;
+        tx = tile - ty * done.tw;
+        const BigTri &B = big[tri];
+        const float4 e0 = __ldg(&B.e0), e1 = __ldg(&B.e1), e2 = __ldg(&B.e2);
+        const int4 box = __ldg(&B.box);
+        tn = __ldg(&B.tn);
+        const float x0 = (float)(tx * 8) + 0.5f, y0 = (float)(ty * 8) + 0.5f;
+        unsigned half[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            unsigned out = 0u;                       // bit = 1: an edge is negative
+#pragma unroll
+            for (int r = 3; r >= 0; r--) {
+                const float y = y0 + (float)(4 * h + r);
+                const float c0 = fmaf(e0.y, y, e0.z), c1 = fmaf(e1.y, y, e1.z), c2 = fmaf(e2.y, y, e2.z);
+#pragma unroll
+                for (int k = 7; k >= 0; k--) {
+                    const float x = x0 + (float)k;
+                    const float m = fminf(fminf(fmaf(e0.x, x, c0), fmaf(e1.x, x, c1)), fmaf(e2.x, x, c2));
+                    out = (out << 1) | (m >= 0.f ? 0u : 1u);
+                }
+            }
+            half[h] = ~out;
+        }
+        mask = half[0] | ((unsigned long long)half[1] << 32);
+        // the box's columns and rows in the tile
+        const int cl = max(box.x - tx * 8, 0), cr = min(box.z - tx * 8, 7), rl = max(box.y - ty * 8, 0), rr = min(box.w - ty * 8, 7);
+        const unsigned long long col = ((0xffu << cl) & (0xffu >> (7 - cr)) & 0xffu) * 0x0101010101010101ull;
+        const unsigned long long row = (~0ull << (8 * rl)) & (~0ull >> (8 * (7 - rr)));
+        mask &= col & row & ~__ldg(&done.bits[tile]);
+    }
+    // the pixels as one list
+    const int np = __popcll(mask);
+    int incl = np;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    int at = incl - np;
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+        for (unsigned m = h ? (unsigned)(mask >> 32) : (unsigned)mask; m; m &= m - 1)
+            Q.px[at++] = (uint16_t)((lane << 6) | (32 * h + __ffs(m) - 1));
+    __syncwarp();
+    const unsigned lt = (1u << lane) - 1u;
+    for (int w = 0; w < total; w += 32) {
+        const int e = w + lane < total ? Q.px[w + lane] : 0;
+        const int o = e >> 6, b = e & 63;
+        const uint32_t t = __shfl_sync(0xffffffffu, tri, o);
+        const float bound = __shfl_sync(0xffffffffu, tn, o);
+        const int i = __shfl_sync(0xffffffffu, tx, o) * 8 + (b & 7), j = __shfl_sync(0xffffffffu, ty, o) * 8 + (b >> 3);
+        const bool live = w + lane < total && !occluded(keys, (size_t)j * cam.W + i, bound);
+        const unsigned m = __ballot_sync(0xffffffffu, live);
+        if (live) {
+            const int p = tests + __popc(m & lt);
+            Q.test_tri[p] = t;
+            Q.test_ij[p] = make_int2(i, j);
+        }
+        tests += __popc(m);
+        __syncwarp();
+        if (tests >= 32) {
+            tests -= 32;
+            test_listed(cam, sc, keys, big, Q, tests, 32, lane);
+        }
     }
 }
 
-// queued triangles: persistent blocks claim chunks of kChunkPx candidate pixels
-__global__ void __launch_bounds__(kRastThreads) k_rast_big(DevCam cam, SceneDev sc, unsigned long long *keys,
-                                                            const BigTri *big, const uint32_t *n_big,
-                                                            const uint32_t *chunk_start, const uint32_t *n_chunks,
-                                                            uint32_t *cursor) {
-    __shared__ float e[9];
-    __shared__ float4 v[3];
-    __shared__ int box[4];
-    __shared__ float tn;
-    __shared__ uint32_t claim[2];
-    const uint32_t total = *n_chunks;
-    const int nb = (int)*n_big;
+// The queued triangles: warps claim them one at a time, then the chunks of the others.  The
+// lanes look at 32 tiles of the box at once and drop a tile when it is finished or when an
+// edge is negative at its best corner -- edge_at is monotone in x and in y, roundings
+// included, so every pixel of the tile fails the same test.  The others are covered 32 at a
+// time, across triangles.
+__global__ void __launch_bounds__(kBigThreads) k_rast_big(const __grid_constant__ DevCam cam, const __grid_constant__ SceneDev sc,
+                                                           unsigned long long *keys, const __grid_constant__ Done done,
+                                                           const BigTri *__restrict__ big, int max_big, Cut cutting,
+                                                           const uint32_t *__restrict__ chunk_start, BigCounts *counts) {
+    __shared__ RastWarp lists[kBigThreads / 32];
+    RastWarp &Q = lists[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t nb = __ldg(&counts->one);
+    const unsigned long long cut = __ldg(&counts->cut);
+    const uint32_t n_cut = (uint32_t)(cut >> 32);
+    const unsigned long long total = (unsigned long long)nb + (uint32_t)cut;
+    int queued = 0, tests = 0;
     for (;;) {
-        if (threadIdx.x == 0) {
-            const uint32_t c = atomicAdd(cursor, 1u);
-            int b = 0;
-            if (c < total) {
-                // last triangle whose chunks start at or before c
-                int lo = 0, hi = nb - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (chunk_start[mid] <= c) lo = mid; else hi = mid - 1;
-                }
-                b = lo;
-                const BigTri &B = big[b];
-                e[0] = B.e0.x; e[1] = B.e0.y; e[2] = B.e0.z;
-                e[3] = B.e1.x; e[4] = B.e1.y; e[5] = B.e1.z;
-                e[6] = B.e2.x; e[7] = B.e2.y; e[8] = B.e2.z;
-                box[0] = B.box.x; box[1] = B.box.y; box[2] = B.box.z; box[3] = B.box.w;
-                tn = B.tn;
-                const float4 *tp = sc.tris + 3 * (size_t)B.k;
-                v[0] = __ldg(tp); v[1] = __ldg(tp + 1); v[2] = __ldg(tp + 2);
-            }
-            claim[0] = c;
-            claim[1] = c < total ? c - chunk_start[b] : 0u;
-        }
-        __syncthreads();
-        const uint32_t c = claim[0];
+        uint32_t c = 0;
+        if (lane == 0) c = atomicAdd(&counts->cursor, 1u);
+        c = __shfl_sync(0xffffffffu, c, 0);
         if (c >= total) break;
-        const int bw = box[2], npx = box[3];
-        const int first = (int)claim[1] * kChunkPx;
-        const int last = min(npx, first + kChunkPx);
-        for (int w = first + threadIdx.x; w < last; w += kRastThreads) {
-            const int q = w / bw, r = w - q * bw;
-            const int i = box[0] + r, j = box[1] + q;
-            if (edges_pass(e, i + 0.5f, j + 0.5f) && !occluded(keys, (size_t)j * cam.W + i, tn))
-                test_pixel(cam, keys, i, j, v[0], v[1], v[2]);
+        uint32_t at = c;
+        int t0 = 0, t1;
+        if (c < nb) {
+            t1 = __ldg(&big[at].tiles);
+        } else {
+            c -= nb;
+            // the last triangle whose chunks start at or before c: 32 places looked at per step
+            uint32_t lo = 0, n = n_cut;
+            while (n > 1) {
+                const uint32_t step = (n + 31) / 32, p = lo + (uint32_t)lane * step;
+                const bool le = (uint32_t)lane * step < n && __ldg(&chunk_start[p]) <= c;
+                const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, le));   // lane 0 always is
+                n = min(step, n - k * step);
+                lo += k * step;
+            }
+            at = (uint32_t)max_big - 1u - lo;
+            const int tiles = __ldg(&big[at].tiles);
+            const uint32_t per = cutting.per_chunk(tiles);
+            t0 = (int)((c - __ldg(&chunk_start[lo])) * per);
+            t1 = min(tiles, t0 + (int)per);
         }
-        __syncthreads();
+        const BigTri &B = big[at];
+        const float4 e0 = __ldg(&B.e0), e1 = __ldg(&B.e1), e2 = __ldg(&B.e2);
+        const int4 box = __ldg(&B.box);
+        const float e[9] = {e0.x, e0.y, e0.z, e1.x, e1.y, e1.z, e2.x, e2.y, e2.z};
+        const int tx0 = box.x >> kTileShift, ty0 = box.y >> kTileShift;
+        const int tw = (box.z >> kTileShift) - tx0 + 1;
+        const float rtw = 1.f / (float)tw;
+        for (int base = t0; base < t1; base += 32) {
+            const int t = base + lane;
+            int tile = 0;
+            bool in = t < t1;
+            if (in) {
+                int q, r;
+                divmod(t, tw, rtw, q, r);
+                const int tx = tx0 + r, ty = ty0 + q;
+                tile = ty * done.tw + tx;
+                // the box's pixel centres in the tile
+                const float xl = (float)max(tx * 8, box.x) + 0.5f, xh = (float)min(tx * 8 + 7, box.z) + 0.5f;
+                const float yl = (float)max(ty * 8, box.y) + 0.5f, yh = (float)min(ty * 8 + 7, box.w) + 0.5f;
+#pragma unroll
+                for (int k = 0; k < 3; k++)
+                    in = in && edge_at(e + 3 * k, e[3 * k] > 0.f ? xh : xl, e[3 * k + 1] > 0.f ? yh : yl) >= 0.f;
+                in = in && ~__ldg(&done.bits[tile]) != 0ull;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const int o = queued + __popc(m & lt);
+                Q.tri[o] = at;
+                Q.tile[o] = tile;
+            }
+            queued += __popc(m);
+            __syncwarp();
+            if (queued >= 32) {
+                queued -= 32;
+                cover_tiles(cam, sc, keys, done, big, Q, queued, 32, lane, tests);
+                __syncwarp();
+            }
+        }
     }
+    if (queued > 0) cover_tiles(cam, sc, keys, done, big, Q, 0, queued, lane, tests);
+    if (tests > 0) test_listed(cam, sc, keys, big, Q, 0, tests, lane);
 }
 
 // closest hit per pixel -> colour, depth, normal, id (as the ray-cast producer writes them)
@@ -503,8 +633,9 @@ __global__ void __launch_bounds__(kRastThreads) k_rast_resolve(DevCam cam, DevPa
     normal[q] = make_float4(n.x, n.y, n.z, 0.f);
 }
 
-// per triangle: its distance bound, and the sort key (the bound's bits: non-negative
-// floats order as unsigned integers) with its index
+// per triangle: its distance bound, and the sort key (the top 16 of the bound's 31 bits:
+// non-negative floats order as unsigned integers, and 1/256 of the distance is order enough)
+// with its index
 __global__ void k_tri_near(DevCam cam, SceneDev sc, int n_tot, float *tnear, unsigned long long *skeys,
                            uint32_t *svals) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -512,7 +643,7 @@ __global__ void k_tri_near(DevCam cam, SceneDev sc, int n_tot, float *tnear, uns
     const float4 *tp = sc.tris + 3 * (size_t)k;
     const float tn = near_bound(cam, __ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
     tnear[k] = tn;
-    skeys[k] = (unsigned long long)__float_as_uint(tn);
+    skeys[k] = (unsigned long long)(__float_as_uint(tn) >> 15);
     svals[k] = (uint32_t)k;
 }
 
@@ -531,9 +662,9 @@ void launch_prim_index(const float4 *tris, int n, int32_t *prim_k, cudaStream_t 
     }
 }
 
-// triangles of the depth-ordered batches: the nearest 1/32, then 1/32, 1/16, 1/8, 1/4
-// and the farthest half; scenes under kSortedMin triangles run as one batch in scene
-// order (the sort and the launches would cost more than they save)
+// ends of the depth-ordered batches: the nearest 1/32, as many again, then twice as many each; scenes under
+// kSortedMin triangles run as one batch in scene order (the sort and the launches would cost
+// more than they save)
 constexpr int kBatches = 6;
 constexpr int kSortedMin = 65536;
 __host__ inline int batch_end(int b, int nb, int n) { return b + 1 >= nb ? n : (int)((long long)n >> (nb - 1 - b)); }
@@ -542,11 +673,11 @@ __host__ inline int batch_end(int b, int nb, int n) { return b + 1 >= nb ? n : (
 size_t raster_scratch_bytes(int W, int H, int n_tot) {
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t n = (size_t)n_tot;
-    const size_t t1 = (size_t)((W + 15) >> kHizShift1) * ((H + 15) >> kHizShift1);
-    const size_t t2 = (size_t)((W + 127) >> kHizShift2) * ((H + 127) >> kHizShift2);
-    return up(8 * (size_t)W * H) + up(sizeof(BigTri) * n) + up(4 * (n + 1)) + up(16 * kBatches) +
-           up(4 * n) + 2 * up(8 * n) + 2 * up(4 * n) + up(4 * sort_pairs_scratch_ints(n_tot)) + up(4 * t1) +
-           up(4 * t2);
+    const size_t t1 = (size_t)((W + 7) >> kTileShift) * ((H + 7) >> kTileShift);
+    const size_t t2 = (size_t)((W + 63) >> kCoarseShift) * ((H + 63) >> kCoarseShift);
+    return up(8 * (size_t)W * H) + up(sizeof(BigTri) * n) + up(4 * (n + 1)) + up(sizeof(BigCounts) * kBatches) +
+           up(4 * n) + 2 * up(8 * n) + 2 * up(4 * n) + up(4 * sort_pairs_scratch_ints(n_tot)) + up(8 * t1) +
+           up(t2);
 }
 
 cudaError_t launch_raster(const DevCam &cam, const DevParams &p, const SceneDev &sc, const int32_t *prim_k,
@@ -561,8 +692,11 @@ cudaError_t launch_raster(const DevCam &cam, const DevParams &p, const SceneDev 
     base += up(sizeof(BigTri) * (size_t)n_tot);
     uint32_t *chunk_start = reinterpret_cast<uint32_t *>(base);
     base += up(4 * ((size_t)n_tot + 1));
-    uint32_t *counters = reinterpret_cast<uint32_t *>(base);   // per batch: n_big, n_chunks, cursor
-    base += up(16 * kBatches);
+    BigCounts *counts = reinterpret_cast<BigCounts *>(base);
+    base += up(sizeof(BigCounts) * kBatches);
+    Cut cut;
+    cut.tiles = std::min(kChunkTiles, std::max(kChunkTilesFew, n_tot / 1024));
+    cut.most = std::min(65536u, std::max(1u, 0x7FFFFFFFu / (uint32_t)std::max(n_tot, 1)));
     const size_t n = (size_t)n_tot;
     float *tnear = reinterpret_cast<float *>(base);
     base += up(4 * n);
@@ -576,43 +710,34 @@ cudaError_t launch_raster(const DevCam &cam, const DevParams &p, const SceneDev 
     base += up(4 * n);
     int *sort_scratch = reinterpret_cast<int *>(base);
     base += up(4 * sort_pairs_scratch_ints(n_tot));
-    Hiz hiz;
-    hiz.tw1 = (cam.W + 15) >> kHizShift1; hiz.th1 = (cam.H + 15) >> kHizShift1;
-    hiz.tw2 = (cam.W + 127) >> kHizShift2; hiz.th2 = (cam.H + 127) >> kHizShift2;
-    float *hiz1 = reinterpret_cast<float *>(base);
-    base += up(4 * (size_t)hiz.tw1 * hiz.th1);
-    float *hiz2 = reinterpret_cast<float *>(base);
-    hiz.l1 = hiz1;
-    hiz.l2 = hiz2;
+    Done done;
+    done.tw = (cam.W + 7) >> kTileShift; done.th = (cam.H + 7) >> kTileShift;
+    done.tw2 = (cam.W + 63) >> kCoarseShift; done.th2 = (cam.H + 63) >> kCoarseShift;
+    done.bits = reinterpret_cast<unsigned long long *>(base);
+    base += up(8 * (size_t)done.tw * done.th);
+    done.all = reinterpret_cast<uint8_t *>(base);
     cudaError_t e = cudaMemsetAsync(keys, 0xFF, 8 * (size_t)cam.W * cam.H, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counters, 0, 16 * kBatches, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(BigCounts) * kBatches, st);
     if (e != cudaSuccess) return e;
     if (n_tot > 0) {
         // the triangles nearest first
         const int nbat = n_tot >= kSortedMin ? kBatches : 1;
         k_tri_near<<<(n_tot + 255) / 256, 256, 0, st>>>(cam, sc, n_tot, tnear, skeys, order);
-        if (nbat > 1) sort_pairs_by_low_bits(skeys, order, skeys2, order2, n_tot, 32, sort_scratch, st);
+        if (nbat > 1) sort_pairs_by_low_bits(skeys, order, skeys2, order2, n_tot, 16, sort_scratch, st);
         for (int bt = 0, b0 = 0; bt < nbat; bt++) {
             const int b1 = batch_end(bt, nbat, n_tot);
             if (b1 <= b0) continue;
-            uint32_t *cb = counters + 4 * bt;
+            BigCounts *cb = counts + bt;
+            k_done<<<dim3(done.tw2, done.th2), 256, 0, st>>>(keys, cam.W, cam.H, done, nbat > 1 ? skeys : nullptr, b0);
             // at least 32 warps per SM: groups of 32 triangles are split over several warps
             const int groups = (b1 - b0 + 31) / 32;
             const int split = std::min(16, std::max(1, (32 * sm_count + groups - 1) / groups));
             const int warps = groups * split;
             k_rast_small<<<(warps + kRastThreads / 32 - 1) / (kRastThreads / 32), kRastThreads, 0, st>>>(
-                cam, sc, order + b0, b1 - b0, split, tnear, hiz, b0 > 0, keys, big, cb);
-            k_big_chunks<<<1, 1024, 0, st>>>(big, cb, chunk_start, cb + 1);
-            k_rast_big<<<4 * sm_count, kRastThreads, 0, st>>>(cam, sc, keys, big, cb, chunk_start, cb + 1, cb + 2);
+                cam, sc, order + b0, b1 - b0, split, tnear, done, keys, big, n_tot, cut, chunk_start, cb);
+            k_rast_big<<<8 * sm_count, kBigThreads, 0, st>>>(cam, sc, keys, done, big, n_tot, cut, chunk_start, cb);
             count_launches(3);
             b0 = b1;
-            if (b0 < n_tot) {
-                // the depth pyramid for the next batch
-                k_hiz1<<<dim3(hiz.tw1, hiz.th1), 256, 0, st>>>(keys, cam.W, cam.H, hiz1, hiz.tw1);
-                k_hiz2<<<dim3((hiz.tw2 + 15) / 16, (hiz.th2 + 15) / 16), dim3(16, 16), 0, st>>>(
-                    hiz1, hiz.tw1, hiz.th1, hiz2, hiz.tw2, hiz.th2);
-                count_launches(2);
-            }
         }
         count_launches(1);
     }
