@@ -229,7 +229,8 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
     c->gather_h = 8;
     c->recon_w = 32;
     c->recon_h = 8;
-    c->main_form = 0;
+    c->main_form = -1;
+    c->gather_set = 0;
     c->ploc_radius = 48;
     c->bvh_width = 4;
     c->bvh_width_set = 0;
@@ -324,6 +325,7 @@ extern "C" int dof_ctx_set_option(DofCtx *ctx, int option, int64_t value) {
             if (option == DOF_OPT_GATHER_BLOCK) {
                 ctx->gather_w = (int)w;
                 ctx->gather_h = (int)h;
+                ctx->gather_set = 1;
             } else {
                 ctx->recon_w = (int)w;
                 ctx->recon_h = (int)h;
@@ -750,6 +752,28 @@ static void shape_grid(const BatchArgs &A, const SessDesc &d, const DofHistory *
     }
 }
 
+// The main filter's form and block.  Left open, or left to reads through L1 (form 1): columns of
+// four pixels from kColumnsMinPx half-resolution pixels on, where they fill the chip's warps
+// twice, in blocks of 32 x 2 threads unless the caller set them.  Below, the halo tile where it
+// fits (form 1: one pixel per thread).  Measured (us, FP32; halo tile 32 x 8 / one pixel per
+// thread 32 x 4 / columns 32 x 2): 360p 26.3 / 26.6 / 34.4, 540p 44.6 / 45.2 / 44.2, 720p 60.7 /
+// 71.6 / 58.1, 1080p 127 / 133 / 115, with the 85 mm lens (radius to 32) 540p 56 / 55 / 55 and
+// 1080p 146 / 146 / 123; 4K, the tile past 64 KB: - / 511 / 407 (32 x 4).
+constexpr long long kColumnsMinPx = 180000;
+static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchArgs &A) {
+    long long px = 0;
+    for (uint32_t s = 0; s < n; s++) px += reqs[s].hist ? reqs[s].hist->N : 0;
+    A.main_form = ctx->main_form;
+    A.gather_w = ctx->gather_w;
+    A.gather_h = ctx->gather_h;
+    if ((ctx->main_form == -1 || ctx->main_form == 1) && px >= kColumnsMinPx) {
+        A.main_form = 3;
+        if (!ctx->gather_set) A.gather_h = 2;
+    } else if (ctx->main_form == -1) {
+        A.main_form = 0;
+    }
+}
+
 // The tracer of a step whose context leaves it open: warp packets, taken in pixel order, but
 // by lens cells of 1/8 aperture where the blur of the far field (cocK, its asymptotic
 // diameter) spans 11 px and more, so that a packet's rays leave one patch of the lens.  One ray
@@ -785,11 +809,9 @@ static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchAr
     if (n > (uint32_t)kMaxBatch) return dof_set_error(DOF_ERR_INVALID_ARG, "dof_batch_frame: %u > %d sessions", n, kMaxBatch);
     memset(&A, 0, sizeof(A));
     A.ns = (int)n;
-    A.gather_w = ctx->gather_w;
-    A.gather_h = ctx->gather_h;
+    choose_main_filter(ctx, reqs, n, A);
     A.recon_w = ctx->recon_w;
     A.recon_h = ctx->recon_h;
-    A.main_form = ctx->main_form;
     adaptive = false;
     for (uint32_t s = 0; s < n; s++) {
         for (uint32_t t = 0; t < s; t++)

@@ -103,7 +103,8 @@ struct DofCtx {
     int bvh_rotations;             // passes of tree rotations after the build
     int trace_blocks_per_sm, trace_refill_idle, trace_steps, trace_stats;
     int ray_order_grid, trace_packets;   // 0 / -1: not set, the library chooses (choose_tracer)
-    int gather_w, gather_h, main_form;   // main filter launch shape and form
+    int gather_w, gather_h, main_form;   // main filter launch shape and form (-1: not set, the library chooses)
+    int gather_set;                      // the caller chose the launch shape
     int recon_w, recon_h;                // reconstruction launch shape
     int stack_depth;                     // requested traversal stack entries (raised to the tree's need)
     int ploc_radius;
@@ -293,6 +294,18 @@ __device__ __forceinline__ float4 f4add(float4 a, float4 b) { return make_float4
 __device__ __forceinline__ float4 f4scale(float s, float4 a) { return make_float4(s * a.x, s * a.y, s * a.z, s * a.w); }
 __device__ __forceinline__ float4 f4fma(float s, float4 a, float4 acc) {
     return make_float4(fmaf(s, a.x, acc.x), fmaf(s, a.y, acc.y), fmaf(s, a.z, acc.z), fmaf(s, a.w, acc.w));
+}
+
+// two floats per instruction (packed FP32): each rounds as the scalar operation does
+__device__ __forceinline__ float2 f2fma(float s, float2 a, float2 acc) { return __ffma2_rn(make_float2(s, s), a, acc); }
+__device__ __forceinline__ float4 f4fma2(float s, float4 a, float4 acc) {
+    const float2 l = f2fma(s, make_float2(a.x, a.y), make_float2(acc.x, acc.y));
+    const float2 h = f2fma(s, make_float2(a.z, a.w), make_float2(acc.z, acc.w));
+    return make_float4(l.x, l.y, h.x, h.y);
+}
+__device__ __forceinline__ float4 f4scale2(float s, float4 a) {
+    const float2 l = __fmul2_rn(make_float2(s, s), make_float2(a.x, a.y)), h = __fmul2_rn(make_float2(s, s), make_float2(a.z, a.w));
+    return make_float4(l.x, l.y, h.x, h.y);
 }
 
 // signed CoC diameter (full-resolution px) of depth z

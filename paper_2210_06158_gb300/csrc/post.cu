@@ -150,15 +150,12 @@ __device__ __forceinline__ void main_taps(int i, int j, int W2, int H2, const De
                                           const float *__restrict__ z_h, float R, float z0, float r0, MainAcc &m) {
     const int ring = p.ring;
 #pragma unroll 3
-    for (int t = 0; t < 81; t++) {
-        const float3 u = c_rings[ring][t];
-        const float dist = __fmul_rn(u.z, R);
-        const float x = fmaf(dist, u.x, (float)i), y = fmaf(dist, u.y, (float)j);
+    for (int k = 0; k < 81; k++) {
+        const MainTap t = main_tap(c_rings[ring][k], R);
         float4 s;
         float zi;
-        if (CLAMP) bilinear4z<H>(pre, z_h, W2, H2, x, y, s, zi);
-        else bilinear4z_interior<H>(pre, z_h, W2, x, y, s, zi);
-        main_tap_add(p, dist, z0, r0, s, zi, m);
+        main_sample<CLAMP, H>(pre, z_h, W2, H2, i, j, t, s, zi);
+        main_tap_add(p, t.dist, z0, r0, s, zi, m);
     }
 }
 
@@ -204,67 +201,44 @@ __global__ void __launch_bounds__(512) k_main_filter(const __grid_constant__ AS 
     st_img(out, q, make_float4(m.ax * r, m.ay * r, m.az * r, m.bright * r), f16);
 }
 
-// A4 by columns of four pixels: R is the dilated maximum of the pixel's 8 x 8 tile, so
-// the four pixels (i, 4jt .. 4jt + 3) of one tile column take every tap at the same x
-// (same x weights) and, as long as floor(y + r) = floor(y) + r, at consecutive texel
-// rows.  The thread then reads the five rows y0 .. y0 + 4 once (two texels each) instead
-// of four rows pairs, and finishes pixel r when row r + 1 arrives; otherwise (the rare
-// tap whose rows are not consecutive in FP32) each pixel reads its own two rows.  Every
-// pixel sums its texels in the same order and with the same weights as the other forms.
+// A4 by columns of four pixels: R is the dilated maximum of the pixel's 8 x 8 tile, so the four
+// pixels (i, 4jt .. 4jt + 3) of one tile column take every tap at the same offset, with the
+// same weights, at consecutive texel rows.  The thread reads the five rows y0 .. y0 + 4 once
+// (two texels each) instead of four row pairs, and finishes pixel r when row r + 1 arrives.
+// Every pixel sums its texels in the same order and with the same weights as the other forms.
+//
+// Bound: L1 wavefronts and issue slots together.  Per pixel and tap it reads 2.5 texels where a
+// pixel alone reads 4, and computes the tap's position and weights once for four pixels: 1080p
+// 0.136 -> 0.115 ms, 4K 0.496 -> 0.407 ms (32 x 4) against the form that took positions per
+// pixel.  Columns of eight are even (4K 0.395, 1080p 0.122 ms: spills), of two slower (0.442,
+// 0.125); a cap of 80 or 96 registers gives 0.388-0.408 at 4K and 0.120-0.126 at 1080p.
 template <bool CLAMP, bool H>
 __device__ __forceinline__ void main_strip_taps(int i, int jb, int W2, int H2, const DevParams &p,
                                                 const float4 *__restrict__ pre, const float *__restrict__ z_h, float R,
                                                 const float *z0, const float *r0, MainAcc *m) {
     const int ring = p.ring;
 #pragma unroll 1
-    for (int t = 0; t < 81; t++) {
-        const float3 u = c_rings[ring][t];
-        const float dist = __fmul_rn(u.z, R);
-        const float x = fmaf(dist, u.x, (float)i);
-        const float xf = floorf(x), fx = x - xf;
-        const int x0 = (int)xf;
-        float fy[4];
-        int y0[4];
+    for (int k = 0; k < 81; k++) {
+        const MainTap t = main_tap(c_rings[ring][k], R);
+        const int x0 = i + t.dx, y0 = jb + t.dy;
+        const int xa = CLAMP ? min(max(x0, 0), W2 - 1) : x0, xb = CLAMP ? min(max(x0 + 1, 0), W2 - 1) : x0 + 1;
+        auto row = [&](int r, float4 &a, float4 &b, float &za, float &zb) {
+            const int y = CLAMP ? min(max(y0 + r, 0), H2 - 1) : y0 + r;
+            const size_t q = (size_t)y * W2;
+            ld_pre<H>(pre, z_h, q + xa, a, za);
+            ld_pre<H>(pre, z_h, q + xb, b, zb);
+        };
+        float4 a0, b0;
+        float za0, zb0;
+        row(0, a0, b0, za0, zb0);
 #pragma unroll
         for (int r = 0; r < 4; r++) {
-            const float y = fmaf(dist, u.y, (float)(jb + r));
-            const float yf = floorf(y);
-            fy[r] = y - yf;
-            y0[r] = (int)yf;
-        }
-        if (y0[1] == y0[0] + 1 && y0[2] == y0[0] + 2 && y0[3] == y0[0] + 3) {
-            const int xa = CLAMP ? min(max(x0, 0), W2 - 1) : x0, xb = CLAMP ? min(max(x0 + 1, 0), W2 - 1) : x0 + 1;
-            auto row = [&](int k, float4 &a, float4 &b, float &za, float &zb) {
-                const int y = CLAMP ? min(max(y0[0] + k, 0), H2 - 1) : y0[0] + k;
-                const size_t q = (size_t)y * W2;
-                ld_pre<H>(pre, z_h, q + xa, a, za);
-                ld_pre<H>(pre, z_h, q + xb, b, zb);
-            };
-            float4 a0, b0;
-            float za0, zb0;
-            row(0, a0, b0, za0, zb0);
-#pragma unroll
-            for (int r = 0; r < 4; r++) {
-                float4 a1, b1;
-                float za1, zb1;
-                row(r + 1, a1, b1, za1, zb1);
-                const float w00 = __fmul_rn(1.f - fx, 1.f - fy[r]), w10 = __fmul_rn(fx, 1.f - fy[r]);
-                const float w01 = __fmul_rn(1.f - fx, fy[r]), w11 = __fmul_rn(fx, fy[r]);
-                const float4 s = f4fma(w11, b1, f4fma(w01, a1, f4fma(w10, b0, f4scale(w00, a0))));
-                const float zi = fmaf(w11, zb1, fmaf(w01, za1, fmaf(w10, zb0, __fmul_rn(w00, za0))));
-                main_tap_add(p, dist, z0[r], r0[r], s, zi, m[r]);
-                a0 = a1; b0 = b1; za0 = za1; zb0 = zb1;
-            }
-        } else {
-#pragma unroll
-            for (int r = 0; r < 4; r++) {
-                const float y = fmaf(dist, u.y, (float)(jb + r));
-                float4 s;
-                float zi;
-                if (CLAMP) bilinear4z<H>(pre, z_h, W2, H2, x, y, s, zi);
-                else bilinear4z_interior<H>(pre, z_h, W2, x, y, s, zi);
-                main_tap_add(p, dist, z0[r], r0[r], s, zi, m[r]);
-            }
+            float4 a1, b1, s;
+            float za1, zb1, zi;
+            row(r + 1, a1, b1, za1, zb1);
+            main_blend<H>(t, a0, za0, b0, zb0, a1, za1, b1, zb1, s, zi);
+            main_tap_add(p, t.dist, z0[r], r0[r], s, zi, m[r]);
+            a0 = a1; b0 = b1; za0 = za1; zb0 = zb1;
         }
     }
 }
@@ -332,15 +306,9 @@ __device__ __forceinline__ void main_tile_taps(const float4 *sm_pre, const float
                                                int j, const DevParams &p, float R, float z0, float r0, MainAcc &m) {
     const int ring = p.ring;
 #pragma unroll 3
-    for (int t = 0; t < 81; t++) {
-        const float3 u = c_rings[ring][t];
-        const float dist = __fmul_rn(u.z, R);
-        const float x = fmaf(dist, u.x, (float)i), y = fmaf(dist, u.y, (float)j);
-        const float xf = floorf(x), yf = floorf(y);
-        const float fx = x - xf, fy = y - yf;
-        const int b = ((int)yf - oy) * tw + ((int)xf - ox);
-        const float w00 = __fmul_rn(1.f - fx, 1.f - fy), w10 = __fmul_rn(fx, 1.f - fy);
-        const float w01 = __fmul_rn(1.f - fx, fy), w11 = __fmul_rn(fx, fy);
+    for (int k = 0; k < 81; k++) {
+        const MainTap t = main_tap(c_rings[ring][k], R);
+        const int b = (j + t.dy - oy) * tw + (i + t.dx - ox);
         float4 c00, c10, c01, c11;
         float z00, z10, z01, z11;
         if (H) {
@@ -352,9 +320,10 @@ __device__ __forceinline__ void main_tile_taps(const float4 *sm_pre, const float
             c00 = sm_pre[b]; c10 = sm_pre[b + 1]; c01 = sm_pre[b + tw]; c11 = sm_pre[b + tw + 1];
             z00 = sm_z[b]; z10 = sm_z[b + 1]; z01 = sm_z[b + tw]; z11 = sm_z[b + tw + 1];
         }
-        const float4 s = f4fma(w11, c11, f4fma(w01, c01, f4fma(w10, c10, f4scale(w00, c00))));
-        const float zi = fmaf(w11, z11, fmaf(w01, z01, fmaf(w10, z10, __fmul_rn(w00, z00))));
-        main_tap_add(p, dist, z0, r0, s, zi, m);
+        float4 s;
+        float zi;
+        main_blend<H>(t, c00, z00, c10, z10, c01, z01, c11, z11, s, zi);
+        main_tap_add(p, t.dist, z0, r0, s, zi, m);
     }
 }
 
