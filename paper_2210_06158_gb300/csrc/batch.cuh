@@ -157,7 +157,8 @@ __device__ __forceinline__ const BatchArgs &batch_args(const BatchArgs *a) { ret
 // gives the launch shapes, `as` is what the kernels receive (A itself, or a device
 // pointer to a copy of it)
 template <class AS> void launch_tiles_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistory *timing);  // A1
-template <class AS> void launch_pp_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistory *timing);     // A3 - A5
+// A3 - A5; the main filter waits for `before_main` (none if null)
+template <class AS> void launch_pp_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistory *timing, cudaEvent_t before_main);
 int main_filter_tile_bytes(const BatchArgs &A);   // the main filter's launch form (post.cu)
 template <class AS>
 void launch_mask_b(const BatchArgs &A, const AS &as, bool any_adaptive, cudaStream_t st, DofHistory *timing);

@@ -112,9 +112,10 @@ struct DofCtx {
     int bvh_width_set;             // the caller chose it (and with it one ray per lane, unless packets are set)
     // A frame's ray path (mask .. reconstruction) runs on ray_stream (highest priority)
     // while its post-process filters run on the caller's stream; ev_fork / ev_join order
-    // them around the shared inputs (tiles) and the composite.
+    // them around the shared inputs (tiles) and the composite, ev_mask holds the filters back
+    // until the tracer is next.
     cudaStream_t ray_stream;
-    cudaEvent_t ev_fork, ev_join;
+    cudaEvent_t ev_fork, ev_mask, ev_join;
     std::mutex launch_mu;          // one frame's enqueue at a time on ray_stream
     cudaMemPool_t pool;            // stream-ordered scratch of the rasterising G-buffer producer
 };

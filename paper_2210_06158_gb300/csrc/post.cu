@@ -488,10 +488,11 @@ static void launch_main_filter(const BatchArgs &A, const AS &as, int tile_bytes,
 }
 
 template <class AS>
-void launch_pp_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistory *tm) {
+void launch_pp_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistory *tm, cudaEvent_t before_main) {
     const int n = A.ns;
     k_prefilter<AS><<<A.start[SH_HPX][n], dim3(32, 8), 0, st>>>(as);
     tmark(tm, DOF_K_PREFILTER, st);
+    if (before_main) cudaStreamWaitEvent(st, before_main, 0);
     // the shared-memory form when every session's halo tile fits
     const int tile_bytes = main_filter_tile_bytes(A);
     switch (image_storage_mode(A)) {
@@ -508,5 +509,5 @@ void launch_pp_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistory *
 // the two argument forms: by value (a kernel parameter) and from device memory (graphs)
 template void launch_tiles_b<BatchArgs>(const BatchArgs &, const BatchArgs &, cudaStream_t, DofHistory *);
 template void launch_tiles_b<const BatchArgs *>(const BatchArgs &, const BatchArgs *const &, cudaStream_t, DofHistory *);
-template void launch_pp_b<BatchArgs>(const BatchArgs &, const BatchArgs &, cudaStream_t, DofHistory *);
-template void launch_pp_b<const BatchArgs *>(const BatchArgs &, const BatchArgs *const &, cudaStream_t, DofHistory *);
+template void launch_pp_b<BatchArgs>(const BatchArgs &, const BatchArgs &, cudaStream_t, DofHistory *, cudaEvent_t);
+template void launch_pp_b<const BatchArgs *>(const BatchArgs &, const BatchArgs *const &, cudaStream_t, DofHistory *, cudaEvent_t);
