@@ -9,6 +9,8 @@ raises.
 from __future__ import annotations
 
 import ctypes as C
+import operator
+import struct
 import threading
 from pathlib import Path
 
@@ -139,6 +141,8 @@ def library_path() -> Path:
 def lib():
     """Load libdof.so (built in-tree by `_build.build()`); raises if it is missing."""
     global _lib
+    if _lib is not None:        # set once, after every signature is
+        return _lib
     with _lock:
         if _lib is None:
             if not _LIB_PATH.exists():
@@ -171,28 +175,76 @@ def _ptr(t):
 # structures from the shared input generators
 # ---------------------------------------------------------------------------
 
+# A call that takes a camera and parameters marshals them each time, which is what the shortest
+# calls cost, so both are filled by few large stores.
+_POSE = operator.attrgetter("pos", "right", "up", "fwd", "prev_pos", "prev_right", "prev_up", "prev_fwd")
+_F32 = np.dtype(np.float32)
+_f24, _f4 = C.c_float * 24, C.c_float * 4
+_POSE_OFFSET = DofCamera.pos.offset         # the eight vectors lie one after the other,
+_JITTER_OFFSET = DofCamera.jitter.offset    # and so do the two jitters
+
+
 def camera_struct(cam) -> DofCamera:
     c = DofCamera()
     c.f_m, c.f_number, c.focus_m, c.sensor_w_m = cam.f_m, cam.f_number, cam.focus_m, cam.sensor_w_m
-    for name in ("pos", "right", "up", "fwd", "prev_pos", "prev_right", "prev_up", "prev_fwd"):
-        setattr(c, name, _f3(*[float(x) for x in np.asarray(getattr(cam, name), dtype=np.float32)]))
+    pose = []
+    for v in _POSE(cam):
+        if type(v) is not np.ndarray or v.dtype is not _F32:
+            v = np.asarray(v, dtype=np.float32)
+        v = v.tolist()
+        if len(v) != 3:
+            if len(v) > 3:
+                raise IndexError(f"camera: a vector of {len(v)} components")
+            v += [0.0] * (3 - len(v))
+        pose += v
+    at = C.addressof(c)
+    C.memmove(at + _POSE_OFFSET, _f24(*pose), 96)
     c.frame_index = int(cam.frame_index)
     jx, jy = getattr(cam, "jitter", (0.0, 0.0))
     pjx, pjy = getattr(cam, "prev_jitter", (0.0, 0.0))
-    c.jitter[0], c.jitter[1] = float(jx), float(jy)
-    c.prev_jitter[0], c.prev_jitter[1] = float(pjx), float(pjy)
+    C.memmove(at + _JITTER_OFFSET, _f4(float(jx), float(jy), float(pjx), float(pjy)), 16)
     return c
 
 
+_FLOAT_PARAMS = ("s", "var_w_mask", "depth_range_m", "alpha", "alpha_motion", "var_w_recon", "b_max", "h_edge",
+                 "lod_scale", "lod_max", "max_coc_px", "zof_ramp_px", "cover_ramp_px", "bright_lum",
+                 "bright_ramp", "mask_near_hpx", "z_far_m", "k_a", "k_d", "emit", "taa_alpha")
+_INT_PARAMS = ("m", "spp", "ray_mode", "tile", "seed", "session", "image_storage", "aperture_blades")
+_PACK = struct.Struct("@" + "".join(
+    {C.c_float: "f", C.c_uint32: "I", C.c_uint64: "Q", _f3: "3f"}[t] for _, t in DofParams._fields_))
+assert _PACK.size == C.sizeof(DofParams)
+_defaults = None                            # of every field, in order (dof_params_default)
+
+
 def params_struct(p: dict) -> DofParams:
+    global _defaults
+    if _defaults is None:
+        o = DofParams()
+        lib().dof_params_default(C.byref(o))
+        _defaults = [(k, float if t is C.c_float else list if t is _f3 else int,
+                      tuple(getattr(o, k)) if t is _f3 else getattr(o, k)) for k, t in DofParams._fields_]
+    values = []
+    for k, t, d in _defaults:
+        v = p.get(k, d)
+        if t is not list:
+            values.append(t(v))
+        elif len(v) == 3:
+            values += [float(x) for x in v]
+        else:
+            return _params_by_field(p)
+    try:
+        return DofParams.from_buffer_copy(_PACK.pack(*values))
+    except (struct.error, OverflowError):   # out of a field's range: as the fields convert it
+        return _params_by_field(p)
+
+
+def _params_by_field(p: dict) -> DofParams:
     o = DofParams()
     lib().dof_params_default(C.byref(o))
-    for k in ("s", "var_w_mask", "depth_range_m", "alpha", "alpha_motion", "var_w_recon", "b_max", "h_edge",
-              "lod_scale", "lod_max", "max_coc_px", "zof_ramp_px", "cover_ramp_px", "bright_lum",
-              "bright_ramp", "mask_near_hpx", "z_far_m", "k_a", "k_d", "emit", "taa_alpha"):
+    for k in _FLOAT_PARAMS:
         if k in p:
             setattr(o, k, float(p[k]))
-    for k in ("m", "spp", "ray_mode", "tile", "seed", "session", "image_storage", "aperture_blades"):
+    for k in _INT_PARAMS:
         if k in p:
             setattr(o, k, int(p[k]))
     if "albedo_seed" in p:
