@@ -375,7 +375,9 @@ extern "C" size_t dof_ctx_bytes_in_use(const DofCtx *ctx) { return ctx ? (size_t
 // scene
 // ---------------------------------------------------------------------------
 
-constexpr size_t kPoolKeep = (size_t)256 << 20;
+// what the scratch pool keeps after an upload: the scratch of 2M triangles (growing and trimming it
+// costs such an upload 0.7 of 5 ms); given back to the device when an allocation fails
+constexpr size_t kPoolKeep = (size_t)768 << 20;
 
 extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts, const uint32_t *tri_idx,
                                 const uint32_t *tri_mat, uint32_t n_tris, void *stream, DofScene **out) {
@@ -391,32 +393,29 @@ extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts,
     s->n_tris = n_tris;
     s->n_nodes = n_tris >= 2 ? n_tris - 1 : 0;
     int rc = DOF_OK;
-    float *d_xyz = nullptr;
-    uint32_t *d_idx = nullptr, *d_mat = nullptr;
     if (n_tris == 0) { s->depth = 0; s->root = ~0; ctx_retain(ctx); *out = s; return DOF_OK; }
-    s->tris_bytes = sizeof(float4) * 3 * (size_t)n_tris;
-    s->nodes_bytes = sizeof(BvhNode) * (size_t)s->n_nodes;
-    rc = dof_alloc(ctx, s->tris_bytes, (void **)&s->tris, &s->bytes);
-    if (rc == DOF_OK) rc = dof_alloc(ctx, 4 * (size_t)n_tris, (void **)&s->prim_k, &s->bytes);
-    if (rc == DOF_OK && s->n_nodes) rc = dof_alloc(ctx, s->nodes_bytes, (void **)&s->nodes, &s->bytes);
-    if (rc == DOF_OK) rc = dof_cuda_check(cudaMalloc(&d_xyz, sizeof(float) * 3 * (size_t)n_verts), "scene vertices");
-    if (rc == DOF_OK) rc = dof_cuda_check(cudaMalloc(&d_idx, sizeof(uint32_t) * 3 * (size_t)n_tris), "scene indices");
-    if (rc == DOF_OK && tri_mat) rc = dof_cuda_check(cudaMalloc(&d_mat, sizeof(uint32_t) * (size_t)n_tris), "scene materials");
-    if (rc == DOF_OK) rc = dof_cuda_check(cudaMemcpyAsync(d_xyz, xyz, sizeof(float) * 3 * (size_t)n_verts, cudaMemcpyHostToDevice, st), "upload");
-    if (rc == DOF_OK) rc = dof_cuda_check(cudaMemcpyAsync(d_idx, tri_idx, sizeof(uint32_t) * 3 * (size_t)n_tris, cudaMemcpyHostToDevice, st), "upload");
-    if (rc == DOF_OK && tri_mat) rc = dof_cuda_check(cudaMemcpyAsync(d_mat, tri_mat, sizeof(uint32_t) * (size_t)n_tris, cudaMemcpyHostToDevice, st), "upload");
-    if (rc == DOF_OK) rc = launch_bvh_build(s, d_xyz, n_verts, d_idx, d_mat, ctx->bvh_builder, ctx->ploc_radius, ctx->bvh_rotations, st);
+    {
+        // one allocation for what every tree has (an allocation or a release costs the host 50 us)
+        auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+        const size_t tris = up(sizeof(float4) * 3 * (size_t)n_tris), nodes = up(sizeof(BvhNode) * (size_t)s->n_nodes);
+        s->base_bytes = tris + nodes + 4 * (size_t)n_tris;
+        rc = dof_alloc(ctx, s->base_bytes, &s->base, &s->bytes);
+        if (rc == DOF_OK) {
+            char *p = static_cast<char *>(s->base);
+            s->tris = reinterpret_cast<float4 *>(p);
+            s->nodes = s->n_nodes ? reinterpret_cast<BvhNode *>(p + tris) : nullptr;
+            s->prim_k = reinterpret_cast<int32_t *>(p + tris + nodes);
+        }
+    }
+    if (rc == DOF_OK) rc = launch_bvh_build(s, xyz, n_verts, tri_idx, tri_mat, ctx->bvh_builder, ctx->ploc_radius, ctx->bvh_rotations, st);
     if (rc == DOF_OK) {
         launch_prim_index(s->tris, (int)n_tris, s->prim_k, st);
         rc = dof_cuda_check(cudaStreamSynchronize(st), "scene triangle index");
     }
-    cudaFree(d_xyz); cudaFree(d_idx); cudaFree(d_mat);
     // the pool keeps at most kPoolKeep of the build's scratch for the next call
     if (ctx->pool) cudaMemPoolTrimTo(ctx->pool, kPoolKeep);
     if (rc != DOF_OK) {
-        dof_free(ctx, s->tris, s->tris_bytes);
-        dof_free(ctx, s->prim_k, 4 * (size_t)n_tris);
-        dof_free(ctx, s->nodes, s->nodes_bytes);
+        dof_free(ctx, s->base, s->base_bytes);
         dof_free(ctx, s->nodes4, s->nodes4_bytes);
         delete s;
         return rc;
@@ -431,9 +430,7 @@ extern "C" void dof_scene_destroy(DofScene *s) {
     DofCtx *ctx = s->ctx;
     {
         DeviceGuard g(ctx->device);
-        dof_free(ctx, s->tris, s->tris_bytes);
-        dof_free(ctx, s->prim_k, 4 * (size_t)s->n_tris);
-        dof_free(ctx, s->nodes, s->nodes_bytes);
+        dof_free(ctx, s->base, s->base_bytes);
         dof_free(ctx, s->nodes4, s->nodes4_bytes);
     }
     delete s;

@@ -547,14 +547,15 @@ __global__ void k_ploc_scatter(int count, const int *keep, const int *pos, const
 // G-buffer 0.917 -> 0.615 ms; the 4K tracer (2M triangles) is even.
 //
 // The build itself is bound by latency at the top (a level of few segments cannot fill the
-// chip: 14 levels x 4 launches, 0.4 ms) and by the warps' serial splits at the bottom
-// (k_sah_small 0.67 ms).  Scratch comes from one pool block and the host reads back three
+// chip: 14 levels x 3 launches, 0.4 ms) and by the warps' serial splits at the bottom
+// (k_sah_small).  Scratch comes from one pool block and the host reads back three
 // times, where every PLOC round used to end in a synchronisation (65 of them): upload and
 // first view of 496k triangles 7.1 -> 2.9 ms.
 // ---------------------------------------------------------------------------
 constexpr int kSahBins = 16;             // per axis
 constexpr int kSahSmall = 256;           // clusters a warp finishes alone (uint8 indices)
-constexpr int kSahChunk = 1024;          // clusters of one work item of a large segment
+constexpr int kSahSweep = 10;            // clusters up to which it tries every plane (3 x 10 lanes)
+constexpr int kSahChunk = 512;           // clusters of one work item of a large segment
 constexpr int kSahThreads = 256;
 constexpr int kSahSlotInts = 3 * 7 * kSahBins;   // [axis][count, lo.xyz, hi.xyz][bin]
 constexpr int kSahMaxLevel = 48;         // from here on segments are halved by position, so that
@@ -786,9 +787,11 @@ __global__ void __launch_bounds__(kSahThreads) k_sah_root_bounds(const SahState 
 
 // one level, step 1: the chunks of the large segments fill their bins (in shared memory, then
 // one global atomic per non-empty bin and component)
-__global__ void __launch_bounds__(kSahThreads) k_sah_bin(const SahState *st, int par, const SahSeg *segs, const int2 *items,
+__global__ void __launch_bounds__(kSahThreads) k_sah_bin(SahState *st, int par, const SahSeg *segs, const int2 *items,
                                                          const float4 *lo, const float4 *hi, int *bins) {
     __shared__ int sb[kSahSlotInts];
+    // the tables of the level before are free for the level after
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->n_seg[par ^ 1] = st->n_item[par ^ 1] = 0;
     const int n = st->n_item[par];
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         const int2 w = items[it];
@@ -999,13 +1002,12 @@ __global__ void __launch_bounds__(kSahThreads) k_sah_part(const SahState *st, in
     }
 }
 
-// the finished level's counters are cleared for the level after next
-__global__ void k_sah_next(SahState *st, int par) { st->n_seg[par] = st->n_item[par] = 0; }
-
 // Small segments, one warp each (taken from a counter): the clusters' boxes are loaded into
 // shared memory once, and the warp splits index ranges depth-first, the larger side pushed
-// (at most 8 pending), with the same bins and costs as the large segments.  A segment of n
-// clusters reserves its n - 1 nodes with one atomic.
+// (at most 8 pending), with the same bins and costs as the large segments; up to kSahSweep
+// clusters it tries every plane instead, a lane each, which takes a tenth of the instructions
+// of filling and scanning the bins (0.67 -> 0.38 ms at 265k clusters).  A segment of n clusters
+// reserves its n - 1 nodes with one atomic.
 constexpr int kSmallWarps = 4;
 struct SahSmallWarp {
     float4 lo[kSahSmall], hi[kSahSmall];
@@ -1055,6 +1057,76 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_sah_small(SahState *st, in
                     bl[s][0] = a.x; bl[s][1] = a.y; bl[s][2] = a.z;
                     bh[s][0] = b.x; bh[s][1] = b.y; bh[s][2] = b.z;
                 }
+            } else if (cnt <= kSahSweep) {
+                // every plane of every axis: lane (axis, k) puts the clusters up to the k-th one's
+                // centre (ties by position) on the left
+                const int axis = (int)lane / cnt, i = (int)lane - axis * cnt;
+                const bool mine = axis < 3;
+                auto centre = [&](const float4 &a, const float4 &b, int ax) {
+                    return ax == 0 ? sah_centre(a.x, b.x) : (ax == 1 ? sah_centre(a.y, b.y) : sah_centre(a.z, b.z));
+                };
+                const int own = S.idx[first + i];
+                const float ci = centre(S.lo[own], S.hi[own], axis);
+                float cost = INFINITY;
+                int n = 0;
+#pragma unroll
+                for (int s = 0; s < 2; s++)
+#pragma unroll
+                    for (int q = 0; q < 3; q++) { bl[s][q] = INFINITY; bh[s][q] = -INFINITY; }
+                for (int k = 0; k < cnt; k++) {
+                    const int o = S.idx[first + k];
+                    const float4 a = S.lo[o], b = S.hi[o];
+                    const float ck = centre(a, b, axis);
+                    if (ck < ci || (ck == ci && k <= i)) {
+                        n++;
+                        bl[0][0] = fminf(bl[0][0], a.x); bl[0][1] = fminf(bl[0][1], a.y); bl[0][2] = fminf(bl[0][2], a.z);
+                        bh[0][0] = fmaxf(bh[0][0], b.x); bh[0][1] = fmaxf(bh[0][1], b.y); bh[0][2] = fmaxf(bh[0][2], b.z);
+                    } else {
+                        bl[1][0] = fminf(bl[1][0], a.x); bl[1][1] = fminf(bl[1][1], a.y); bl[1][2] = fminf(bl[1][2], a.z);
+                        bh[1][0] = fmaxf(bh[1][0], b.x); bh[1][1] = fmaxf(bh[1][1], b.y); bh[1][2] = fmaxf(bh[1][2], b.z);
+                    }
+                }
+                if (mine && n > 0 && n < cnt)
+                    cost = half_area(make_float4(bl[0][0], bl[0][1], bl[0][2], 0.f), make_float4(bh[0][0], bh[0][1], bh[0][2], 0.f)) * (float)n +
+                           half_area(make_float4(bl[1][0], bl[1][1], bl[1][2], 0.f), make_float4(bh[1][0], bh[1][1], bh[1][2], 0.f)) * (float)(cnt - n);
+                if (!(cost < INFINITY)) cost = INFINITY;
+                const int low = __reduce_min_sync(0xffffffffu, ord_of(cost));
+                const unsigned at = __ballot_sync(0xffffffffu, mine && cost < INFINITY && ord_of(cost) == low);
+                if (at == 0u || level >= kSahMaxLevel) {
+                    // no plane: by position, both sides with the box of all
+                    nl = cnt / 2;
+#pragma unroll
+                    for (int q = 0; q < 3; q++) {
+                        bl[0][q] = bl[1][q] = float_of(warp_min(ord_of(fminf(bl[0][q], bl[1][q]))));
+                        bh[0][q] = bh[1][q] = float_of(warp_max(ord_of(fmaxf(bh[0][q], bh[1][q]))));
+                    }
+                } else {
+                    const int win = __ffs(at) - 1, wa = win / cnt, wi = win - wa * cnt;
+                    nl = __shfl_sync(0xffffffffu, n, win);
+#pragma unroll
+                    for (int s = 0; s < 2; s++)
+#pragma unroll
+                        for (int q = 0; q < 3; q++) {
+                            bl[s][q] = __shfl_sync(0xffffffffu, bl[s][q], win);
+                            bh[s][q] = __shfl_sync(0xffffffffu, bh[s][q], win);
+                        }
+                    const float cw = __shfl_sync(0xffffffffu, ci, win);
+                    uint8_t v = 0;
+                    bool left = false;
+                    if ((int)lane < cnt) {
+                        v = S.idx[first + (int)lane];
+                        const float ck = centre(S.lo[v], S.hi[v], wa);
+                        left = ck < cw || (ck == cw && (int)lane <= wi);
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, left), all = (1u << cnt) - 1u;
+                    __syncwarp();
+                    if ((int)lane < cnt) {
+                        const int o = left ? __popc(m & lt) : nl + __popc(~m & all & lt);
+                        if (o < cnt) S.idx[first + o] = v;
+                        else atomicExch(bad, 11);
+                    }
+                }
+                __syncwarp();
             } else {
                 // the centroids' bounds, then the bins
                 int l[3] = {0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF}, h[3] = {(int)0x80000000, (int)0x80000000, (int)0x80000000};
@@ -1421,16 +1493,16 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(const unsigned long
     }
 }
 
-// Stable sort of (keys, vals) by the key's low `bits` bits (a multiple of 16: an even
+// Stable sort of (keys, vals) by bits [from, to) of the keys (a multiple of 16 of them: an even
 // number of 8-bit passes); the result ends in (keys, vals), (keys2, vals2) and hist are
 // scratch (hist: 256 * ceil(n / 2048) ints, sums: ceil(256 * ceil(n / 2048) / 2048) ints).
 void device_radix_sort_pairs(unsigned long long *keys, uint32_t *vals, unsigned long long *keys2, uint32_t *vals2,
-                             int n, int *hist, int *sums, cudaStream_t st, int bits = 64) {
+                             int n, int *hist, int *sums, cudaStream_t st, int from = 0, int to = 64) {
     if (n <= 1) return;
     const int nb = (n + kSortTile - 1) / kSortTile;
     unsigned long long *ki = keys, *ko = keys2;
     uint32_t *vi = vals, *vo = vals2;
-    for (int shift = 0; shift < bits; shift += 8) {
+    for (int shift = from; shift < to; shift += 8) {
         k_rs_hist<<<nb, kSortThreads, 0, st>>>(ki, n, shift, hist, nb);
         device_exclusive_scan(hist, hist, kSortBins * nb, sums, st);
         k_rs_scatter<<<nb, kSortThreads, 0, st>>>(ki, vi, ko, vo, n, shift, hist, nb);
@@ -1451,7 +1523,7 @@ size_t sort_pairs_scratch_ints(int n) {
 void sort_pairs_by_low_bits(unsigned long long *keys, uint32_t *vals, unsigned long long *keys2, uint32_t *vals2,
                             int n, int bits, int *scratch, cudaStream_t st) {
     const size_t nh = (size_t)kSortBins * ((n + kSortTile - 1) / kSortTile);
-    device_radix_sort_pairs(keys, vals, keys2, vals2, n, scratch, scratch + nh, st, bits);
+    device_radix_sort_pairs(keys, vals, keys2, vals2, n, scratch, scratch + nh, st, 0, bits);
 }
 
 static inline unsigned blocks_for(size_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -1548,7 +1620,6 @@ void sah_levels(const BuildScratch &b, DofScene *s, int m, int from, int count, 
                                          b.ibuf + 6);
         k_sah_part<<<4 * sms, kSahThreads, 0, st>>>(b.state, p, b.segs[p], b.items[p], b.clo[p], b.chi[p], b.clo[p ^ 1],
                                                     b.chi[p ^ 1], b.segs[p ^ 1], s->nodes, b.ibuf + 6);
-        k_sah_next<<<1, 1, 0, st>>>(b.state, p);
     }
 }
 
@@ -1591,8 +1662,7 @@ int ploc_sah_build(const BuildScratch &b, DofScene *s, int m, int radius, int sm
 }
 }  // namespace
 
-int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const uint32_t *d_idx,
-                     const uint32_t *d_mat, int builder, int ploc_radius, int rotations, cudaStream_t st) {
+int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint32_t *idx, const uint32_t *mat, int builder, int ploc_radius, int rotations, cudaStream_t st) {
     const int n = (int)s->n_tris;
     const int B = 256, sms = s->ctx->sm_count;
     const bool ploc = builder == DOF_BVH_PLOC;
@@ -1603,11 +1673,19 @@ int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const ui
     Arena arena;
     BuildScratch b{};
     b.lay_out(arena, n, ploc);
+    float *d_xyz = arena.take<float>(3 * (size_t)n_verts);
+    uint32_t *d_idx = arena.take<uint32_t>(3 * (size_t)n), *d_mat = mat ? arena.take<uint32_t>(n) : nullptr;
     if (s->ctx->pool) ck(cudaMallocFromPoolAsync((void **)&arena.base, arena.used, s->ctx->pool, st), "bvh scratch");
     else ck(cudaMallocAsync((void **)&arena.base, arena.used, st), "bvh scratch");
     if (rc != DOF_OK) return rc;
     arena.used = 0;
     b.lay_out(arena, n, ploc);
+    d_xyz = arena.take<float>(3 * (size_t)n_verts);
+    d_idx = arena.take<uint32_t>(3 * (size_t)n);
+    d_mat = mat ? arena.take<uint32_t>(n) : nullptr;
+    ck(cudaMemcpyAsync(d_xyz, xyz, sizeof(float) * 3 * (size_t)n_verts, cudaMemcpyHostToDevice, st), "upload");
+    ck(cudaMemcpyAsync(d_idx, idx, sizeof(uint32_t) * 3 * (size_t)n, cudaMemcpyHostToDevice, st), "upload");
+    if (mat) ck(cudaMemcpyAsync(d_mat, mat, sizeof(uint32_t) * (size_t)n, cudaMemcpyHostToDevice, st), "upload");
     int hbuf[16];
     int n_small = n, n_big = 0;
     {
@@ -1628,7 +1706,9 @@ int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const ui
         n_small = n - n_big;
         k_morton<<<blocks_for(n, B), B, 0, st>>>(b.cen, (uint32_t)n, separate ? b.ibuf + 9 : b.ibuf, b.ibuf, share, separate,
                                                  b.keys, b.vals);
-        device_radix_sort_pairs(b.keys, b.vals, b.keys2, b.vals2, n, b.hist, b.sums, st);
+        // the radix tree needs the whole key; the clustering round only looks at neighbours, and the
+        // upper 32 bits (a 1/1000 of the extent per axis) leave its trees as they are
+        device_radix_sort_pairs(b.keys, b.vals, b.keys2, b.vals2, n, b.hist, b.sums, st, ploc ? 32 : 0, 64);
         // sorted (key, triangle) pairs are in (keys, vals)
         k_sorted_tris<<<blocks_for(n, B), B, 0, st>>>(d_xyz, d_idx, d_mat, (uint32_t)n, n_verts, b.vals, s->tris);
         const int m = n_small;
@@ -1669,7 +1749,7 @@ int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const ui
             ck(cudaMemsetAsync(b.n4, 0, sizeof(int) * (kCollapseLevels + 2), st), "memset");
             k_collapse_root<<<1, 1, 0, st>>>(b.root, b.front[0], b.n4);
             for (bool more = true; more && rc == DOF_OK;) {
-                for (int k = 0; k < 20 && levels4 < kCollapseLevels; k++, levels4++)
+                for (int k = 0; k < 16 && levels4 < kCollapseLevels; k++, levels4++)
                     k_collapse<<<2 * sms, 128, 0, st>>>(s->nodes, m - 1, b.front[levels4 & 1], b.n4 + 1 + levels4, b.wide, m - 1,
                                                        b.n4, b.front[(levels4 + 1) & 1], b.n4 + 2 + levels4, b.ibuf + 6);
                 k_summary<<<1, 1, 0, st>>>(b.ibuf, b.state, b.root, s->nodes, m - 1, b.summary);

@@ -125,7 +125,8 @@ struct DofScene {
     uint32_t n_tris, n_nodes, depth;
     uint32_t n_tree, n_large;      // triangles in the tree / tested directly
     int root;
-    size_t tris_bytes, nodes_bytes;  // allocation sizes (for the context's budget)
+    void *base;                    // one allocation: tris, nodes, prim_k
+    size_t base_bytes;
     Bvh4Node *nodes4;
     size_t nodes4_bytes;
     int root4, n_nodes4, depth4;
@@ -207,8 +208,8 @@ void ctx_release(DofCtx *ctx);   // frees the context with its last reference
 void dof_free(DofCtx *ctx, void *ptr, size_t bytes);
 
 // launch wrappers (one per kernel group, defined in the .cu files)
-int launch_bvh_build(DofScene *s, const float *d_xyz, uint32_t n_verts, const uint32_t *d_idx,
-                     const uint32_t *d_mat, int builder, int ploc_radius, int rotations, cudaStream_t st);
+// xyz, idx, mat: host arrays
+int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint32_t *idx, const uint32_t *mat, int builder, int ploc_radius, int rotations, cudaStream_t st);
 void launch_primary(const DevCam &cam, const DevParams &p, const SceneDev &sc, float4 *color, float *depth, float4 *normal,
                     int32_t *prim, cudaStream_t st);
 // host-side tally of this library's kernel launches (dof_launch_count); each launch
