@@ -777,29 +777,34 @@ static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint3
 // The tracer of a step whose context leaves it open: warp packets, taken in pixel order, but
 // by lens cells of 1/8 aperture where the blur of the far field (cocK, its asymptotic
 // diameter) spans 11 px and more, so that a packet's rays leave one patch of the lens.  One ray
-// per lane stays where both the aperture is wide (cocK >= 6) and the rays are too few to fill
-// the chip's warps more than twice: the packets' unions are then large and the longest one
-// sets the time.  Measured (tracer + mask kernel, us; packets against one ray per lane at its
-// former default order):
+// per lane stays where the rays are too few to fill the chip's warps more than twice and the
+// packets' unions are large, so that the longest one sets the time: through a wide aperture
+// (cocK >= 6) below 400k rays, and in scenes of 32k triangles and more below 300k.  Measured
+// (tracer + mask kernel, us; packets against one ray per lane at its former default order):
 //   35 mm f/2 (cocK 1.6), 1080p: 1 ray 171 / 277, 2 rays 232 / 491, 4 rays 409 / 919;
 //     768p, up to 4 rays by Eq. 4: 191 / 328
-//   50 mm f/1.4, 256 x 144: 53 / 60; 720p, 4 rays (cocK 4.2): 101 / 189
+//   the same lens, one ray (tracer alone, pixel order): 360p 114 / 92, 540p 127 / 106, 720p 137 /
+//     120, 1080p 157 / 224; four sessions of 272 x 204 to 544 x 408 in a step 0.44 / 0.24 ms
+//   50 mm f/1.4, 2.8k triangles, 256 x 144: 53 / 60; 540p 46 / 56; 720p, 4 rays (cocK 4.2) 101 / 189
 //   85 mm f/1.2, 1080p (cocK 16): 1 ray 234 / 239, 4 rays 593 / 736; 4K (cocK 32) 583 / 733;
 //     720p, up to 8 rays (cocK 10.7): 634 in pixel order, 601 by lens cells / 645;
 //     540p, 1 ray (cocK 8): 137 / 110, 4 rays 219 / 227
 static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
-    double rays = 0, wide_rays = 0;
+    double rays = 0, wide_rays = 0, dense_rays = 0;
     for (int s = 0; s < A.ns; s++) {
         const SessDesc &d = A.s[s];
         const double r = (double)d.N * (d.p.ray_mode ? 0.5 * d.p.m : (double)d.p.spp);
         rays += r;
         if (d.cam.cocK >= 6.f) wide_rays += r;
+        if (d.sc.n_tris >= 32768) dense_rays += r;
     }
+    const bool few = (wide_rays > 0.5 * rays && rays < 400e3) || (dense_rays > 0.5 * rays && rays < 300e3);
     if (ctx->trace_packets >= 0) A.packets = ctx->trace_packets;
     else if (ctx->bvh_width_set) A.packets = 0;
-    else A.packets = !(wide_rays > 0.5 * rays && rays < 400e3);
+    else A.packets = !few;
     for (int s = 0; s < A.ns; s++) {
-        const int g = A.packets ? (A.s[s].cam.cocK >= 11.f ? 8 : 1) : 4;
+        const float k = A.s[s].cam.cocK;
+        const int g = A.packets ? (k >= 11.f ? 8 : 1) : (k >= 6.f ? 4 : 1);
         A.s[s].lens_grid = ctx->ray_order_grid ? ctx->ray_order_grid : g;
     }
 }
