@@ -8,6 +8,8 @@
 
 #include "batch.cuh"
 
+#include <algorithm>
+
 int post_init_tables();
 int recon_init_tables();
 
@@ -745,7 +747,12 @@ static void shape_grid(const BatchArgs &A, const SessDesc &d, const DofHistory *
             gy = ((int)h->H2 + rows - 1) / rows;
             break;
         }
-        case SH_RECON: gx = ((int)h->W2 + A.recon_w - 1) / A.recon_w; gy = ((int)h->H2 + A.recon_h - 1) / A.recon_h; break;
+        case SH_RECON: {
+            const int w = d.recon_split ? A.recon_w / 4 : A.recon_w;
+            gx = ((int)h->W2 + w - 1) / w;
+            gy = ((int)h->H2 + A.recon_h - 1) / A.recon_h;
+            break;
+        }
         case SH_HPX: gx = ((int)h->W2 + 31) / 32; gy = ((int)h->H2 + 7) / 8; break;
         case SH_FPX: gx = ((int)h->W + 31) / 32; gy = ((int)h->H + 7) / 8; break;
         default: gx = ((int)h->N + 127) / 128; gy = 1; break;   // SH_SHADE
@@ -773,6 +780,9 @@ static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint3
         A.main_form = 0;
     }
 }
+
+// half-resolution pixels below which a session's reconstruction takes four lanes per pixel
+constexpr int kReconSplitPx = 40000;
 
 // The tracer of a step whose context leaves it open: warp packets, taken in pixel order, but
 // by lens cells of 1/8 aperture where the blur of the far field (cocK, its asymptotic
@@ -815,8 +825,11 @@ static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchAr
     memset(&A, 0, sizeof(A));
     A.ns = (int)n;
     choose_main_filter(ctx, reqs, n, A);
-    A.recon_w = ctx->recon_w;
-    A.recon_h = ctx->recon_h;
+    // split sessions need whole warps along x: a block of another width is taken as 32 wide
+    bool split = false;
+    for (uint32_t s = 0; s < n; s++) split |= reqs[s].hist && (int)reqs[s].hist->N < kReconSplitPx;
+    A.recon_w = split && ctx->recon_w % 32 ? 32 : ctx->recon_w;
+    A.recon_h = A.recon_w == ctx->recon_w ? ctx->recon_h : std::max(2, ctx->recon_w * ctx->recon_h / 32);
     adaptive = false;
     for (uint32_t s = 0; s < n; s++) {
         for (uint32_t t = 0; t < s; t++)
@@ -825,6 +838,7 @@ static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchAr
         int rc = make_desc(ctx, reqs[s], A.s[s]);
         if (rc) return rc;
         adaptive |= A.s[s].p.ray_mode == 1;
+        A.s[s].recon_split = A.s[s].N < kReconSplitPx;
         for (int sh = 0; sh < SH_COUNT; sh++) {
             int gx, gy;
             shape_grid(A, A.s[s], reqs[s].hist, sh, gx, gy);

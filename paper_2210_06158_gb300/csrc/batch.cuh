@@ -26,6 +26,7 @@ struct SessDesc {
     int gx[SH_COUNT];              // blocks per row of each shape
     int N, max_rays, valid, record_rays;
     int lens_grid;                 // tracer work order: lens-cell grid of the mask kernel (1 = pixel order)
+    int recon_split;               // the reconstruction takes four lanes per pixel
     // frame inputs and output (caller-owned)
     const float4 *color;
     const float *depth;

@@ -257,12 +257,13 @@ __device__ __forceinline__ void bilin_acc(const MipLevel &L, float x, float y, f
     b.y = fmaf(w11, c11.y, fmaf(w01, c01.y, fmaf(w10, c10.y, fmaf(w00, c00.y, b.y))));
 }
 
+// taps [k0, k1) of the 81
 template <bool CLAMP, bool H>
 __device__ __forceinline__ void recon_taps(const MipLevel &L0, const MipLevel &L1, int i, int j, float R, float t,
-                                           float inv_ramp, int ring, float4 &num, float &den) {
+                                           float inv_ramp, int ring, int k0, int k1, float4 &num, float &den) {
     const float fi = (float)i, fj = (float)j, t0 = 1.f - t;
 #pragma unroll 3
-    for (int k = 0; k < 81; k++) {
+    for (int k = k0; k < k1; k++) {
         const float3 u = c_rings[ring][k];
         // dist and the cover weight D are rounded explicitly (no contraction left to the
         // compiler), so that every instance of this kernel computes the same bits
@@ -280,19 +281,84 @@ __device__ __forceinline__ void recon_taps(const MipLevel &L0, const MipLevel &L
     }
 }
 
+// The reconstruction of a small session: four lanes of a warp take a run of a pixel's taps each
+// (lane & 7: the pixel, lane >> 3: the run, of 21, 20, 20 and 20 taps), and the runs' sums are
+// added in order.  One thread per pixel leaves most of the chip idle then, and the chain of its
+// 81 taps sets the time: 256 x 144 31 -> 17 us, 480 x 270 32 -> 27, 640 x 360 47 -> 41 but in a
+// batch that fills the chip it costs 10% (960 x 540 67 -> 74).  Which sessions take it depends on their own size
+// alone (SessDesc::recon_split), so that a session's bits do not depend on its batch.
+template <bool H>
+__device__ __forceinline__ void recon_split(const SessDesc &S, int bx, int by) {
+    const DevParams &p = S.p;
+    const int W2 = S.cam.W2, H2 = S.cam.H2, mL = S.mip_L;
+    const int reach = (int)ceilf(p.rmax_hpx) + (2 << (mL - 1)) + 2;
+    const int lane = (int)(threadIdx.x & 31u), run = lane >> 3;
+    const int i = bx + (int)(threadIdx.x >> 5) * 8 + (lane & 7), j = by + (int)threadIdx.y;
+    const bool interior = bx - reach >= 0 && by - reach >= 0 && bx + (int)blockDim.x / 4 + reach < W2 &&
+                          by + (int)blockDim.y + reach < H2;
+    const bool in = i < W2 && j < H2;
+    const size_t q = in ? (size_t)j * W2 + i : 0;
+    float4 *out = S.recon;
+    float4 num = make_float4(0.f, 0.f, 0.f, 0.f), o = num;
+    float den = 0.f, b = 0.f;
+    bool taps = false;
+    if (in) {
+        if (__ldg(&S.nrays[q]) <= 0) {
+            if (run == 0) st_img(out, q, num, H);
+        } else {
+            o = ld_img(S.rt_med, q, H);
+            b = fminf(fmaxf(__ldg(&S.var_out[q]) * p.var_w_recon, 0.f), p.b_max);
+            taps = b >= 5.9604645e-8f;       // as below
+            if (!taps && run == 0) st_img(out, q, make_float4(o.x + 0.f, o.y + 0.f, o.z + 0.f, o.w + 0.f), H);
+        }
+    }
+    if (taps) {
+        const float R = __ldg(&S.ct[q]);
+        const float lod = fminf(fmaxf(R * p.lod_scale, 0.f), p.lod_max);
+        int l0 = (int)floorf(lod);
+        float t = lod - (float)l0;
+        if (l0 >= mL - 1) { l0 = mL - 1; t = 0.f; }
+        const MipLevel L0 = mip_level(S, l0), L1 = mip_level(S, min(l0 + 1, mL - 1));
+        const int k0 = run ? 1 + 20 * run : 0, k1 = 21 + 20 * run;
+        if (interior) recon_taps<false, H>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, k0, k1, num, den);
+        else recon_taps<true, H>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, k0, k1, num, den);
+    }
+    float4 n = num;
+    float d = den;
+#pragma unroll
+    for (int r = 1; r < 4; r++) {
+        const int from = (lane & 7) + 8 * r;
+        n = f4add(n, make_float4(__shfl_sync(0xffffffffu, num.x, from), __shfl_sync(0xffffffffu, num.y, from),
+                                 __shfl_sync(0xffffffffu, num.z, from), __shfl_sync(0xffffffffu, num.w, from)));
+        d += __shfl_sync(0xffffffffu, den, from);
+    }
+    if (run != 0 || !taps) return;
+    const float4 f = d > 0.f ? f4scale(1.f / d, n) : o;
+    st_img(out, q, make_float4(lerpf(o.x, f.x, b), lerpf(o.y, f.y, b), lerpf(o.z, f.z, b), lerpf(o.w, f.w, b)), H);
+}
+
 // A11: reconstruction.  Blocks whose footprint (+-rmax + 2, at every level) lies
 // inside the image take taps without index clamping.  kStore: the launch's image storage
 // (image_storage_mode); the specialised instances hold the code of one storage only, and
 // with it fewer registers.  72 registers hold either storage's taps without spilling
 // (three 256-thread blocks per SM; a cap of 64 spilled the FP32 form's state through
 // L1, the unit that bounds it, and was 1-2% slower).
-template <class AS, int kStore>
+// kSplit: 0 no session of the launch is split (recon_split), 1 all are, 2 some are; the
+// unsplit instances stay free of the other form's registers.
+template <class AS, int kStore, int kSplit>
 __global__ void __maxnreg__(72) k_recon(const __grid_constant__ AS as_) {
     const BatchArgs &A = batch_args(as_);
     int i, j;
     const SessDesc &S = block_session(A, SH_RECON, i, j);
     const DevParams &p = S.p;
     const bool f16 = kStore == 2 ? p.f16 != 0 : kStore == 1;
+    if (kSplit == 1 || (kSplit == 2 && S.recon_split)) {
+        const int bx = (i - (int)threadIdx.x) / 4, by = j - (int)threadIdx.y;    // its blocks are a quarter as wide
+        if (f16) recon_split<true>(S, bx, by);
+        else recon_split<false>(S, bx, by);
+        return;
+    }
+    if constexpr (kSplit != 1) {
     const int W2 = S.cam.W2, H2 = S.cam.H2;
     const int mL = S.mip_L;
     const float4 *__restrict__ med = S.rt_med;
@@ -325,14 +391,15 @@ __global__ void __maxnreg__(72) k_recon(const __grid_constant__ AS as_) {
     float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
     float den = 0.f;
     if (f16) {
-        if (interior) recon_taps<false, true>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, num, den);
-        else recon_taps<true, true>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, num, den);
+        if (interior) recon_taps<false, true>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, 0, 81, num, den);
+        else recon_taps<true, true>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, 0, 81, num, den);
     } else {
-        if (interior) recon_taps<false, false>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, num, den);
-        else recon_taps<true, false>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, num, den);
+        if (interior) recon_taps<false, false>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, 0, 81, num, den);
+        else recon_taps<true, false>(L0, L1, i, j, R, t, p.inv_cover_ramp, p.ring, 0, 81, num, den);
     }
     float4 f = den > 0.f ? f4scale(1.f / den, num) : o;
     st_img(out, q, make_float4(lerpf(o.x, f.x, b), lerpf(o.y, f.y, b), lerpf(o.z, f.z, b), lerpf(o.w, f.w, b)), f16);
+    }
 }
 
 // A12: composite.  One thread per half-resolution pixel (i, j) writes its 2x2
@@ -513,11 +580,17 @@ void launch_recon_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistor
     tmark(tm, DOF_K_MEDIAN_RT, st);
     tmark(tm, DOF_K_MIPS, st);
     const dim3 rg(A.start[SH_RECON][n]), rb(A.recon_w, A.recon_h);
-    switch (image_storage_mode(A)) {
-    case 0: k_recon<AS, 0><<<rg, rb, 0, st>>>(as); break;
-    case 1: k_recon<AS, 1><<<rg, rb, 0, st>>>(as); break;
-    default: k_recon<AS, 2><<<rg, rb, 0, st>>>(as); break;
-    }
+    int n_split = 0;
+    for (int k = 0; k < n; k++) n_split += A.s[k].recon_split != 0;
+    const int split = n_split == 0 ? 0 : (n_split == n ? 1 : 2);
+    const int mode = image_storage_mode(A);
+    if (mode == 2) k_recon<AS, 2, 2><<<rg, rb, 0, st>>>(as);
+    else if (mode == 1 && split == 0) k_recon<AS, 1, 0><<<rg, rb, 0, st>>>(as);
+    else if (mode == 1 && split == 1) k_recon<AS, 1, 1><<<rg, rb, 0, st>>>(as);
+    else if (mode == 1) k_recon<AS, 1, 2><<<rg, rb, 0, st>>>(as);
+    else if (split == 0) k_recon<AS, 0, 0><<<rg, rb, 0, st>>>(as);
+    else if (split == 1) k_recon<AS, 0, 1><<<rg, rb, 0, st>>>(as);
+    else k_recon<AS, 0, 2><<<rg, rb, 0, st>>>(as);
     count_launches(2);
     tmark(tm, DOF_K_RECON, st);
 }
@@ -528,12 +601,20 @@ void preload_recon_kernels() {
     cudaFuncAttributes a;
     cudaFuncGetAttributes(&a, k_taa<BatchArgs>);
     cudaFuncGetAttributes(&a, k_taa<const BatchArgs *>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 0>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 1>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 2>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 0>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 1>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 2>);
+    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 0, 0>);
+    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 0, 1>);
+    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 0, 2>);
+    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 1, 0>);
+    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 1, 1>);
+    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 1, 2>);
+    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 2, 2>);
+    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 0, 0>);
+    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 0, 1>);
+    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 0, 2>);
+    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 1, 0>);
+    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 1, 1>);
+    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 1, 2>);
+    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 2, 2>);
     cudaGetLastError();
 }
 
