@@ -278,11 +278,12 @@ class Context:
             pass
 
     def set_bvh_builder(self, name: str):
-        """'ploc' (default) or 'lbvh' for scenes uploaded afterwards."""
+        """'ploc' (default: a clustering round, then surface-area splits) or 'lbvh' for scenes uploaded
+        afterwards."""
         _check(lib().dof_ctx_set_option(self.ptr, 1, {"ploc": 0, "lbvh": 1}[name]))
 
     def set_ploc_radius(self, r: int):
-        """PLOC search radius for scenes uploaded afterwards (tree quality vs build time)."""
+        """Search radius of the clustering round for scenes uploaded afterwards."""
         _check(lib().dof_ctx_set_option(self.ptr, 5, int(r)))
 
     def set_bvh_rotations(self, passes: int):
@@ -290,7 +291,7 @@ class Context:
         _check(lib().dof_ctx_set_option(self.ptr, 13, int(passes)))
 
     def set_bvh_width(self, width: int):
-        """Tree the rays traverse: 4 (collapsed 4-wide nodes, default) or 2 (binary)."""
+        """Tree that one ray per lane traverses: 4 (collapsed 4-wide nodes, default) or 2 (binary)."""
         _check(lib().dof_ctx_set_option(self.ptr, 6, int(width)))
 
     def set_trace(self, blocks_per_sm=None, refill_idle=None, steps=None, bvh_width=None, ray_grid=None, stack=None,

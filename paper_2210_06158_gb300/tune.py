@@ -1,4 +1,4 @@
-"""Autotuners of the ray tracer -- the BVH build (PLOC search radius), the persistent
+"""Autotuners of the ray tracer -- the BVH build (the clustering round's radius), the persistent
 tracer's tree width, work order, launch shape and scheduling -- and of the 81-tap
 gathers' launch shape and main-filter form.
 
