@@ -1793,6 +1793,7 @@ int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint
             s->n_nodes4 = n_front[0];
             s->nodes4_bytes = sizeof(Bvh4Node) * (size_t)s->n_nodes4;
             rc = dof_alloc(s->ctx, s->nodes4_bytes, (void **)&s->nodes4, &s->bytes);
+            if (rc != DOF_OK) goto done;
             ck(cudaMemcpyAsync(s->nodes4, b.wide, s->nodes4_bytes, cudaMemcpyDeviceToDevice, st), "collapse copy");
             s->root4 = 0;
             // bounds of the tree's triangles

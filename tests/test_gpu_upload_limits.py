@@ -1,0 +1,36 @@
+"""Uploads at the memory budget's limits: what is refused leaves nothing behind."""
+
+import numpy as np
+import pytest
+
+from synth import Scene
+
+pytestmark = pytest.mark.gpu
+
+
+def _scene(n):
+    rng = np.random.default_rng(n)
+    c = rng.uniform((-1.5, -1, 2), (1.5, 1, 6), (n, 1, 3))
+    v = (c + 0.05 * rng.uniform(-1, 1, (n, 3, 3))).astype(np.float32).reshape(-1, 3)
+    return Scene(v, np.arange(3 * n, dtype=np.uint32).reshape(n, 3), np.zeros(n, np.uint32), 1)
+
+
+def test_a_budget_without_room_for_the_wide_tree_leaves_no_error_behind():
+    """The budget admits the triangles and the binary tree but not the 4-wide nodes: the upload
+    reports that, gives back what it took and leaves no error pending for the next library's check on
+    this thread."""
+    import torch
+    from paper_2210_06158_gb300 import dof
+    n = 5000
+    with_all = dof.Context(0)
+    sc = dof.Scene(with_all, _scene(n))
+    total = with_all.bytes_in_use
+    assert sc.info().n_nodes4 > 100
+    ctx = dof.Context(0, mem_budget_bytes=total - 1024)
+    with pytest.raises(dof.DofError) as e:
+        dof.Scene(ctx, _scene(n))
+    assert e.value.code == -3
+    assert ctx.bytes_in_use == 0
+    x = torch.ones(1000, device="cuda") * 2         # a launch whose error check is torch's
+    torch.cuda.synchronize()
+    assert float(x.sum()) == 2000.0
