@@ -180,13 +180,13 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
                                          * set the library chooses per session.  Same hits either way */
 /* block of the main filter's 81-tap gather in half-resolution pixels: value = width |
  * height << 16, width >= 8, width * height a multiple of 32 in 64..512 (until it is set:
- * 32 x 8, and 32 x 2 for the columns of DOF_OPT_MAIN_FILTER_FORM) */
+ * 32 x 8, and 32 x 2 for the columns that the library takes by itself) */
 #define DOF_OPT_GATHER_BLOCK        8
 /* the main filter's reads: 0 = the block's halo tile staged in shared memory when it fits in
  * 64 KB, else through L1; 1 = through L1; 2 = the halo tile whenever it fits in the SM's
  * opt-in shared memory; 3 = through L1, each thread taking a column of four pixels of one 8 x 8
- * tile (they share the tile's radius, so their taps share texel rows).  Until it is set, and
- * with 1, the library takes the columns where the step has pixels enough for them.  Same
+ * tile (they share the tile's radius, so their taps share texel rows).  Until it is set the
+ * library takes the columns where the step has pixels enough for them, else form 0.  Same
  * results either way */
 #define DOF_OPT_MAIN_FILTER_FORM    9
 /* block of the reconstruction's 81-tap gather, encoded as DOF_OPT_GATHER_BLOCK (default 32 x 8) */

@@ -759,13 +759,13 @@ static void shape_grid(const BatchArgs &A, const SessDesc &d, const DofHistory *
     }
 }
 
-// The main filter's form and block.  Left open, or left to reads through L1 (form 1): columns of
-// four pixels from kColumnsMinPx half-resolution pixels on, where they fill the chip's warps
-// twice, in blocks of 32 x 2 threads unless the caller set them.  Below, the halo tile where it
-// fits (form 1: one pixel per thread).  Measured (us, FP32; halo tile 32 x 8 / one pixel per
-// thread 32 x 4 / columns 32 x 2): 360p 26.3 / 26.6 / 34.4, 540p 44.6 / 45.2 / 44.2, 720p 60.7 /
-// 71.6 / 58.1, 1080p 127 / 133 / 115, with the 85 mm lens (radius to 32) 540p 56 / 55 / 55 and
-// 1080p 146 / 146 / 123; 4K, the tile past 64 KB: - / 511 / 407 (32 x 4).
+// The main filter's form and block.  Left open: columns of four pixels from kColumnsMinPx
+// half-resolution pixels on, where they fill the chip's warps twice, in blocks of 32 x 2 threads
+// unless the caller set them; below, the halo tile where it fits.  A form that the caller set is
+// the one that runs.  Measured (us, FP32; halo tile 32 x 8 / one pixel per thread 32 x 4 /
+// columns 32 x 2): 360p 26.3 / 26.6 / 34.4, 540p 44.6 / 45.2 / 44.2, 720p 60.7 / 71.6 / 58.1, 1080p
+// 127 / 133 / 115, with the 85 mm lens (radius to 32) 540p 56 / 55 / 55 and 1080p 146 / 146 /
+// 123; 4K, the tile past 64 KB: - / 511 / 407 (32 x 4).
 constexpr long long kColumnsMinPx = 180000;
 static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchArgs &A) {
     long long px = 0;
@@ -773,12 +773,9 @@ static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint3
     A.main_form = ctx->main_form;
     A.gather_w = ctx->gather_w;
     A.gather_h = ctx->gather_h;
-    if ((ctx->main_form == -1 || ctx->main_form == 1) && px >= kColumnsMinPx) {
-        A.main_form = 3;
-        if (!ctx->gather_set) A.gather_h = 2;
-    } else if (ctx->main_form == -1) {
-        A.main_form = 0;
-    }
+    if (ctx->main_form >= 0) return;
+    A.main_form = px >= kColumnsMinPx ? 3 : 0;
+    if (A.main_form == 3 && !ctx->gather_set) A.gather_h = 2;
 }
 
 // half-resolution pixels below which a session's reconstruction takes four lanes per pixel

@@ -314,8 +314,8 @@ class Context:
         warps, 64..512 threads) -- and the main filter's form: 0 = halo tile in shared
         memory when it fits in 64 KB, 1 = through L1, 2 = halo tile up to the SM's opt-in
         shared memory, 3 = through L1 by columns of four pixels (no effect on results).
-        Until it is set, and with 1, the library takes the columns where a step has pixels
-        enough for them."""
+        Until it is set the library takes the columns where a step has pixels enough for
+        them, else form 0."""
         for opt, b in ((8, block), (10, recon_block)):
             if b is not None:
                 w, h = (int(v) for v in b)
