@@ -781,6 +781,15 @@ static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint3
 // half-resolution pixels below which a session's reconstruction takes four lanes per pixel
 constexpr int kReconSplitPx = 40000;
 
+// Lens-cell grid of each session's rays, by the tracer of the step: the caller's (grid), or where that
+// is open (0) the one that choose_tracer's figures favour.
+static void choose_lens_cells(int grid, BatchArgs &A) {
+    for (int s = 0; s < A.ns; s++) {
+        const float k = A.s[s].cam.cocK;
+        A.s[s].lens_grid = grid ? grid : (A.packets ? (k >= 11.f ? 8 : 1) : (k >= 6.f ? 4 : 1));
+    }
+}
+
 // The tracer of a step whose context leaves it open: warp packets, taken in pixel order, but
 // by lens cells of 1/8 aperture where the blur of the far field (cocK, its asymptotic
 // diameter) spans 11 px and more, so that a packet's rays leave one patch of the lens.  One ray
@@ -809,11 +818,7 @@ static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
     if (ctx->trace_packets >= 0) A.packets = ctx->trace_packets;
     else if (ctx->bvh_width_set) A.packets = 0;
     else A.packets = !few;
-    for (int s = 0; s < A.ns; s++) {
-        const float k = A.s[s].cam.cocK;
-        const int g = A.packets ? (k >= 11.f ? 8 : 1) : (k >= 6.f ? 4 : 1);
-        A.s[s].lens_grid = ctx->ray_order_grid ? ctx->ray_order_grid : g;
-    }
+    choose_lens_cells(ctx->ray_order_grid, A);
 }
 
 // The batch descriptor of one step of `reqs` (validated); *adaptive: a session uses Eq. 4.
@@ -1060,22 +1065,23 @@ extern "C" int dof_graph_launch(DofGraph *g, const DofFrameReq *reqs, uint32_t n
     bool adaptive = false;
     int rc = build_batch(ctx, reqs, n, A, adaptive);
     if (rc) return rc;
-    // a tracer that the library chose is the captured one whatever the cameras are now
+    // the tracer's options are those of the capture, and a tracer that the library chose is the
+    // captured one whatever the cameras are now
+    A.refill_idle = g->refill_idle;
+    A.steps_per_round = g->steps_per_round;
+    A.stack_depth = g->stack_depth;
     if (ctx->trace_packets == g->packets_opt && ctx->bvh_width_set == g->width_set) A.packets = g->packets;
-    for (int s = 0; s < A.ns; s++)
-        if (g->lens_grid) A.s[s].lens_grid = g->lens_grid;
+    choose_lens_cells(g->lens_grid, A);
+    // packets traverse the binary tree: whether there is a 4-wide one matters to one ray per lane
+    const bool other_tree = !(A.packets && g->packets) && all_wide(A) != g->wide;
     if (A.packets && g->packets && packet_capacity(A) > g->packet_need)
         return dof_set_error(DOF_ERR_MISMATCH, "dof_graph_launch: a scene's tree is deeper than the captured stack");
-    if (memcmp(A.start, g->start, sizeof(A.start)) != 0 || adaptive != g->adaptive || all_wide(A) != g->wide ||
+    if (memcmp(A.start, g->start, sizeof(A.start)) != 0 || adaptive != g->adaptive || other_tree ||
         ctx->sm_count * ctx->trace_blocks_per_sm != g->trace_blocks || main_filter_tile_bytes(A) != g->main_tile ||
         A.gather_w != g->gather_w || A.gather_h != g->gather_h || A.main_form != g->main_form ||
         A.recon_w != g->recon_w || A.recon_h != g->recon_h || A.packets != g->packets || A.stats != g->stats ||
         image_storage_mode(A) != g->store_mode || any_taa(A) != g->taa)
         return dof_set_error(DOF_ERR_MISMATCH, "dof_graph_launch: launch shapes differ from the captured step");
-    // the kernels' scheduling knobs come from the staged copy; keep the captured ones
-    A.refill_idle = g->refill_idle;
-    A.steps_per_round = g->steps_per_round;
-    A.stack_depth = g->stack_depth;
     cudaStream_t st = (cudaStream_t)stream;
     cudaGetLastError();
     // the previous launch's copy has consumed the staging buffer
