@@ -173,7 +173,8 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
 #define DOF_OPT_PLOC_RADIUS         5   /* nearest-neighbour search radius of the clustering round, 1..256
                                          * (default 48) */
 #define DOF_OPT_BVH_WIDTH           6   /* tree that one ray per lane traverses: 4 (default) = the binary tree
-                                         * collapsed to 4-wide nodes, 2 = the binary tree; same hits either way */
+                                         * collapsed to 4-wide nodes, 2 = the binary tree (it does not choose
+                                         * the tracer: DOF_OPT_TRACE_PACKETS); same hits either way */
 #define DOF_OPT_RAY_ORDER_GRID      7   /* order in which the tracer takes a block's rays: grouped by the
                                          * cell of their lens point on a g x g grid over the aperture,
                                          * g = 1..16, cells in Morton order; 1 = pixel by pixel.  Until it is
@@ -197,9 +198,9 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
 #define DOF_OPT_TRACE_STACK         11
 /* the tracer: 0 = one ray per lane, persistent threads with dynamic fetch, on the tree of
  * DOF_OPT_BVH_WIDTH; 1 = the 32 rays of a warp as one packet (one node sequence per warp, each
- * lane testing with its own ray and best hit), always on the binary tree.  Until this option
- * or DOF_OPT_BVH_WIDTH (which implies 0) is set the library chooses per step, by the
- * aperture and the number of rays.  Same hits either way */
+ * lane testing with its own ray and best hit), always on the binary tree.  Until it is set the
+ * library chooses per step, by the aperture, the number of rays and the size of the
+ * scenes.  Same hits either way */
 #define DOF_OPT_TRACE_PACKETS       12
 /* passes of tree rotations after the BVH build of scenes uploaded afterwards, 0..16
  * (default 0): each swaps, bottom-up, a child with a grandchild where that shrinks the

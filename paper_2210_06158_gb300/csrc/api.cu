@@ -235,7 +235,6 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
     c->gather_set = 0;
     c->ploc_radius = 48;
     c->bvh_width = 4;
-    c->bvh_width_set = 0;
     c->bvh_rotations = 0;
     cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
     preload_trace_kernels();
@@ -299,7 +298,6 @@ extern "C" int dof_ctx_set_option(DofCtx *ctx, int option, int64_t value) {
         case DOF_OPT_BVH_WIDTH:
             if (value != 2 && value != 4) return dof_set_error(DOF_ERR_INVALID_ARG, "BVH width must be 2 or 4");
             ctx->bvh_width = (int)value;
-            ctx->bvh_width_set = 1;
             return DOF_OK;
         case DOF_OPT_TRACE_STEPS:
             if (value < 1 || value > 256) return dof_set_error(DOF_ERR_INVALID_ARG, "steps per round must be 1..256");
@@ -816,7 +814,6 @@ static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
     }
     const bool few = (wide_rays > 0.5 * rays && rays < 400e3) || (dense_rays > 0.5 * rays && rays < 300e3);
     if (ctx->trace_packets >= 0) A.packets = ctx->trace_packets;
-    else if (ctx->bvh_width_set) A.packets = 0;
     else A.packets = !few;
     choose_lens_cells(ctx->ray_order_grid, A);
 }
@@ -952,7 +949,7 @@ struct DofGraph {
     bool adaptive, wide;
     int trace_blocks, refill_idle, steps_per_round, stack_depth, packets, stats;
     int lens_grid;                // the context's lens-cell grid of that moment (0: chosen per session)
-    int packets_opt, width_set;   // ... and its choice of tracer
+    int packets_opt;              // ... and its choice of tracer (-1: open)
     int packet_need;              // stack entries of the captured packet tracer
     int gather_w, gather_h, main_form, recon_w, recon_h;
     int main_tile;                // the main filter's shared-memory bytes (0: through L1)
@@ -1006,7 +1003,6 @@ extern "C" int dof_graph_create(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n
     g->steps_per_round = A.steps_per_round;
     g->lens_grid = ctx->ray_order_grid;
     g->packets_opt = ctx->trace_packets;
-    g->width_set = ctx->bvh_width_set;
     g->packet_need = packet_capacity(A);
     g->packets = A.packets;
     g->stats = A.stats;
@@ -1070,7 +1066,7 @@ extern "C" int dof_graph_launch(DofGraph *g, const DofFrameReq *reqs, uint32_t n
     A.refill_idle = g->refill_idle;
     A.steps_per_round = g->steps_per_round;
     A.stack_depth = g->stack_depth;
-    if (ctx->trace_packets == g->packets_opt && ctx->bvh_width_set == g->width_set) A.packets = g->packets;
+    if (ctx->trace_packets == g->packets_opt) A.packets = g->packets;
     choose_lens_cells(g->lens_grid, A);
     // packets traverse the binary tree: whether there is a 4-wide one matters to one ray per lane
     const bool other_tree = !(A.packets && g->packets) && all_wide(A) != g->wide;

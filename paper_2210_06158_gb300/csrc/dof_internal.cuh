@@ -108,8 +108,7 @@ struct DofCtx {
     int recon_w, recon_h;                // reconstruction launch shape
     int stack_depth;                     // requested traversal stack entries (raised to the tree's need)
     int ploc_radius;
-    int bvh_width;                 // 4: traverse the collapsed 4-wide tree, 2: the binary tree
-    int bvh_width_set;             // the caller chose it (and with it one ray per lane, unless packets are set)
+    int bvh_width;                 // one ray per lane: 4 the collapsed 4-wide tree, 2 the binary tree
     // A frame's ray path (mask .. reconstruction) runs on ray_stream (highest priority)
     // while its post-process filters run on the caller's stream; ev_fork / ev_join order
     // them around the shared inputs (tiles) and the composite, ev_mask holds the filters back

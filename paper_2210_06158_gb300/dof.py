@@ -300,8 +300,8 @@ class Context:
         order it takes the rays in (lens-cell grid; 1 = pixel order), its traversal
         stack depth (raised to what the tree needs), whether a warp's rays traverse
         the binary tree as one packet, and whether that packet tracer counts node
-        visits and triangle tests for stats() -- no effect on results.  Until packets,
-        bvh_width or ray_grid is set the library chooses them."""
+        visits and triangle tests for stats() -- no effect on results.  Until packets or
+        ray_grid is set the library chooses it."""
         for opt, v in ((2, blocks_per_sm), (3, refill_idle), (4, steps), (6, bvh_width), (7, ray_grid), (11, stack),
                        (12, None if packets is None else int(bool(packets))),
                        (14, None if stats is None else int(bool(stats)))):

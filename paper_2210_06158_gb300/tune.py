@@ -162,7 +162,8 @@ SCENE_RADII = [8, 12, 16, 24, 32, 40, 48, 56, 64, 96, 128, 192]
 
 def tune_scene(ctx, host_scene, run_frame, radii=None, widths=(4, 2), frames=4, stream=None):
     """Build the scene's BVH with each PLOC search radius and time `frames` frames with
-    each tree width; keep the fastest.  run_frame(scene, k) enqueues frame k of a
+    each tree width (which counts where one ray per lane is traced: the context's choice of
+    tracer is left as it is); keep the fastest.  run_frame(scene, k) enqueues frame k of a
     representative session with the given device scene (the hits, hence the images,
     do not depend on the tree).  Returns (device scene, {"ploc_radius", "bvh_width"},
     {(radius, width): ms per frame}); the context keeps the chosen width."""
