@@ -190,7 +190,8 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
  * library takes the columns where the step has pixels enough for them, else form 0.  Same
  * results either way */
 #define DOF_OPT_MAIN_FILTER_FORM    9
-/* block of the reconstruction's 81-tap gather, encoded as DOF_OPT_GATHER_BLOCK (default 32 x 8) */
+/* block of the reconstruction's 81-tap gather, encoded as DOF_OPT_GATHER_BLOCK (default 32 x 8);
+ * sessions below 40,000 half-resolution pixels run in blocks of as many threads, 8 pixels wide */
 #define DOF_OPT_RECON_BLOCK         10
 /* entries of the tracer's per-ray traversal stack, 1..96 (default 96); the launch takes the
  * smallest compiled capacity (32, 64, 96) that holds both this and what the batch's trees

@@ -736,6 +736,9 @@ static int make_desc(DofCtx *ctx, const DofFrameReq &r, SessDesc &d) {
     return DOF_OK;
 }
 
+// half-resolution pixels below which a session's reconstruction takes four lanes per pixel
+constexpr int kReconSplitPx = 40000;
+
 static void shape_grid(const BatchArgs &A, const SessDesc &d, const DofHistory *h, int shape, int &gx, int &gy) {
     switch (shape) {
         case SH_GATHER: {
@@ -745,10 +748,16 @@ static void shape_grid(const BatchArgs &A, const SessDesc &d, const DofHistory *
             gy = ((int)h->H2 + rows - 1) / rows;
             break;
         }
-        case SH_RECON: {
-            const int w = d.recon_split ? A.recon_w / 4 : A.recon_w;
+        case SH_RECON:
+        case SH_RECON_SPLIT: {
+            const bool split = d.N < kReconSplitPx;
+            if (split != (shape == SH_RECON_SPLIT)) {
+                gx = gy = 0;
+                break;
+            }
+            const int w = split ? 8 : A.recon_w, rows = split ? A.recon_w * A.recon_h / 32 : A.recon_h;
             gx = ((int)h->W2 + w - 1) / w;
-            gy = ((int)h->H2 + A.recon_h - 1) / A.recon_h;
+            gy = ((int)h->H2 + rows - 1) / rows;
             break;
         }
         case SH_HPX: gx = ((int)h->W2 + 31) / 32; gy = ((int)h->H2 + 7) / 8; break;
@@ -775,9 +784,6 @@ static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint3
     A.main_form = px >= kColumnsMinPx ? 3 : 0;
     if (A.main_form == 3 && !ctx->gather_set) A.gather_h = 2;
 }
-
-// half-resolution pixels below which a session's reconstruction takes four lanes per pixel
-constexpr int kReconSplitPx = 40000;
 
 // Lens-cell grid of each session's rays, by the tracer of the step: the caller's (grid), or where that
 // is open (0) the one that choose_tracer's figures favour.
@@ -824,11 +830,8 @@ static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchAr
     memset(&A, 0, sizeof(A));
     A.ns = (int)n;
     choose_main_filter(ctx, reqs, n, A);
-    // split sessions need whole warps along x: a block of another width is taken as 32 wide
-    bool split = false;
-    for (uint32_t s = 0; s < n; s++) split |= reqs[s].hist && (int)reqs[s].hist->N < kReconSplitPx;
-    A.recon_w = split && ctx->recon_w % 32 ? 32 : ctx->recon_w;
-    A.recon_h = A.recon_w == ctx->recon_w ? ctx->recon_h : std::max(2, ctx->recon_w * ctx->recon_h / 32);
+    A.recon_w = ctx->recon_w;
+    A.recon_h = ctx->recon_h;
     adaptive = false;
     for (uint32_t s = 0; s < n; s++) {
         for (uint32_t t = 0; t < s; t++)
@@ -837,7 +840,6 @@ static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchAr
         int rc = make_desc(ctx, reqs[s], A.s[s]);
         if (rc) return rc;
         adaptive |= A.s[s].p.ray_mode == 1;
-        A.s[s].recon_split = A.s[s].N < kReconSplitPx;
         for (int sh = 0; sh < SH_COUNT; sh++) {
             int gx, gy;
             shape_grid(A, A.s[s], reqs[s].hist, sh, gx, gy);

@@ -13,7 +13,8 @@ enum LaunchShape {
     SH_FPX,         // 32x8 full-resolution pixels per block
     SH_SHADE,       // 128 queue entries per block
     SH_GATHER,      // the main filter's 81-tap gather: gather_w x gather_h hpx
-    SH_RECON,       // the reconstruction's 81-tap gather: recon_w x recon_h hpx
+    SH_RECON,       // the reconstruction's 81-tap gather: recon_w x recon_h hpx (no block of a small session)
+    SH_RECON_SPLIT, // ... of the small sessions alone: 8 hpx by one row per warp
     SH_COUNT
 };
 
@@ -26,7 +27,6 @@ struct SessDesc {
     int gx[SH_COUNT];              // blocks per row of each shape
     int N, max_rays, valid, record_rays;
     int lens_grid;                 // tracer work order: lens-cell grid of the mask kernel (1 = pixel order)
-    int recon_split;               // the reconstruction takes four lanes per pixel
     // frame inputs and output (caller-owned)
     const float4 *color;
     const float *depth;
@@ -62,7 +62,7 @@ struct BatchArgs {
     int stats;                     // 1: the packet tracer counts node visits and triangle tests
     int stack_depth;               // requested traversal stack entries (the launch takes an instance >= the need)
     int gather_w, gather_h;        // block of the main filter (SH_GATHER), <= 512 threads
-    int recon_w, recon_h;          // block of the reconstruction (SH_RECON), <= 512 threads
+    int recon_w, recon_h;          // block of the reconstruction (SH_RECON; SH_RECON_SPLIT as many threads), <= 512 threads
     int main_form;                 // main filter: 0 halo tile up to 64 KB, 1 through L1, 2 halo tile up
                                    // to the SM's opt-in shared memory, 3 columns of four pixels
     int start[SH_COUNT][kMaxBatch + 1];
@@ -92,7 +92,8 @@ inline bool any_taa(const BatchArgs &A) {
 }
 
 #ifdef __CUDACC__
-// session of a flat block index for `shape`; *local = the block's index in that session
+// session of a flat block index for `shape`; *local = the block's index in that session (the last
+// session that starts at or before the block: one without blocks of the shape is never found)
 __device__ __forceinline__ int find_session(const BatchArgs &A, int shape, int block, int &local) {
     int lo = 0, hi = A.ns;
     while (hi - lo > 1) {

@@ -281,21 +281,24 @@ __device__ __forceinline__ void recon_taps(const MipLevel &L0, const MipLevel &L
     }
 }
 
-// The reconstruction of a small session: four lanes of a warp take a run of a pixel's taps each
-// (lane & 7: the pixel, lane >> 3: the run, of 21, 20, 20 and 20 taps), and the runs' sums are
-// added in order.  One thread per pixel leaves most of the chip idle then, and the chain of its
-// 81 taps sets the time: 256 x 144 31 -> 17 us, 480 x 270 32 -> 27, 640 x 360 47 -> 41 but in a
-// batch that fills the chip it costs 10% (960 x 540 67 -> 74).  Which sessions take it depends on their own size
-// alone (SessDesc::recon_split), so that a session's bits do not depend on its batch.
+// A11 of the small sessions (below kReconSplitPx half-resolution pixels): four lanes of a warp take a
+// run of a pixel's taps each (lane & 7: the pixel, lane >> 3: the run, of 21, 20, 20 and 20 taps), and
+// the runs' sums are added in order.  One thread per pixel leaves most of the chip idle then, and
+// the chain of its 81 taps sets the time: 256 x 144 31 -> 17 us, 480 x 270 32 -> 27, 640 x 360 47 -> 41,
+// but where a session fills the chip it costs 10% (960 x 540 67 -> 74).  Which sessions take it depends
+// on their own size alone, so that a session's bits do not depend on its batch.
+//
+// A block covers 8 pixels by as many rows as it has warps, whatever its shape.  A kernel of its own:
+// beside the other form in one kernel it spilled at that form's 72 registers, and so did the
+// large sessions of a batch that held a small one.
 template <bool H>
-__device__ __forceinline__ void recon_split(const SessDesc &S, int bx, int by) {
+__device__ __forceinline__ void recon_split(const SessDesc &S, int bx, int by, int rows) {
     const DevParams &p = S.p;
     const int W2 = S.cam.W2, H2 = S.cam.H2, mL = S.mip_L;
     const int reach = (int)ceilf(p.rmax_hpx) + (2 << (mL - 1)) + 2;
     const int lane = (int)(threadIdx.x & 31u), run = lane >> 3;
-    const int i = bx + (int)(threadIdx.x >> 5) * 8 + (lane & 7), j = by + (int)threadIdx.y;
-    const bool interior = bx - reach >= 0 && by - reach >= 0 && bx + (int)blockDim.x / 4 + reach < W2 &&
-                          by + (int)blockDim.y + reach < H2;
+    const int i = bx + (lane & 7), j = by + (int)(threadIdx.x >> 5);
+    const bool interior = bx - reach >= 0 && by - reach >= 0 && bx + 8 + reach < W2 && by + rows + reach < H2;
     const bool in = i < W2 && j < H2;
     const size_t q = in ? (size_t)j * W2 + i : 0;
     float4 *out = S.recon;
@@ -337,28 +340,30 @@ __device__ __forceinline__ void recon_split(const SessDesc &S, int bx, int by) {
     st_img(out, q, make_float4(lerpf(o.x, f.x, b), lerpf(o.y, f.y, b), lerpf(o.z, f.z, b), lerpf(o.w, f.w, b)), H);
 }
 
+template <class AS, int kStore>
+__global__ void __launch_bounds__(512) k_recon_split(const __grid_constant__ AS as_) {
+    const BatchArgs &A = batch_args(as_);
+    int lb;
+    const SessDesc &S = A.s[find_session(A, SH_RECON_SPLIT, blockIdx.x, lb)];
+    const int gx = S.gx[SH_RECON_SPLIT], rows = (int)(blockDim.x >> 5);
+    const int bx = (lb % gx) * 8, by = (lb / gx) * rows;
+    if (kStore == 2 ? S.p.f16 != 0 : kStore == 1) recon_split<true>(S, bx, by, rows);
+    else recon_split<false>(S, bx, by, rows);
+}
+
 // A11: reconstruction.  Blocks whose footprint (+-rmax + 2, at every level) lies
 // inside the image take taps without index clamping.  kStore: the launch's image storage
 // (image_storage_mode); the specialised instances hold the code of one storage only, and
 // with it fewer registers.  72 registers hold either storage's taps without spilling
 // (three 256-thread blocks per SM; a cap of 64 spilled the FP32 form's state through
 // L1, the unit that bounds it, and was 1-2% slower).
-// kSplit: 0 no session of the launch is split (recon_split), 1 all are, 2 some are; the
-// unsplit instances stay free of the other form's registers.
-template <class AS, int kStore, int kSplit>
+template <class AS, int kStore>
 __global__ void __maxnreg__(72) k_recon(const __grid_constant__ AS as_) {
     const BatchArgs &A = batch_args(as_);
     int i, j;
     const SessDesc &S = block_session(A, SH_RECON, i, j);
     const DevParams &p = S.p;
     const bool f16 = kStore == 2 ? p.f16 != 0 : kStore == 1;
-    if (kSplit == 1 || (kSplit == 2 && S.recon_split)) {
-        const int bx = (i - (int)threadIdx.x) / 4, by = j - (int)threadIdx.y;    // its blocks are a quarter as wide
-        if (f16) recon_split<true>(S, bx, by);
-        else recon_split<false>(S, bx, by);
-        return;
-    }
-    if constexpr (kSplit != 1) {
     const int W2 = S.cam.W2, H2 = S.cam.H2;
     const int mL = S.mip_L;
     const float4 *__restrict__ med = S.rt_med;
@@ -399,7 +404,6 @@ __global__ void __maxnreg__(72) k_recon(const __grid_constant__ AS as_) {
     }
     float4 f = den > 0.f ? f4scale(1.f / den, num) : o;
     st_img(out, q, make_float4(lerpf(o.x, f.x, b), lerpf(o.y, f.y, b), lerpf(o.z, f.z, b), lerpf(o.w, f.w, b)), f16);
-    }
 }
 
 // A12: composite.  One thread per half-resolution pixel (i, j) writes its 2x2
@@ -579,42 +583,42 @@ void launch_recon_b(const BatchArgs &A, const AS &as, cudaStream_t st, DofHistor
     k_resolve_rt<AS><<<A.start[SH_HPX][n], b, 0, st>>>(as);
     tmark(tm, DOF_K_MEDIAN_RT, st);
     tmark(tm, DOF_K_MIPS, st);
-    const dim3 rg(A.start[SH_RECON][n]), rb(A.recon_w, A.recon_h);
-    int n_split = 0;
-    for (int k = 0; k < n; k++) n_split += A.s[k].recon_split != 0;
-    const int split = n_split == 0 ? 0 : (n_split == n ? 1 : 2);
-    const int mode = image_storage_mode(A);
-    if (mode == 2) k_recon<AS, 2, 2><<<rg, rb, 0, st>>>(as);
-    else if (mode == 1 && split == 0) k_recon<AS, 1, 0><<<rg, rb, 0, st>>>(as);
-    else if (mode == 1 && split == 1) k_recon<AS, 1, 1><<<rg, rb, 0, st>>>(as);
-    else if (mode == 1) k_recon<AS, 1, 2><<<rg, rb, 0, st>>>(as);
-    else if (split == 0) k_recon<AS, 0, 0><<<rg, rb, 0, st>>>(as);
-    else if (split == 1) k_recon<AS, 0, 1><<<rg, rb, 0, st>>>(as);
-    else k_recon<AS, 0, 2><<<rg, rb, 0, st>>>(as);
-    count_launches(2);
+    // the sessions on either side of kReconSplitPx, each in the kernel of its form
+    const int threads = A.recon_w * A.recon_h, mode = image_storage_mode(A);
+    const int blocks = A.start[SH_RECON][n], split = A.start[SH_RECON_SPLIT][n];
+    const dim3 rb(A.recon_w, A.recon_h);
+    if (mode == 0) {
+        if (blocks) k_recon<AS, 0><<<blocks, rb, 0, st>>>(as);
+        if (split) k_recon_split<AS, 0><<<split, threads, 0, st>>>(as);
+    } else if (mode == 1) {
+        if (blocks) k_recon<AS, 1><<<blocks, rb, 0, st>>>(as);
+        if (split) k_recon_split<AS, 1><<<split, threads, 0, st>>>(as);
+    } else {
+        if (blocks) k_recon<AS, 2><<<blocks, rb, 0, st>>>(as);
+        if (split) k_recon_split<AS, 2><<<split, threads, 0, st>>>(as);
+    }
+    count_launches(1 + (blocks > 0) + (split > 0));
     tmark(tm, DOF_K_RECON, st);
 }
 
+template <class AS, int kStore>
+static void preload_recon() {
+    cudaFuncAttributes a;
+    cudaFuncGetAttributes(&a, k_recon<AS, kStore>);
+    cudaFuncGetAttributes(&a, k_recon_split<AS, kStore>);
+}
 // the final TAA and the reconstruction's storage instances loaded now (a kernel first
 // launched in a later frame would otherwise stall that frame on its load)
 void preload_recon_kernels() {
     cudaFuncAttributes a;
     cudaFuncGetAttributes(&a, k_taa<BatchArgs>);
     cudaFuncGetAttributes(&a, k_taa<const BatchArgs *>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 0, 0>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 0, 1>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 0, 2>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 1, 0>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 1, 1>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 1, 2>);
-    cudaFuncGetAttributes(&a, k_recon<BatchArgs, 2, 2>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 0, 0>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 0, 1>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 0, 2>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 1, 0>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 1, 1>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 1, 2>);
-    cudaFuncGetAttributes(&a, k_recon<const BatchArgs *, 2, 2>);
+    preload_recon<BatchArgs, 0>();
+    preload_recon<BatchArgs, 1>();
+    preload_recon<BatchArgs, 2>();
+    preload_recon<const BatchArgs *, 0>();
+    preload_recon<const BatchArgs *, 1>();
+    preload_recon<const BatchArgs *, 2>();
     cudaGetLastError();
 }
 
