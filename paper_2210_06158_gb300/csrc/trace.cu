@@ -536,15 +536,15 @@ __global__ void __launch_bounds__(256) k_mask_compact(const __grid_constant__ AS
         b_ray = (uint32_t)(old >> 32);
     }
     __syncthreads();     // b_pix, b_ray and the warp offsets are read by every thread below
+    const uint32_t first = b_ray + w_ray[warp] + (uint32_t)(incl - n);
+    if (n > 0) {
+        queue[b_pix + w_pix[warp] + __popc(ball & ((1u << lane) - 1u))] = q;
+        first_ray[q] = first;
+    }
     const int grid = S.lens_grid;
     if (grid <= 1) {
         // pixel order: the work items follow the pixels' own slots
-        if (n > 0) {
-            queue[b_pix + w_pix[warp] + __popc(ball & ((1u << lane) - 1u))] = q;
-            const uint32_t f = b_ray + w_ray[warp] + (uint32_t)(incl - n);
-            first_ray[q] = f;
-            for (int s = 0; s < n; s++) ray_pix[f + s] = (q << 6) | (uint32_t)s;
-        }
+        for (int s = 0; s < n; s++) ray_pix[first + s] = (q << 6) | (uint32_t)s;
         return;
     }
     // lens cells of the block's rays (Morton indices below the power-of-two square that
@@ -554,7 +554,6 @@ __global__ void __launch_bounds__(256) k_mask_compact(const __grid_constant__ AS
     const int tid = (int)(warp * 32u + lane);
     cell_n[tid] = 0u;                       // 256 threads, 256 cells
     __syncthreads();
-    const uint32_t first = b_ray + w_ray[warp] + (uint32_t)(incl - n);
     for (int s = 0; s < n; s++) {
         // kept in the ray's slot for the tracer, which would otherwise draw it again
         const float2 u = lens_draw(S.cam, p, q, s);
@@ -579,13 +578,9 @@ __global__ void __launch_bounds__(256) k_mask_compact(const __grid_constant__ AS
         for (int k = 0; k < 8; k++) cell_at[lane * 8 + k] = base + v[k];
     }
     __syncthreads();
-    if (n > 0) {
-        queue[b_pix + w_pix[warp] + __popc(ball & ((1u << lane) - 1u))] = q;
-        first_ray[q] = first;
-        for (int s = 0; s < n; s++) {
-            const uint32_t at = atomicAdd(&cell_at[cell_of[s][tid]], 1u);
-            ray_pix[b_ray + at] = (q << 6) | (uint32_t)s;
-        }
+    for (int s = 0; s < n; s++) {
+        const uint32_t at = atomicAdd(&cell_at[cell_of[s][tid]], 1u);
+        ray_pix[b_ray + at] = (q << 6) | (uint32_t)s;
     }
 }
 
