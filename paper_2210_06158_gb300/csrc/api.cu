@@ -240,6 +240,13 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
     preload_trace_kernels();
     preload_post_kernels();
     preload_recon_kernels();
+    if (cudaMalloc(&c->d_status, sizeof(uint32_t)) != cudaSuccess ||
+        cudaMemset(c->d_status, 0, sizeof(uint32_t)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(c->d_status);
+        delete c;
+        return dof_set_error(DOF_ERR_OOM, "dof_ctx_create: status word");
+    }
     int prio_least = 0, prio_greatest = 0;
     cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
     if (cudaStreamCreateWithPriority(&c->ray_stream, cudaStreamNonBlocking, prio_greatest) != cudaSuccess ||
@@ -250,6 +257,7 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
         if (c->ray_stream) cudaStreamDestroy(c->ray_stream);
         if (c->ev_fork) cudaEventDestroy(c->ev_fork);
         if (c->ev_mask) cudaEventDestroy(c->ev_mask);
+        cudaFree(c->d_status);
         delete c;
         return dof_set_error(DOF_ERR_CUDA, "dof_ctx_create: stream or events");
     }
@@ -268,6 +276,7 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
         }
     }
     if (post_init_tables() != 0 || recon_init_tables() != 0) {
+        cudaFree(c->d_status);
         delete c;
         return dof_set_error(DOF_ERR_CUDA, "dof_ctx_create: uploading filter tables failed");
     }
@@ -359,6 +368,7 @@ void ctx_release(DofCtx *ctx) {
         cudaEventDestroy(ctx->ev_mask);
         cudaEventDestroy(ctx->ev_join);
         if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+        cudaFree(ctx->d_status);
         delete ctx;
     }
 }
@@ -491,7 +501,7 @@ extern "C" int dof_gbuffer(DofCtx *ctx, const DofScene *scene, const DofCamera *
     if (rc) return rc;
     cudaGetLastError();   // drop a stale error of an earlier call of another library on this thread
     launch_primary(dc, dp, scene_dev(scene), reinterpret_cast<float4 *>(color), depth,
-                   reinterpret_cast<float4 *>(normal), prim, (cudaStream_t)stream);
+                   reinterpret_cast<float4 *>(normal), prim, ctx->d_status, (cudaStream_t)stream);
     return dof_cuda_check(cudaGetLastError(), "dof_gbuffer launch");
 }
 

@@ -109,6 +109,7 @@ struct DofCtx {
     int stack_depth;                     // requested traversal stack entries (raised to the tree's need)
     int ploc_radius;
     int bvh_width;                 // one ray per lane: 4 the collapsed 4-wide tree, 2 the binary tree
+    uint32_t *d_status;            // device status word of context-level launches
     // A frame's ray path (mask .. reconstruction) runs on ray_stream (highest priority)
     // while its post-process filters run on the caller's stream; ev_fork / ev_join order
     // them around the shared inputs (tiles) and the composite, ev_mask holds the filters back
@@ -210,7 +211,7 @@ void dof_free(DofCtx *ctx, void *ptr, size_t bytes);
 // xyz, idx, mat: host arrays
 int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint32_t *idx, const uint32_t *mat, int builder, int ploc_radius, int rotations, cudaStream_t st);
 void launch_primary(const DevCam &cam, const DevParams &p, const SceneDev &sc, float4 *color, float *depth, float4 *normal,
-                    int32_t *prim, cudaStream_t st);
+                    int32_t *prim, uint32_t *status, cudaStream_t st);
 // host-side tally of this library's kernel launches (dof_launch_count); each launch
 // wrapper adds the launches it enqueued
 void count_launches(long long n);

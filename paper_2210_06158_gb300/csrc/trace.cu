@@ -331,17 +331,64 @@ __device__ __forceinline__ void packet_traverse(const SceneDev &sc, const Ray &r
     }
 }
 
+// One ray's traversal, of the 4-wide tree where the scene has one (else the binary one): closest
+// hit = lexicographic min of (t, prim id); boxes with entry == best are kept.  A reference outside
+// the tree, a full stack or more steps than a valid tree can take set the status word and end
+// the query (no fault, no endless loop).
+__device__ __forceinline__ HitRec closest_hit(const SceneDev &sc, const Ray &r, uint32_t *status) {
+    HitRec h{INFINITY, -1, -1};
+    uint32_t nv = 0, nt = 0;
+    // large triangles first: their hits bound the tree traversal
+    for (int k = sc.n_tris; k < sc.n_tris + sc.n_large; k++) tri_update(r, sc.tris, k, h);
+    if (sc.n_tris <= 0) return h;
+    int stack[kStack];
+    int sp = 0, node = sc.nodes4 ? sc.root4 : sc.root;
+    const long long most = 4ll * sc.n_tris + 64;
+    for (long long steps = 0;; steps++) {
+        if (steps > most) {
+            atomicOr(status, 2u);
+            break;
+        }
+        if (sc.nodes4 ? step4<kStack>(r, sc.nodes4, sc.n_nodes4, sc.tris, sc.n_tris, node, stack, sp, h, nv, nt, status)
+                      : step2<kStack>(r, sc.nodes, sc.n_tris - 1, sc.tris, sc.n_tris, node, stack, sp, h, nv, nt, status))
+            break;
+    }
+    return h;
+}
+
 // ---------------------------------------------------------------------------
 // A0: G-buffer producer
 // ---------------------------------------------------------------------------
+struct PrimaryOut {
+    float4 *color;
+    float *depth;
+    float4 *normal;
+    int32_t *prim;
+};
+__device__ __forceinline__ void store_primary(const DevCam &cam, const DevParams &p, const SceneDev &sc, const PrimaryOut &o,
+                                              size_t q, float3 d, const HitRec &h) {
+    if (o.prim) o.prim[q] = h.prim;
+    if (h.prim < 0) {
+        o.color[q] = make_float4(p.sky.x, p.sky.y, p.sky.z, 1.f);
+        o.depth[q] = INFINITY;
+        o.normal[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
+    }
+    float3 n;
+    const float3 col = shade(p, sc, h, d, n);
+    o.color[q] = make_float4(col.x, col.y, col.z, 1.f);
+    o.depth[q] = h.t * dot(d, cam.F);
+    o.normal[q] = make_float4(n.x, n.y, n.z, 0.f);
+}
+
 // One pinhole ray per pixel; a warp's rays, an 8 x 4 pixel tile, go through the tree as one
-// packet.  They leave one point through neighbouring pixels, so the packet visits little more
-// than each ray alone would and every lane steps with it.  One ray per lane spent its time in
-// divergent steps: 0.598 -> 0.273 ms at 1080p with 496k triangles.
+// packet.  They leave one point through neighbouring pixels, so in an image of many pixels the
+// packet visits little more than each ray alone would and every lane steps with it.  One ray per
+// lane spent its time in divergent steps: 0.598 -> 0.273 ms at 1080p with 496k triangles.
 constexpr int kPrimaryThreads = 128;     // 16 x 8 pixels
 __global__ void __launch_bounds__(kPrimaryThreads, 8) k_primary(const __grid_constant__ DevCam cam, const __grid_constant__ DevParams p,
-                                                                const __grid_constant__ SceneDev sc, float4 *color, float *depth,
-                                                                float4 *normal, int32_t *prim) {
+                                                                const __grid_constant__ SceneDev sc,
+                                                                const __grid_constant__ PrimaryOut o) {
     __shared__ int stacks[kPrimaryThreads / 32][kStack];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7), j = blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
@@ -356,20 +403,18 @@ __global__ void __launch_bounds__(kPrimaryThreads, 8) k_primary(const __grid_con
     if (sc.n_tris > 0)
         packet_traverse<false>(sc, r, make_slab_ray(r), (unsigned)__shfl_sync(0xffffffffu, r.oct, 0) & 7u, act,
                                act ? h.t : -1.f, stacks[warp], h, nv, nt);
-    if (!act) return;
-    const size_t q = (size_t)j * cam.W + i;
-    if (prim) prim[q] = h.prim;
-    if (h.prim < 0) {
-        color[q] = make_float4(p.sky.x, p.sky.y, p.sky.z, 1.f);
-        depth[q] = INFINITY;
-        normal[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        return;
-    }
-    float3 n;
-    float3 col = shade(p, sc, h, d, n);
-    color[q] = make_float4(col.x, col.y, col.z, 1.f);
-    depth[q] = h.t * dot(d, cam.F);
-    normal[q] = make_float4(n.x, n.y, n.z, 0.f);
+    if (act) store_primary(cam, p, sc, o, (size_t)j * cam.W + i, d, h);
+}
+
+// The same image by one ray per lane, for few pixels in a dense scene (few_primary).
+__global__ void __launch_bounds__(kPrimaryThreads) k_primary_lanes(const __grid_constant__ DevCam cam,
+                                                                   const __grid_constant__ DevParams p,
+                                                                   const __grid_constant__ SceneDev sc,
+                                                                   const __grid_constant__ PrimaryOut o, uint32_t *status) {
+    const int i = blockIdx.x * 16 + (threadIdx.x & 15), j = blockIdx.y * 8 + (threadIdx.x >> 4);
+    if (i >= cam.W || j >= cam.H) return;
+    const float3 d = pixel_dir(cam, i + 0.5f, j + 0.5f);
+    store_primary(cam, p, sc, o, (size_t)j * cam.W + i, d, closest_hit(sc, make_ray(cam.O, d), status));
 }
 
 // ---------------------------------------------------------------------------
@@ -948,10 +993,24 @@ __global__ void __launch_bounds__(128) k_shade(const __grid_constant__ AS as_) {
 
 }  // namespace
 
+// Few pixels in a dense scene take one ray per lane: their packets span wide angles, visit the union
+// of what the rays need, and the longest one sets the time.  Line: four pixels per triangle, and
+// 180,000 pixels.  Measured (us, packets / one ray per lane; lawn of that many triangles): 2.8k
+// 64 x 36 51 / 47, 160 x 90 36 / 44; 10k 160 x 90 65 / 54, 400 x 224 51 / 59; 30k 320 x 180 67 / 63,
+// 480 x 270 59 / 70; 60k 480 x 270 79 / 77, 640 x 360 71 / 83; 250k 64 x 36 165 / 57, 560 x 316 98 / 90,
+// 640 x 360 92 / 102; 500k 320 x 180 128 / 82, 560 x 316 114 / 98, 640 x 360 106 / 119; 1M through the
+// 85 mm lens 560 x 316 131 / 96, 640 x 360 113 / 109, 800 x 450 125 / 138.
+static bool few_primary(const DevCam &cam, const SceneDev &sc) {
+    const long long px = (long long)cam.W * cam.H;
+    return px < 180000 && px < 4ll * sc.n_tris;
+}
+
 void launch_primary(const DevCam &cam, const DevParams &p, const SceneDev &sc, float4 *color, float *depth, float4 *normal,
-                    int32_t *prim, cudaStream_t st) {
+                    int32_t *prim, uint32_t *status, cudaStream_t st) {
     const dim3 g((cam.W + 15) / 16, (cam.H + 7) / 8);
-    k_primary<<<g, kPrimaryThreads, 0, st>>>(cam, p, sc, color, depth, normal, prim);
+    const PrimaryOut o{color, depth, normal, prim};
+    if (few_primary(cam, sc)) k_primary_lanes<<<g, kPrimaryThreads, 0, st>>>(cam, p, sc, o, status);
+    else k_primary<<<g, kPrimaryThreads, 0, st>>>(cam, p, sc, o);
     count_launches(1);
 }
 
