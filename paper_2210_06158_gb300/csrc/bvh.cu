@@ -1493,16 +1493,16 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(const unsigned long
     }
 }
 
-// Stable sort of (keys, vals) by bits [from, to) of the keys (a multiple of 16 of them: an even
+// Stable sort of (keys, vals) by the key's low `bits` bits (a multiple of 16: an even
 // number of 8-bit passes); the result ends in (keys, vals), (keys2, vals2) and hist are
 // scratch (hist: 256 * ceil(n / 2048) ints, sums: ceil(256 * ceil(n / 2048) / 2048) ints).
 void device_radix_sort_pairs(unsigned long long *keys, uint32_t *vals, unsigned long long *keys2, uint32_t *vals2,
-                             int n, int *hist, int *sums, cudaStream_t st, int from = 0, int to = 64) {
+                             int n, int *hist, int *sums, cudaStream_t st, int bits = 64) {
     if (n <= 1) return;
     const int nb = (n + kSortTile - 1) / kSortTile;
     unsigned long long *ki = keys, *ko = keys2;
     uint32_t *vi = vals, *vo = vals2;
-    for (int shift = from; shift < to; shift += 8) {
+    for (int shift = 0; shift < bits; shift += 8) {
         k_rs_hist<<<nb, kSortThreads, 0, st>>>(ki, n, shift, hist, nb);
         device_exclusive_scan(hist, hist, kSortBins * nb, sums, st);
         k_rs_scatter<<<nb, kSortThreads, 0, st>>>(ki, vi, ko, vo, n, shift, hist, nb);
@@ -1523,7 +1523,7 @@ size_t sort_pairs_scratch_ints(int n) {
 void sort_pairs_by_low_bits(unsigned long long *keys, uint32_t *vals, unsigned long long *keys2, uint32_t *vals2,
                             int n, int bits, int *scratch, cudaStream_t st) {
     const size_t nh = (size_t)kSortBins * ((n + kSortTile - 1) / kSortTile);
-    device_radix_sort_pairs(keys, vals, keys2, vals2, n, scratch, scratch + nh, st, 0, bits);
+    device_radix_sort_pairs(keys, vals, keys2, vals2, n, scratch, scratch + nh, st, bits);
 }
 
 static inline unsigned blocks_for(size_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -1706,9 +1706,10 @@ int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint
         n_small = n - n_big;
         k_morton<<<blocks_for(n, B), B, 0, st>>>(b.cen, (uint32_t)n, separate ? b.ibuf + 9 : b.ibuf, b.ibuf, share, separate,
                                                  b.keys, b.vals);
-        // the radix tree needs the whole key; the clustering round only looks at neighbours, and the
-        // upper 32 bits (a 1/1000 of the extent per axis) leave its trees as they are
-        device_radix_sort_pairs(b.keys, b.vals, b.keys2, b.vals2, n, b.hist, b.sums, st, ploc ? 32 : 0, 64);
+        // by the whole key: with its upper half alone (10 bits per axis) the clusters of a scene whose
+        // detail lies in a small part of its extent follow the order of the input, and a packet of a
+        // lawn beside one far triangle visits 120 nodes instead of 58 (7% less of the upload's time)
+        device_radix_sort_pairs(b.keys, b.vals, b.keys2, b.vals2, n, b.hist, b.sums, st);
         // sorted (key, triangle) pairs are in (keys, vals)
         k_sorted_tris<<<blocks_for(n, B), B, 0, st>>>(d_xyz, d_idx, d_mat, (uint32_t)n, n_verts, b.vals, s->tris);
         const int m = n_small;
