@@ -405,16 +405,16 @@ extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts,
     int rc = DOF_OK;
     if (n_tris == 0) { s->depth = 0; s->root = ~0; ctx_retain(ctx); *out = s; return DOF_OK; }
     {
-        // one allocation for what every tree has (an allocation or a release costs the host 50 us)
-        auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-        const size_t tris = up(sizeof(float4) * 3 * (size_t)n_tris), nodes = up(sizeof(BvhNode) * (size_t)s->n_nodes);
-        s->base_bytes = tris + nodes + 4 * (size_t)n_tris;
+        // one allocation for what every tree has (an allocation or a release costs the host 50 us),
+        // in an order that leaves each piece aligned without padding
+        const size_t nodes = sizeof(BvhNode) * (size_t)s->n_nodes, tris = sizeof(float4) * 3 * (size_t)n_tris;
+        s->base_bytes = nodes + tris + 4 * (size_t)n_tris;
         rc = dof_alloc(ctx, s->base_bytes, &s->base, &s->bytes);
         if (rc == DOF_OK) {
             char *p = static_cast<char *>(s->base);
-            s->tris = reinterpret_cast<float4 *>(p);
-            s->nodes = s->n_nodes ? reinterpret_cast<BvhNode *>(p + tris) : nullptr;
-            s->prim_k = reinterpret_cast<int32_t *>(p + tris + nodes);
+            s->nodes = s->n_nodes ? reinterpret_cast<BvhNode *>(p) : nullptr;
+            s->tris = reinterpret_cast<float4 *>(p + nodes);
+            s->prim_k = reinterpret_cast<int32_t *>(p + nodes + tris);
         }
     }
     if (rc == DOF_OK) rc = launch_bvh_build(s, xyz, n_verts, tri_idx, tri_mat, ctx->bvh_builder, ctx->ploc_radius, ctx->bvh_rotations, st);

@@ -34,3 +34,22 @@ def test_a_budget_without_room_for_the_wide_tree_leaves_no_error_behind():
     x = torch.ones(1000, device="cuda") * 2         # a launch whose error check is torch's
     torch.cuda.synchronize()
     assert float(x.sum()) == 2000.0
+
+
+@pytest.mark.parametrize("n", [1, 2, 37, 5001])
+def test_a_scene_takes_what_its_parts_take(n):
+    """48 bytes per triangle and 4 for its index, 64 per binary node, 128 per 4-wide node, nothing for
+    padding: a budget of just that admits it, a byte less does not."""
+    from paper_2210_06158_gb300 import dof
+    ctx = dof.Context(0)
+    i = dof.Scene(ctx, _scene(n)).info()
+    total = 52 * n + 64 * (n - 1) + 128 * i.n_nodes4
+    assert i.device_bytes == total
+    exact = dof.Context(0, mem_budget_bytes=total)
+    sc = dof.Scene(exact, _scene(n))
+    assert exact.bytes_in_use == total
+    sc.close()
+    assert exact.bytes_in_use == 0
+    with pytest.raises(dof.DofError) as e:
+        dof.Scene(dof.Context(0, mem_budget_bytes=total - 1), _scene(n))
+    assert e.value.code == -3
