@@ -154,11 +154,14 @@ typedef struct {
 
 /* Create a context on CUDA device `device`.  mem_budget_bytes (0 = unlimited) caps
  * the device memory that scenes and histories of this context may hold; an upload or
- * history that would exceed it fails with DOF_ERR_BUDGET.  Owns nothing of the
- * caller's. */
+ * history that would exceed it fails with DOF_ERR_BUDGET.  Between calls the context also
+ * keeps scratch of uploads and of dof_gbuffer_raster in a pool of its own: after an upload at
+ * most 768 MB, and no more than the budget leaves beside the scenes and histories.  It
+ * is given back when an allocation of the context finds no memory, and with the context.
+ * Owns nothing of the caller's. */
 int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out);
 void dof_ctx_destroy(DofCtx *ctx);
-/* bytes currently held by the context's scenes and histories */
+/* bytes currently held by the context's scenes and histories (without the kept scratch) */
 size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
 
 /* Context options (dof_ctx_set_option). */
@@ -260,8 +263,8 @@ int dof_gbuffer(DofCtx *ctx, const DofScene *scene, const DofCamera *cam, const 
  * centres that can see it), the pixels of that conservative region run the same
  * watertight ray/triangle test, and the closest hit per pixel is kept by a 64-bit
  * atomic minimum of (distance bits, triangle id), then shaded.  Scratch (8 bytes per
- * pixel plus 68 bytes per triangle) comes from a stream-ordered pool that the context
- * keeps until it is destroyed; the call does not synchronise `stream`. */
+ * pixel plus ~112 bytes per triangle) comes from the context's stream-ordered pool
+ * (dof_ctx_create); the call does not synchronise `stream`. */
 int dof_gbuffer_raster(DofCtx *ctx, const DofScene *scene, const DofCamera *cam, const DofParams *p,
                        uint32_t width, uint32_t height, float *color, float *depth, float *normal,
                        int32_t *prim, void *stream);

@@ -38,25 +38,48 @@ int dof_cuda_check(cudaError_t e, const char *what) {
     return dof_set_error(code, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// Scratch that the pool keeps between calls: at most that of an upload of 2M triangles (growing and
+// trimming it costs such an upload 0.7 of 5 ms), and no more than the context's budget leaves
+// beside its scenes and histories.  All of it goes back to the device when an allocation fails.
+constexpr size_t kPoolKeep = (size_t)768 << 20;
+static void trim_pool(DofCtx *ctx) {
+    if (!ctx->pool) return;
+    const size_t used = ctx->in_use, left = !ctx->budget ? kPoolKeep : (ctx->budget > used ? ctx->budget - used : 0);
+    cudaMemPoolTrimTo(ctx->pool, std::min(kPoolKeep, left));
+}
+
+// runs `get` again, once the pool's unused scratch is back on the device, when it finds no memory
+template <class F>
+static cudaError_t with_pool_given_back(DofCtx *ctx, F get) {
+    cudaError_t e = get();
+    if (e == cudaErrorMemoryAllocation && ctx->pool) {
+        cudaGetLastError();
+        cudaMemPoolTrimTo(ctx->pool, 0);
+        e = get();
+    }
+    return e;
+}
+
+int dof_scratch(DofCtx *ctx, size_t bytes, void **ptr, cudaStream_t st, const char *what) {
+    return dof_cuda_check(with_pool_given_back(ctx, [&] {
+        return ctx->pool ? cudaMallocFromPoolAsync(ptr, bytes, ctx->pool, st) : cudaMallocAsync(ptr, bytes, st);
+    }), what);
+}
+
 int dof_alloc(DofCtx *ctx, size_t bytes, void **ptr, size_t *acc) {
     *ptr = nullptr;
     if (bytes == 0) return DOF_OK;
     if (ctx->budget && ctx->in_use + bytes > ctx->budget)
         return dof_set_error(DOF_ERR_BUDGET, "allocation of %zu bytes exceeds the budget (%zu of %zu in use)", bytes,
                              (size_t)ctx->in_use, ctx->budget);
-    cudaError_t e = cudaMalloc(ptr, bytes);
-    if (e == cudaErrorMemoryAllocation && ctx->pool) {
-        // the scratch that the pool keeps between calls goes back to the device first
-        cudaGetLastError();
-        cudaMemPoolTrimTo(ctx->pool, 0);
-        e = cudaMalloc(ptr, bytes);
-    }
+    cudaError_t e = with_pool_given_back(ctx, [&] { return cudaMalloc(ptr, bytes); });
     if (e != cudaSuccess) {
         *ptr = nullptr;
         return dof_cuda_check(e, "cudaMalloc");
     }
     ctx->in_use += bytes;
     if (acc) *acc += bytes;
+    if (ctx->budget) trim_pool(ctx);
     return DOF_OK;
 }
 
@@ -262,7 +285,7 @@ extern "C" int dof_ctx_create(int device, size_t mem_budget_bytes, DofCtx **out)
         return dof_set_error(DOF_ERR_CUDA, "dof_ctx_create: stream or events");
     }
     {
-        // scratch of dof_gbuffer_raster: kept in the pool between calls
+        // scratch of uploads and of dof_gbuffer_raster: kept in the pool between calls (trim_pool)
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -385,10 +408,6 @@ extern "C" size_t dof_ctx_bytes_in_use(const DofCtx *ctx) { return ctx ? (size_t
 // scene
 // ---------------------------------------------------------------------------
 
-// what the scratch pool keeps after an upload: the scratch of 2M triangles (growing and trimming it
-// costs such an upload 0.7 of 5 ms); given back to the device when an allocation fails
-constexpr size_t kPoolKeep = (size_t)768 << 20;
-
 extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts, const uint32_t *tri_idx,
                                 const uint32_t *tri_mat, uint32_t n_tris, void *stream, DofScene **out) {
     if (!ctx || !out || (n_tris && (!xyz || !tri_idx || !n_verts)))
@@ -422,11 +441,12 @@ extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts,
         launch_prim_index(s->tris, (int)n_tris, s->prim_k, st);
         rc = dof_cuda_check(cudaStreamSynchronize(st), "scene triangle index");
     }
-    // the pool keeps at most kPoolKeep of the build's scratch for the next call
-    if (ctx->pool) cudaMemPoolTrimTo(ctx->pool, kPoolKeep);
     if (rc != DOF_OK) {
         dof_free(ctx, s->base, s->base_bytes);
         dof_free(ctx, s->nodes4, s->nodes4_bytes);
+    }
+    trim_pool(ctx);
+    if (rc != DOF_OK) {
         delete s;
         return rc;
     }
@@ -527,7 +547,7 @@ extern "C" int dof_gbuffer_raster(DofCtx *ctx, const DofScene *scene, const DofC
     const SceneDev sd = scene_dev(scene);
     const size_t bytes = raster_scratch_bytes((int)width, (int)height, (int)scene->n_tris);
     void *scratch = nullptr;
-    rc = dof_cuda_check(cudaMallocFromPoolAsync(&scratch, bytes, ctx->pool, st), "dof_gbuffer_raster scratch");
+    rc = dof_scratch(ctx, bytes, &scratch, st, "dof_gbuffer_raster scratch");
     if (rc) return rc;
     cudaError_t e = launch_raster(dc, dp, sd, scene->prim_k, scratch, ctx->sm_count, reinterpret_cast<float4 *>(color),
                                   depth, reinterpret_cast<float4 *>(normal), prim, st);
@@ -1028,7 +1048,7 @@ extern "C" int dof_graph_create(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n
     cudaStream_t cs = nullptr;
     cudaGraph_t graph = nullptr;
     auto ck = [&](cudaError_t e, const char *w) { if (rc == DOF_OK && e != cudaSuccess) rc = dof_cuda_check(e, w); };
-    ck(cudaMalloc(&g->d_args, sizeof(BatchArgs)), "dof_graph_create: device arguments");
+    ck(with_pool_given_back(ctx, [&] { return cudaMalloc(&g->d_args, sizeof(BatchArgs)); }), "dof_graph_create: device arguments");
     ck(cudaHostAlloc(&g->h_stage, sizeof(BatchArgs), cudaHostAllocDefault), "dof_graph_create: staging");
     ck(cudaEventCreateWithFlags(&g->staged, cudaEventDisableTiming), "dof_graph_create: event");
     ck(cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming), "dof_graph_create: event");

@@ -1675,8 +1675,7 @@ int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint
     b.lay_out(arena, n, ploc);
     float *d_xyz = arena.take<float>(3 * (size_t)n_verts);
     uint32_t *d_idx = arena.take<uint32_t>(3 * (size_t)n), *d_mat = mat ? arena.take<uint32_t>(n) : nullptr;
-    if (s->ctx->pool) ck(cudaMallocFromPoolAsync((void **)&arena.base, arena.used, s->ctx->pool, st), "bvh scratch");
-    else ck(cudaMallocAsync((void **)&arena.base, arena.used, st), "bvh scratch");
+    rc = dof_scratch(s->ctx, arena.used, (void **)&arena.base, st, "bvh scratch");
     if (rc != DOF_OK) return rc;
     arena.used = 0;
     b.lay_out(arena, n, ploc);

@@ -117,7 +117,7 @@ struct DofCtx {
     cudaStream_t ray_stream;
     cudaEvent_t ev_fork, ev_mask, ev_join;
     std::mutex launch_mu;          // one frame's enqueue at a time on ray_stream
-    cudaMemPool_t pool;            // stream-ordered scratch of the rasterising G-buffer producer
+    cudaMemPool_t pool;            // stream-ordered scratch of uploads and of the rasterising G-buffer producer
 };
 
 struct DofScene {
@@ -206,6 +206,8 @@ int dof_alloc(DofCtx *ctx, size_t bytes, void **ptr, size_t *acc);
 void ctx_retain(DofCtx *ctx);
 void ctx_release(DofCtx *ctx);   // frees the context with its last reference
 void dof_free(DofCtx *ctx, void *ptr, size_t bytes);
+// stream-ordered scratch, outside the budget (cudaFreeAsync gives it back to the context's pool)
+int dof_scratch(DofCtx *ctx, size_t bytes, void **ptr, cudaStream_t st, const char *what);
 
 // launch wrappers (one per kernel group, defined in the .cu files)
 // xyz, idx, mat: host arrays

@@ -53,3 +53,33 @@ def test_a_scene_takes_what_its_parts_take(n):
     with pytest.raises(dof.DofError) as e:
         dof.Scene(dof.Context(0, mem_budget_bytes=total - 1), _scene(n))
     assert e.value.code == -3
+
+
+def test_kept_scratch_stays_within_what_the_budget_leaves():
+    """The upload's scratch (over 300 MB here) is kept for the next one only as far as the budget has
+    room beside the scene, and a history that takes the room takes it from the kept scratch."""
+    import torch
+    from paper_2210_06158_gb300 import dof
+    host = _scene(1_000_000)
+    first = dof.Context(0)
+    sc = dof.Scene(first, host)
+    total = first.bytes_in_use
+    sc.close()
+    first.close()
+    room = 32 << 20
+    ctx = dof.Context(0, mem_budget_bytes=total + room)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+
+    def kept():
+        torch.cuda.synchronize()
+        return free - torch.cuda.mem_get_info()[0] - ctx.bytes_in_use
+
+    sc = dof.Scene(ctx, host)
+    assert kept() <= room + (8 << 20)                  # the allocator rounds up to pages of 2 MB
+    hist = dof.History(ctx, 640, 360)
+    # the history's some forty buffers are each rounded up to pages
+    assert kept() <= total + room - ctx.bytes_in_use + (88 << 20)
+    hist.close()
+    sc.close()
+    assert ctx.bytes_in_use == 0
