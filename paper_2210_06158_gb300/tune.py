@@ -108,6 +108,8 @@ GATHER_SPACE = {
     "main_form": [0, 1, 2, 3],
     "recon_block": [(32, 8), (16, 16), (64, 4), (32, 4), (16, 8), (32, 16), (64, 8)],
 }
+# 32 x 8 pixels in columns of four, what the library itself takes for them; tried once the columns lead
+COLUMN_BLOCKS = [(32, 2)]
 GATHER_DEFAULT = {"gather_block": (32, 8), "main_form": 0, "recon_block": (32, 8)}
 
 
@@ -115,8 +117,8 @@ def tune_gathers(ctx, run_frame, frames=4, rounds=2, stream=None):
     """The 81-tap gathers' launch shapes (block of the main filter, block of the
     reconstruction) and the main filter's form (halo tile in shared memory up to 64 KB,
     through L1, halo tile up to the SM's opt-in shared memory, or columns of four pixels
-    through L1): coordinate descent
-    over GATHER_SPACE from GATHER_DEFAULT with the same timing rules as tune_trace.
+    through L1): coordinate descent over GATHER_SPACE (and COLUMN_BLOCKS while the columns
+    lead) from GATHER_DEFAULT with the same timing rules as tune_trace.
     Returns (best settings, {settings tuple: ms per frame}); the context keeps the best."""
     import torch
     st = stream if stream is not None else torch.cuda.current_stream()
@@ -139,6 +141,8 @@ def tune_gathers(ctx, run_frame, frames=4, rounds=2, stream=None):
     for _ in range(rounds):
         improved = False
         for name, values in GATHER_SPACE.items():
+            if name == "gather_block" and best["main_form"] == 3:
+                values = values + COLUMN_BLOCKS
             for v in values:
                 cand = dict(best, **{name: v})
                 ms = measure(cand)
