@@ -24,7 +24,7 @@ def _run(monkeypatch, cost):
             return end.t - self.t
 
     monkeypatch.setattr(torch.cuda, "Event", Event)
-    cfg, tried = {}, []
+    cfg, tried = dict(block=(32, 8), form=0), []        # as the warm-up frames find the context
 
     def set_gather(block, main_form, recon_block):
         cfg.update(block=tuple(block), form=main_form)
