@@ -820,16 +820,17 @@ static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint3
 static void choose_lens_cells(int grid, BatchArgs &A) {
     for (int s = 0; s < A.ns; s++) {
         const float k = A.s[s].cam.cocK;
-        A.s[s].lens_grid = grid ? grid : (A.packets ? (k >= 11.f ? 8 : 1) : (k >= 6.f ? 4 : 1));
+        A.s[s].lens_grid = grid ? grid : (A.packets ? (k >= 10.f ? 8 : 1) : (k >= 6.f ? 4 : 1));
     }
 }
 
 // The tracer of a step whose context leaves it open: warp packets, taken in pixel order, but
 // by lens cells of 1/8 aperture where the blur of the far field (cocK, its asymptotic
-// diameter) spans 11 px and more, so that a packet's rays leave one patch of the lens.  One ray
+// diameter) spans 10 px and more, so that a packet's rays leave one patch of the lens.  One ray
 // per lane stays where the rays are too few to fill the chip's warps more than twice and the
 // packets' unions are large, so that the longest one sets the time: through a wide aperture
-// (cocK >= 6) below 400k rays, and in scenes of 32k triangles and more below 300k.  Measured
+// (cocK >= 6) below 400k rays, or 600k while it is below 13 and the scene has 128k triangles and
+// more; and in scenes of 32k triangles and more below 300k.  Measured
 // (tracer + mask kernel, us; packets against one ray per lane at its former default order):
 //   35 mm f/2 (cocK 1.6), 1080p: 1 ray 171 / 277, 2 rays 232 / 491, 4 rays 409 / 919;
 //     768p, up to 4 rays by Eq. 4: 191 / 328
@@ -839,16 +840,23 @@ static void choose_lens_cells(int grid, BatchArgs &A) {
 //   85 mm f/1.2, 1080p (cocK 16): 1 ray 234 / 239, 4 rays 593 / 736; 4K (cocK 32) 583 / 733;
 //     720p, up to 8 rays (cocK 10.7): 634 in pixel order, 601 by lens cells / 645;
 //     540p, 1 ray (cocK 8): 137 / 110, 4 rays 219 / 227
+//   the same lens, whole frames: 540p, 4 rays, 190k triangles 358 / 349, 1M 451 / 389, 8 rays 628 / 584;
+//     1224 x 766 (cocK 10.2), 2 rays, 100k 372 / 375, 190k 421 / 410, 1M 483 / 440, 4 rays 649 / 593;
+//     1400 x 788 (cocK 11.7), 2 rays, 100k 407 / 424, 190k 459 / 455, 1M 543 / 495; 1080p, 1 ray,
+//     190k 594 / 621, 1M 655 / 665.  By cells against pixel order at cocK 10.2: 1M 483 / 536, 649 / 693,
+//     8 rays 912 / 963; at cocK 8 644 / 628.
 static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
-    double rays = 0, wide_rays = 0, dense_rays = 0;
+    double rays = 0, wide_rays = 0, wide_dense_rays = 0, dense_rays = 0;
     for (int s = 0; s < A.ns; s++) {
         const SessDesc &d = A.s[s];
         const double r = (double)d.N * (d.p.ray_mode ? 0.5 * d.p.m : (double)d.p.spp);
         rays += r;
         if (d.cam.cocK >= 6.f) wide_rays += r;
+        if (d.cam.cocK >= 6.f && d.cam.cocK < 13.f && d.sc.n_tris >= 131072) wide_dense_rays += r;
         if (d.sc.n_tris >= 32768) dense_rays += r;
     }
-    const bool few = (wide_rays > 0.5 * rays && rays < 400e3) || (dense_rays > 0.5 * rays && rays < 300e3);
+    const bool few = (wide_rays > 0.5 * rays && rays < 400e3) || (wide_dense_rays > 0.5 * rays && rays < 600e3) ||
+                     (dense_rays > 0.5 * rays && rays < 300e3);
     if (ctx->trace_packets >= 0) A.packets = ctx->trace_packets;
     else A.packets = !few;
     choose_lens_cells(ctx->ray_order_grid, A);
