@@ -815,6 +815,9 @@ static void choose_main_filter(const DofCtx *ctx, const DofFrameReq *reqs, uint3
     if (A.main_form == 3 && !ctx->gather_set) A.gather_h = 2;
 }
 
+// the rays a session's frame may take: all of its pixels masked, half of an adaptive budget
+static double step_rays(const SessDesc &d) { return (double)d.N * (d.p.ray_mode ? 0.5 * d.p.m : (double)d.p.spp); }
+
 // Lens-cell grid of each session's rays, by the tracer of the step: the caller's (grid), or where that
 // is open (0) the one that choose_tracer's figures favour.
 static void choose_lens_cells(int grid, BatchArgs &A) {
@@ -849,7 +852,7 @@ static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
     double rays = 0, wide_rays = 0, wide_dense_rays = 0, dense_rays = 0;
     for (int s = 0; s < A.ns; s++) {
         const SessDesc &d = A.s[s];
-        const double r = (double)d.N * (d.p.ray_mode ? 0.5 * d.p.m : (double)d.p.spp);
+        const double r = step_rays(d);
         rays += r;
         if (d.cam.cocK >= 6.f) wide_rays += r;
         if (d.cam.cocK >= 6.f && d.cam.cocK < 13.f && d.sc.n_tris >= 131072) wide_dense_rays += r;
@@ -912,26 +915,35 @@ static void enqueue_step(DofCtx *ctx, const BatchArgs &A, const AS &as, bool ada
     } else {
         // the ray path (A6 - A11) on the high-priority stream, the post-process filters
         // (A3 - A5, which only the composite reads) beside it on the caller's stream: the
-        // filters fill the SMs that the tracer's tail leaves idle.  The main filter waits for
-        // the mask, so that the tracer's blocks are placed first: launched before, the filter's
-        // long blocks kept the tracer's persistent ones off the SMs while the edge kernels of
-        // the adaptive mode ran (1080p, ten rays: 1.464 -> 1.397 ms; 768p, four: 0.443 -> 0.418).
-        // With lens-cell order the mask itself is long, and the prefilter waits as well (4K 3.413
-        // -> 3.383 ms; in pixel order it would leave the SMs idle: 1080p 0.559 -> 0.568).
+        // filters fill the SMs that the tracer's tail leaves idle.  Where many rays follow a long
+        // mask stage the main filter waits for the mask, so that the tracer's blocks are placed
+        // first: launched before, the filter's long blocks kept the tracer's persistent ones off the
+        // SMs while the edge kernels of the adaptive mode ran (1080p, ten rays: 1.464 -> 1.397 ms;
+        // 768p, four: 0.443 -> 0.418).  With lens-cell order the mask itself is long, and the
+        // prefilter waits as well (4K 3.413 -> 3.383 ms; in pixel order it would leave the SMs idle:
+        // 1080p 0.559 -> 0.568).  The rays are those the step may take at most: a frame that then
+        // traces none pays for the wait (1080p, adaptive 227 -> 254 us), so steps of fewer than 400k
+        // and those with one count per pixel in pixel order do not wait (540p without a ray: with
+        // the wait 80 -> 90 us).
         std::lock_guard<std::mutex> lock(ctx->launch_mu);
         cudaStream_t rs = ctx->ray_stream;
         bool cells = false;
-        for (int s = 0; s < A.ns; s++) cells |= A.s[s].lens_grid > 1;
+        double rays = 0;
+        for (int s = 0; s < A.ns; s++) {
+            cells |= A.s[s].lens_grid > 1;
+            rays += step_rays(A.s[s]);
+        }
+        const bool hold = (cells || adaptive) && rays >= 400e3;
         cudaEventRecord(ctx->ev_fork, st);
         cudaStreamWaitEvent(rs, ctx->ev_fork, 0);
         launch_mask_b(A, as, adaptive, rs, nullptr);
-        cudaEventRecord(ctx->ev_mask, rs);
+        if (hold) cudaEventRecord(ctx->ev_mask, rs);
         launch_trace_b(A, as, trace_blocks, rs, nullptr);
         launch_temporal_b(A, as, rs, nullptr);
         launch_recon_b(A, as, rs, nullptr);
         cudaEventRecord(ctx->ev_join, rs);
-        if (cells) cudaStreamWaitEvent(st, ctx->ev_mask, 0);
-        launch_pp_b(A, as, st, nullptr, ctx->ev_mask);
+        if (hold && cells) cudaStreamWaitEvent(st, ctx->ev_mask, 0);
+        launch_pp_b(A, as, st, nullptr, hold ? ctx->ev_mask : nullptr);
         cudaStreamWaitEvent(st, ctx->ev_join, 0);
         launch_composite_b(A, as, st, nullptr);
     }
