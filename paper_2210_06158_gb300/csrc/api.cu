@@ -408,6 +408,24 @@ extern "C" size_t dof_ctx_bytes_in_use(const DofCtx *ctx) { return ctx ? (size_t
 // scene
 // ---------------------------------------------------------------------------
 
+// The scene's samples, from the caller's arrays.
+static void sample_triangles(DofScene *s, const float *xyz, uint32_t n_verts, const uint32_t *idx) {
+    const uint32_t n = std::min<uint32_t>(s->n_tris, kSceneSamples);
+    for (uint32_t k = 0; k < n; k++) {
+        // multiples of the golden ratio: spread evenly, and out of step with a mesh's rows
+        const uint32_t *t = idx + 3 * (size_t)((uint64_t)(uint32_t)(k * 2654435769u) * s->n_tris >> 32);
+        if (t[0] >= n_verts || t[1] >= n_verts || t[2] >= n_verts) continue;
+        float *o = s->sample[s->n_samples++];
+        o[3] = 0.f;
+        for (int a = 0; a < 3; a++) {
+            const float p = xyz[3 * (size_t)t[0] + a], q = xyz[3 * (size_t)t[1] + a], r = xyz[3 * (size_t)t[2] + a];
+            const float lo = std::min(p, std::min(q, r)), hi = std::max(p, std::max(q, r));
+            o[a] = 0.5f * (lo + hi);
+            o[3] = std::max(o[3], hi - lo);
+        }
+    }
+}
+
 extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts, const uint32_t *tri_idx,
                                 const uint32_t *tri_mat, uint32_t n_tris, void *stream, DofScene **out) {
     if (!ctx || !out || (n_tris && (!xyz || !tri_idx || !n_verts)))
@@ -422,6 +440,7 @@ extern "C" int dof_scene_upload(DofCtx *ctx, const float *xyz, uint32_t n_verts,
     s->n_tris = n_tris;
     s->n_nodes = n_tris >= 2 ? n_tris - 1 : 0;
     int rc = DOF_OK;
+    sample_triangles(s, xyz, n_verts, tri_idx);
     if (n_tris == 0) { s->depth = 0; s->root = ~0; ctx_retain(ctx); *out = s; return DOF_OK; }
     {
         // one allocation for what every tree has (an allocation or a release costs the host 50 us),

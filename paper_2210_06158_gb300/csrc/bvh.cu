@@ -16,6 +16,7 @@
 #include "dof_internal.cuh"
 
 #include <algorithm>
+#include <cstring>
 
 namespace {
 
@@ -1493,16 +1494,16 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(const unsigned long
     }
 }
 
-// Stable sort of (keys, vals) by the key's low `bits` bits (a multiple of 16: an even
+// Stable sort of (keys, vals) by bits [from, to) of the keys (a multiple of 16 of them: an even
 // number of 8-bit passes); the result ends in (keys, vals), (keys2, vals2) and hist are
 // scratch (hist: 256 * ceil(n / 2048) ints, sums: ceil(256 * ceil(n / 2048) / 2048) ints).
 void device_radix_sort_pairs(unsigned long long *keys, uint32_t *vals, unsigned long long *keys2, uint32_t *vals2,
-                             int n, int *hist, int *sums, cudaStream_t st, int bits = 64) {
+                             int n, int *hist, int *sums, cudaStream_t st, int from = 0, int to = 64) {
     if (n <= 1) return;
     const int nb = (n + kSortTile - 1) / kSortTile;
     unsigned long long *ki = keys, *ko = keys2;
     uint32_t *vi = vals, *vo = vals2;
-    for (int shift = 0; shift < bits; shift += 8) {
+    for (int shift = from; shift < to; shift += 8) {
         k_rs_hist<<<nb, kSortThreads, 0, st>>>(ki, n, shift, hist, nb);
         device_exclusive_scan(hist, hist, kSortBins * nb, sums, st);
         k_rs_scatter<<<nb, kSortThreads, 0, st>>>(ki, vi, ko, vo, n, shift, hist, nb);
@@ -1523,7 +1524,7 @@ size_t sort_pairs_scratch_ints(int n) {
 void sort_pairs_by_low_bits(unsigned long long *keys, uint32_t *vals, unsigned long long *keys2, uint32_t *vals2,
                             int n, int bits, int *scratch, cudaStream_t st) {
     const size_t nh = (size_t)kSortBins * ((n + kSortTile - 1) / kSortTile);
-    device_radix_sort_pairs(keys, vals, keys2, vals2, n, scratch, scratch + nh, st, bits);
+    device_radix_sort_pairs(keys, vals, keys2, vals2, n, scratch, scratch + nh, st, 0, bits);
 }
 
 static inline unsigned blocks_for(size_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -1660,6 +1661,31 @@ int ploc_sah_build(const BuildScratch &b, DofScene *s, int m, int radius, int sm
     ck(cudaGetLastError(), "bvh kernels");
     return rc;
 }
+
+// The first key bit that the clustering round's sort looks at.  Its cells (10, 15 or 21 bits per axis
+// of the centroids' extent) are at most two of the scene's median triangles wide, so that the
+// order inside a cell, the input's, does not matter.  With ten bits whatever the scene, a lawn beside
+// one triangle 14 km away, its triangles shuffled, took 120 node visits per packet ray instead
+// of 58; with all of them every upload pays for eight passes instead of four (300k triangles 1565
+// -> 1672 us, six passes 1622).
+int cluster_key_from(const DofScene *s, const int *bounds) {
+    float e[kSceneSamples];
+    if (s->n_samples == 0) return 0;
+    for (int k = 0; k < s->n_samples; k++) e[k] = s->sample[k][3];
+    std::nth_element(e, e + s->n_samples / 2, e + s->n_samples);
+    const float median = e[s->n_samples / 2];
+    auto value = [](int o) {             // of an ordered int (ord_of)
+        const int i = o >= 0 ? o : o ^ 0x7FFFFFFF;
+        float f;
+        memcpy(&f, &i, sizeof(f));
+        return f;
+    };
+    float extent = 0.f;
+    for (int k = 0; k < 3; k++) extent = std::max(extent, value(bounds[3 + k]) - value(bounds[k]));
+    if (extent <= 2.f * 1024.f * median) return 32;
+    if (extent <= 2.f * 32768.f * median) return 16;
+    return 0;
+}
 }  // namespace
 
 int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint32_t *idx, const uint32_t *mat, int builder, int ploc_radius, int rotations, cudaStream_t st) {
@@ -1705,10 +1731,9 @@ int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint
         n_small = n - n_big;
         k_morton<<<blocks_for(n, B), B, 0, st>>>(b.cen, (uint32_t)n, separate ? b.ibuf + 9 : b.ibuf, b.ibuf, share, separate,
                                                  b.keys, b.vals);
-        // by the whole key: with its upper half alone (10 bits per axis) the clusters of a scene whose
-        // detail lies in a small part of its extent follow the order of the input, and a packet of a
-        // lawn beside one far triangle visits 120 nodes instead of 58 (7% less of the upload's time)
-        device_radix_sort_pairs(b.keys, b.vals, b.keys2, b.vals2, n, b.hist, b.sums, st);
+        // the radix tree needs the whole key, the clustering round as much of it as tells neighbours apart
+        device_radix_sort_pairs(b.keys, b.vals, b.keys2, b.vals2, n, b.hist, b.sums, st,
+                                ploc ? cluster_key_from(s, hbuf + (separate ? 9 : 0)) : 0, 64);
         // sorted (key, triangle) pairs are in (keys, vals)
         k_sorted_tris<<<blocks_for(n, B), B, 0, st>>>(d_xyz, d_idx, d_mat, (uint32_t)n, n_verts, b.vals, s->tris);
         const int m = n_small;

@@ -120,6 +120,8 @@ struct DofCtx {
     cudaMemPool_t pool;            // stream-ordered scratch of uploads and of the rasterising G-buffer producer
 };
 
+constexpr int kSceneSamples = 256;
+
 struct DofScene {
     DofCtx *ctx;
     uint32_t n_tris, n_nodes, depth;
@@ -135,6 +137,9 @@ struct DofScene {
     int32_t *prim_k;               // triangle id -> sorted index (n_tris)
     size_t bytes;
     float lo[3], hi[3];
+    // some triangles as the host gave them: centre of the box, the box's largest extent
+    int n_samples;
+    float sample[kSceneSamples][4];
 };
 
 struct DofHistory {
