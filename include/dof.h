@@ -203,8 +203,8 @@ size_t dof_ctx_bytes_in_use(const DofCtx *ctx);
 /* the tracer: 0 = one ray per lane, persistent threads with dynamic fetch, on the tree of
  * DOF_OPT_BVH_WIDTH; 1 = the 32 rays of a warp as one packet (one node sequence per warp, each
  * lane testing with its own ray and best hit), always on the binary tree.  Until it is set the
- * library chooses per step, by the aperture, the number of rays and the size of the
- * scenes.  Same hits either way */
+ * library chooses per step, by the aperture, the number of rays, the size of the scenes and
+ * how large their triangles appear in the blurred foreground.  Same hits either way */
 #define DOF_OPT_TRACE_PACKETS       12
 /* passes of tree rotations after the BVH build of scenes uploaded afterwards, 0..16
  * (default 0): each swaps, bottom-up, a child with a grandchild where that shrinks the

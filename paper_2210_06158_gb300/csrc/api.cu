@@ -9,6 +9,7 @@
 #include "batch.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 int post_init_tables();
 int recon_init_tables();
@@ -416,13 +417,19 @@ static void sample_triangles(DofScene *s, const float *xyz, uint32_t n_verts, co
         const uint32_t *t = idx + 3 * (size_t)((uint64_t)(uint32_t)(k * 2654435769u) * s->n_tris >> 32);
         if (t[0] >= n_verts || t[1] >= n_verts || t[2] >= n_verts) continue;
         float *o = s->sample[s->n_samples++];
+        float u[3], v[3];
         o[3] = 0.f;
         for (int a = 0; a < 3; a++) {
             const float p = xyz[3 * (size_t)t[0] + a], q = xyz[3 * (size_t)t[1] + a], r = xyz[3 * (size_t)t[2] + a];
+            u[a] = q - p;
+            v[a] = r - p;
             const float lo = std::min(p, std::min(q, r)), hi = std::max(p, std::max(q, r));
             o[a] = 0.5f * (lo + hi);
             o[3] = std::max(o[3], hi - lo);
         }
+        const double nx = (double)u[1] * v[2] - (double)u[2] * v[1], ny = (double)u[2] * v[0] - (double)u[0] * v[2],
+                     nz = (double)u[0] * v[1] - (double)u[1] * v[0];
+        o[4] = (float)std::sqrt(std::sqrt(nx * nx + ny * ny + nz * nz));
     }
 }
 
@@ -522,6 +529,71 @@ static SceneDev scene_dev(const DofScene *s) {
 // G-buffer producer
 // ---------------------------------------------------------------------------
 
+// scenes of fewer triangles are traced by packets whatever their size (their trees are shallow)
+constexpr uint32_t kFineMinTris = 8192;
+
+// A scene's sampled triangles as a camera sees them: where a packet's rays spread over more than a
+// few triangles, the packet steps through the union of what each of its rays needs, and one
+// ray per lane is the faster tracer by up to three times.  `near` keeps the triangles whose blur
+// reaches the mask and measures them against what a packet covers there, a patch of the image
+// and the blur's width (pixel order: 8 x 4 half-resolution pixels; lens cells: a mask block,
+// and 1/8 of the blur); else they are measured in pixels.  Their size is the root of twice the
+// area (the edge of a mesh's cell).  Spheres of 20k to 2.6M triangles at 1, 3 and 10 m, three
+// lenses, 360p and 1080p: frames by packets take 0.82 to 1.04 of the other's time where the
+// median triangle is from 0.5 of a packet's width on, 0.93 to 1.1 near 0.35, 1.1 to 1.4 near 0.25 and
+// up to 3.1 below (1M triangles, 35 mm, 1080p: 704 / 401 us, four rays 1355 / 808).  The lawn
+// workloads are far from the line: at most 0.46 of the triangles of their near field are below
+// it (a few spheres behind the lawn), and the rule wants seven in ten.
+struct MeshView {
+    int seen = 0, fine = 0;
+    double area = 0;                         // of the rectangle that holds the small ones, px
+};
+static MeshView mesh_view(const DofScene *s, const DevCam &c, bool near, float mask_hpx, bool cells) {
+    MeshView v;
+    double sx = 0, sy = 0, sxx = 0, syy = 0;
+    for (int k = 0; k < s->n_samples; k++) {
+        const float *t = s->sample[k];
+        const float rx = t[0] - c.O.x, ry = t[1] - c.O.y, rz = t[2] - c.O.z;
+        const float z = rx * c.F.x + ry * c.F.y + rz * c.F.z;
+        if (!(z > 1e-6f)) continue;
+        const float g = c.Fpx / z;
+        const float x = g * (rx * c.R.x + ry * c.R.y + rz * c.R.z), y = g * (rx * c.U.x + ry * c.U.y + rz * c.U.z);
+        if (!(std::fabs(x) <= c.halfW && std::fabs(y) <= c.halfH)) continue;
+        const float blur = c.cocK * (c.d - z) / z;
+        if (near && !(blur >= 4.f * mask_hpx)) continue;
+        v.seen++;
+        if (!(g * t[4] < (near ? 0.33f * (cells ? 64.f + 0.125f * blur : 16.f + blur) : 8.f))) continue;
+        v.fine++;
+        if (near) continue;
+        sx += x; sy += y; sxx += (double)x * x; syy += (double)y * y;
+    }
+    if (v.fine > 0) {
+        const double n = v.fine, wx = std::max(0.0, sxx / n - sx / n * (sx / n)), wy = std::max(0.0, syy / n - sy / n * (sy / n));
+        v.area = std::min(12.0 * std::sqrt(wx * wy), (double)c.W * c.H);
+    }
+    return v;
+}
+
+// Few pixels in a dense scene take one ray per lane: their packets span wide angles, visit the union
+// of what the rays need, and the longest one sets the time.  Line: four pixels per triangle, and
+// 180,000 pixels.  Measured (us, packets / one ray per lane; lawn of that many triangles): 2.8k
+// 64 x 36 51 / 47, 160 x 90 36 / 44; 10k 160 x 90 65 / 54, 400 x 224 51 / 59; 30k 320 x 180 67 / 63,
+// 480 x 270 59 / 70; 60k 480 x 270 79 / 77, 640 x 360 71 / 83; 250k 64 x 36 165 / 57, 560 x 316 98 / 90,
+// 640 x 360 92 / 102; 500k 320 x 180 128 / 82, 560 x 316 114 / 98, 640 x 360 106 / 119; 1M through the
+// 85 mm lens 560 x 316 131 / 96, 640 x 360 113 / 109, 800 x 450 125 / 138.
+// The same holds where a fine mesh (triangles below 8 pixels, all but 15% of those in view) covers
+// part of the image: packets while its triangles are fewer than the square of the pixels it
+// covers by 500,000.  Spheres, both sides counted (us, packets / one ray per lane): 110k px, 20k
+// triangles 104 / 103, 58k 188 / 152; 223k px, 160k 237 / 206, 360k 307 / 218; 437k px, 360k 269 / 280,
+// 1M 469 / 371; 645k px, 2.6M 862 / 656; the whole image, 1M 355 / 546.
+static bool primary_packets(const DofScene *s, const DevCam &cam) {
+    const double px = (double)cam.W * cam.H;
+    if (px < 180000 && px < 4.0 * s->n_tree) return false;
+    if (s->n_tree < kFineMinTris) return true;
+    const MeshView v = mesh_view(s, cam, false, 0.f, false);
+    return v.fine <= 0.85 * v.seen || (double)s->n_tree * v.fine / s->n_samples < v.area * v.area / 5e5;
+}
+
 extern "C" int dof_gbuffer(DofCtx *ctx, const DofScene *scene, const DofCamera *cam, const DofParams *p,
                            uint32_t width, uint32_t height, float *color, float *depth, float *normal, int32_t *prim,
                            void *stream) {
@@ -540,7 +612,8 @@ extern "C" int dof_gbuffer(DofCtx *ctx, const DofScene *scene, const DofCamera *
     if (rc) return rc;
     cudaGetLastError();   // drop a stale error of an earlier call of another library on this thread
     launch_primary(dc, dp, scene_dev(scene), reinterpret_cast<float4 *>(color), depth,
-                   reinterpret_cast<float4 *>(normal), prim, ctx->d_status, (cudaStream_t)stream);
+                   reinterpret_cast<float4 *>(normal), prim, primary_packets(scene, dc),
+                   ctx->d_status, (cudaStream_t)stream);
     return dof_cuda_check(cudaGetLastError(), "dof_gbuffer launch");
 }
 
@@ -839,11 +912,12 @@ static double step_rays(const SessDesc &d) { return (double)d.N * (d.p.ray_mode 
 
 // Lens-cell grid of each session's rays, by the tracer of the step: the caller's (grid), or where that
 // is open (0) the one that choose_tracer's figures favour.
+static int lens_cells(int grid, bool packets, const SessDesc &d) {
+    const float k = d.cam.cocK;
+    return grid ? grid : (packets ? (k >= 10.f ? 8 : 1) : (k >= 6.f ? 4 : 1));
+}
 static void choose_lens_cells(int grid, BatchArgs &A) {
-    for (int s = 0; s < A.ns; s++) {
-        const float k = A.s[s].cam.cocK;
-        A.s[s].lens_grid = grid ? grid : (A.packets ? (k >= 10.f ? 8 : 1) : (k >= 6.f ? 4 : 1));
-    }
+    for (int s = 0; s < A.ns; s++) A.s[s].lens_grid = lens_cells(grid, A.packets != 0, A.s[s]);
 }
 
 // The tracer of a step whose context leaves it open: warp packets, taken in pixel order, but
@@ -852,8 +926,8 @@ static void choose_lens_cells(int grid, BatchArgs &A) {
 // per lane stays where the rays are too few to fill the chip's warps more than twice and the
 // packets' unions are large, so that the longest one sets the time: through a wide aperture
 // (cocK >= 6) below 400k rays, or 600k while it is below 13 and the scene has 128k triangles and
-// more; and in scenes of 32k triangles and more below 300k.  Measured
-// (tracer + mask kernel, us; packets against one ray per lane at its former default order):
+// more; in scenes of 32k triangles and more below 300k; and where the near field is a fine mesh
+// (mesh_view).  Measured (tracer + mask kernel, us; packets against one ray per lane at its former default order):
 //   35 mm f/2 (cocK 1.6), 1080p: 1 ray 171 / 277, 2 rays 232 / 491, 4 rays 409 / 919;
 //     768p, up to 4 rays by Eq. 4: 191 / 328
 //   the same lens, one ray (tracer alone, pixel order): 360p 114 / 92, 540p 127 / 106, 720p 137 /
@@ -867,8 +941,8 @@ static void choose_lens_cells(int grid, BatchArgs &A) {
 //     1400 x 788 (cocK 11.7), 2 rays, 100k 407 / 424, 190k 459 / 455, 1M 543 / 495; 1080p, 1 ray,
 //     190k 594 / 621, 1M 655 / 665.  By cells against pixel order at cocK 10.2: 1M 483 / 536, 649 / 693,
 //     8 rays 912 / 963; at cocK 8 644 / 628.
-static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
-    double rays = 0, wide_rays = 0, wide_dense_rays = 0, dense_rays = 0;
+static void choose_tracer(const DofCtx *ctx, const DofFrameReq *reqs, BatchArgs &A) {
+    double rays = 0, wide_rays = 0, wide_dense_rays = 0, dense_rays = 0, fine_rays = 0;
     for (int s = 0; s < A.ns; s++) {
         const SessDesc &d = A.s[s];
         const double r = step_rays(d);
@@ -877,8 +951,17 @@ static void choose_tracer(const DofCtx *ctx, BatchArgs &A) {
         if (d.cam.cocK >= 6.f && d.cam.cocK < 13.f && d.sc.n_tris >= 131072) wide_dense_rays += r;
         if (d.sc.n_tris >= 32768) dense_rays += r;
     }
-    const bool few = (wide_rays > 0.5 * rays && rays < 400e3) || (wide_dense_rays > 0.5 * rays && rays < 600e3) ||
-                     (dense_rays > 0.5 * rays && rays < 300e3);
+    bool few = (wide_rays > 0.5 * rays && rays < 400e3) || (wide_dense_rays > 0.5 * rays && rays < 600e3) ||
+               (dense_rays > 0.5 * rays && rays < 300e3);
+    if (ctx->trace_packets < 0 && !few) {
+        for (int s = 0; s < A.ns; s++) {
+            const SessDesc &d = A.s[s];
+            if (reqs[s].scene->n_tree < kFineMinTris) continue;
+            const MeshView v = mesh_view(reqs[s].scene, d.cam, true, d.p.mask_near_hpx, lens_cells(ctx->ray_order_grid, true, d) > 1);
+            if (v.fine > 0.7 * v.seen) fine_rays += step_rays(d);
+        }
+        few = fine_rays > 0.5 * rays;
+    }
     if (ctx->trace_packets >= 0) A.packets = ctx->trace_packets;
     else A.packets = !few;
     choose_lens_cells(ctx->ray_order_grid, A);
@@ -912,7 +995,7 @@ static int build_batch(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, BatchAr
     A.cursor = &reqs[0].hist->counters[2];
     A.refill_idle = ctx->trace_refill_idle;
     A.steps_per_round = ctx->trace_steps;
-    choose_tracer(ctx, A);
+    choose_tracer(ctx, reqs, A);
     A.stats = ctx->trace_stats;
     A.stack_depth = ctx->stack_depth;
     return DOF_OK;

@@ -137,9 +137,10 @@ struct DofScene {
     int32_t *prim_k;               // triangle id -> sorted index (n_tris)
     size_t bytes;
     float lo[3], hi[3];
-    // some triangles as the host gave them: centre of the box, the box's largest extent
+    // some triangles as the host gave them: centre of the box, the box's largest extent, and the
+    // square root of twice the triangle's area
     int n_samples;
-    float sample[kSceneSamples][4];
+    float sample[kSceneSamples][5];
 };
 
 struct DofHistory {
@@ -218,7 +219,7 @@ int dof_scratch(DofCtx *ctx, size_t bytes, void **ptr, cudaStream_t st, const ch
 // xyz, idx, mat: host arrays
 int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint32_t *idx, const uint32_t *mat, int builder, int ploc_radius, int rotations, cudaStream_t st);
 void launch_primary(const DevCam &cam, const DevParams &p, const SceneDev &sc, float4 *color, float *depth, float4 *normal,
-                    int32_t *prim, uint32_t *status, cudaStream_t st);
+                    int32_t *prim, bool packets, uint32_t *status, cudaStream_t st);
 // host-side tally of this library's kernel launches (dof_launch_count); each launch
 // wrapper adds the launches it enqueued
 void count_launches(long long n);

@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(kPrimaryThreads, 8) k_primary(const __grid_con
     if (act) store_primary(cam, p, sc, o, (size_t)j * cam.W + i, d, h);
 }
 
-// The same image by one ray per lane, for few pixels in a dense scene (few_primary).
+// The same image by one ray per lane, for few pixels in a dense scene and for fine meshes
+// (primary_packets).
 __global__ void __launch_bounds__(kPrimaryThreads) k_primary_lanes(const __grid_constant__ DevCam cam,
                                                                    const __grid_constant__ DevParams p,
                                                                    const __grid_constant__ SceneDev sc,
@@ -993,24 +994,12 @@ __global__ void __launch_bounds__(128) k_shade(const __grid_constant__ AS as_) {
 
 }  // namespace
 
-// Few pixels in a dense scene take one ray per lane: their packets span wide angles, visit the union
-// of what the rays need, and the longest one sets the time.  Line: four pixels per triangle, and
-// 180,000 pixels.  Measured (us, packets / one ray per lane; lawn of that many triangles): 2.8k
-// 64 x 36 51 / 47, 160 x 90 36 / 44; 10k 160 x 90 65 / 54, 400 x 224 51 / 59; 30k 320 x 180 67 / 63,
-// 480 x 270 59 / 70; 60k 480 x 270 79 / 77, 640 x 360 71 / 83; 250k 64 x 36 165 / 57, 560 x 316 98 / 90,
-// 640 x 360 92 / 102; 500k 320 x 180 128 / 82, 560 x 316 114 / 98, 640 x 360 106 / 119; 1M through the
-// 85 mm lens 560 x 316 131 / 96, 640 x 360 113 / 109, 800 x 450 125 / 138.
-static bool few_primary(const DevCam &cam, const SceneDev &sc) {
-    const long long px = (long long)cam.W * cam.H;
-    return px < 180000 && px < 4ll * sc.n_tris;
-}
-
 void launch_primary(const DevCam &cam, const DevParams &p, const SceneDev &sc, float4 *color, float *depth, float4 *normal,
-                    int32_t *prim, uint32_t *status, cudaStream_t st) {
+                    int32_t *prim, bool packets, uint32_t *status, cudaStream_t st) {
     const dim3 g((cam.W + 15) / 16, (cam.H + 7) / 8);
     const PrimaryOut o{color, depth, normal, prim};
-    if (few_primary(cam, sc)) k_primary_lanes<<<g, kPrimaryThreads, 0, st>>>(cam, p, sc, o, status);
-    else k_primary<<<g, kPrimaryThreads, 0, st>>>(cam, p, sc, o);
+    if (packets) k_primary<<<g, kPrimaryThreads, 0, st>>>(cam, p, sc, o);
+    else k_primary_lanes<<<g, kPrimaryThreads, 0, st>>>(cam, p, sc, o, status);
     count_launches(1);
 }
 

@@ -56,3 +56,27 @@ def test_tiny_scenes_with_few_pixels(n):
         torch.cuda.synchronize()
         for k in want:
             assert torch.equal(want[k], got[k]), (k, W, H)
+
+
+def test_a_fine_mesh_over_part_of_the_image():
+    """A ball of 60k triangles of a few pixels over a tenth of the image takes one ray per lane where the
+    image alone would not: the same bits."""
+    import numpy as np
+    import torch
+    from paper_2210_06158_gb300 import dof
+    from synth import Camera, Scene, camera_pose
+    rng = np.random.default_rng(4)
+    d = rng.normal(size=(60_000, 3))
+    at = np.array([0.4, 0.2, 10.0]) + d / np.linalg.norm(d, axis=1, keepdims=True)
+    v = (at[:, None, :] + 0.01 * rng.uniform(-1, 1, (60_000, 3, 3))).astype(np.float32).reshape(-1, 3)
+    ctx = dof.Context(0)
+    sc = dof.Scene(ctx, Scene(v, np.arange(len(v), dtype=np.uint32).reshape(-1, 3), np.zeros(len(v) // 3, np.uint32), 1))
+    cam = Camera.from_poses(dict(f_m=0.035, f_number=2.0, focus_m=10.0, sensor_w_m=0.036), camera_pose((0.0, 0.0, 0.0), 0.0))
+    prm = make_workload("c2", W=64, H=36, n_frames=1).params
+    for W, H in ((1280, 720), (1922, 1082)):
+        want = dof.gbuffer(ctx, sc, cam, prm, W, H, raster=True)
+        got = dof.gbuffer(ctx, sc, cam, prm, W, H)
+        torch.cuda.synchronize()
+        assert int((want["prim"] >= 0).sum()) > 10_000
+        for k in want:
+            assert torch.equal(want[k], got[k]), (k, W, H)

@@ -67,3 +67,38 @@ def test_few_rays_through_a_wide_lens_stay_one_per_lane_in_a_dense_scene(share, 
             assert h.stats().rays > 100_000
             assert (h.stats().node_visits > 0) == lanes
     assert torch.equal(images[0], images[1]) and torch.equal(images[0], images[2])
+
+
+@pytest.mark.parametrize("centre,lanes", [((0.0, 0.0, 1.0), True), ((0.0, 0.0, 12.0), False)])
+def test_a_fine_mesh_in_the_blurred_foreground_is_traced_one_ray_per_lane(centre, lanes):
+    """A ball of 20k small triangles in front of (or behind, where it takes no ray) a wall of 800
+    large ones near the camera: its triangles are a fraction of what a packet covers.  518k rays, so
+    that no other rule speaks; the image is the same either way."""
+    import numpy as np
+    import torch
+    from paper_2210_06158_gb300 import dof
+    from synth import Camera, Scene, camera_pose
+    rng = np.random.default_rng(3)
+    d = rng.normal(size=(20_000, 3))
+    at = np.asarray(centre) + 0.3 * d / np.linalg.norm(d, axis=1, keepdims=True)
+    ball = at[:, None, :] + 0.004 * rng.uniform(-1, 1, (20_000, 3, 3))
+    wall = rng.uniform((-1.5, -1, 2.0), (1.5, 1, 2.5), (800, 3))[:, None, :] + 0.3 * rng.uniform(-1, 1, (800, 3, 3))
+    v = np.concatenate([ball, wall] if lanes else [np.repeat(wall, 20, 0), ball[:4000]]).astype(np.float32).reshape(-1, 3)
+    scene = Scene(v, np.arange(len(v), dtype=np.uint32).reshape(-1, 3), np.zeros(len(v) // 3, np.uint32), 1)
+    cam = Camera.from_poses(dict(f_m=0.035, f_number=2.0, focus_m=10.0, sensor_w_m=0.036), camera_pose((0.0, 0.0, 0.0), 0.0))
+    prm = dict(make_workload("c2", W=64, H=36, n_frames=1).params, spp=1)
+    images = []
+    for setting in (None, dict(packets=0), dict(packets=1)):
+        ctx = dof.Context(0)
+        ctx.set_trace(stats=False)
+        if setting:
+            ctx.set_trace(**setting)
+        sc = dof.Scene(ctx, scene)
+        gb = dof.gbuffer(ctx, sc, cam, prm, 1920, 1080)
+        h = dof.History(ctx, 1920, 1080, max_rays=1)
+        images.append(dof.frame(ctx, sc, gb, cam, prm, h))
+        torch.cuda.synchronize()
+        if setting is None:
+            assert h.stats().rays > 10_000
+            assert (h.stats().node_visits > 0) == lanes
+    assert torch.equal(images[0], images[1]) and torch.equal(images[0], images[2])
