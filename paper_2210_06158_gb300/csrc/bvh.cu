@@ -1334,16 +1334,13 @@ __global__ void __launch_bounds__(128) k_collapse(const BvhNode *nodes, int n_bi
 
 // what the host needs to know of the finished tree
 struct TreeSummary {
-    int bad, depth, root, clusters, n_seg[2];
+    int bad, depth, root;
     float lo[3], hi[3];                  // the root's box
 };
-__global__ void k_summary(const int *ibuf, const SahState *st, const int *root, const BvhNode *nodes, int n_nodes, TreeSummary *o) {
+__global__ void k_summary(const int *ibuf, const int *root, const BvhNode *nodes, int n_nodes, TreeSummary *o) {
     o->bad = ibuf[6];
     o->depth = ibuf[7];
     o->root = *root;
-    o->clusters = st->count;
-    o->n_seg[0] = st->n_seg[0];
-    o->n_seg[1] = st->n_seg[1];
     if (*root >= 0 && *root < n_nodes) {
         const BvhNode nd = nodes[*root];
         o->lo[0] = fminf(nd.a.x, nd.a.z); o->lo[1] = fminf(nd.b.x, nd.b.z); o->lo[2] = fminf(nd.c.x, nd.c.z);
@@ -1777,7 +1774,7 @@ int launch_bvh_build(DofScene *s, const float *xyz, uint32_t n_verts, const uint
                 for (int k = 0; k < 16 && levels4 < kCollapseLevels; k++, levels4++)
                     k_collapse<<<2 * sms, 128, 0, st>>>(s->nodes, m - 1, b.front[levels4 & 1], b.n4 + 1 + levels4, b.wide, m - 1,
                                                        b.n4, b.front[(levels4 + 1) & 1], b.n4 + 2 + levels4, b.ibuf + 6);
-                k_summary<<<1, 1, 0, st>>>(b.ibuf, b.state, b.root, s->nodes, m - 1, b.summary);
+                k_summary<<<1, 1, 0, st>>>(b.ibuf, b.root, s->nodes, m - 1, b.summary);
                 ck(cudaMemcpyAsync(n_front, b.n4, sizeof(n_front), cudaMemcpyDeviceToHost, st), "bvh readback");
                 ck(cudaMemcpyAsync(&sum, b.summary, sizeof(sum), cudaMemcpyDeviceToHost, st), "bvh readback");
                 ck(cudaGetLastError(), "bvh kernels");
