@@ -354,13 +354,14 @@ int dof_batch_frame(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, void *stre
  * parameters, G-buffer and output pointers may change between launches.
  *   dof_graph_create: validates `reqs` as dof_batch_frame and captures (nothing runs,
  *     the histories do not advance).  The graph keeps the histories and their order,
- *     the launch shapes (sizes, ray modes, spp / m, tree kinds, the main filter's
- *     shared-memory tile, which follows max_coc_px) and the context's tracer options of
- *     that moment.
+ *     the launch shapes (sizes, ray modes, spp / m, the gathers' blocks and forms, the
+ *     main filter's shared-memory tile, which follows max_coc_px), the tracer, chosen or
+ *     set (with one ray per lane also the kind of tree), and the tracer's options.
  *   dof_graph_launch: one step, results identical to dof_batch_frame on the same
- *     requests.  DOF_ERR_MISMATCH if the requests need other launch shapes or other
- *     histories than the capture.  Launches of one graph on different streams are
- *     ordered by the library (one graph runs one step at a time).
+ *     requests.  DOF_ERR_MISMATCH if the requests or the options set since need other
+ *     launch shapes, another tracer or other histories than the capture, or a scene's
+ *     tree is deeper than the captured packets' stack.  Launches of one graph on
+ *     different streams are ordered by the library (one graph runs one step at a time).
  *   dof_graph_destroy: waits for the graph's last launch and frees it. */
 typedef struct DofGraph DofGraph;
 int dof_graph_create(DofCtx *ctx, const DofFrameReq *reqs, uint32_t n, DofGraph **out);

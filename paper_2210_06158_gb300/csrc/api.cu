@@ -535,15 +535,16 @@ constexpr uint32_t kFineMinTris = 8192;
 // A scene's sampled triangles as a camera sees them: where a packet's rays spread over more than a
 // few triangles, the packet steps through the union of what each of its rays needs, and one
 // ray per lane is the faster tracer by up to three times.  `near` keeps the triangles whose blur
-// reaches the mask and measures them against what a packet covers there, a patch of the image
-// and the blur's width (pixel order: 8 x 4 half-resolution pixels; lens cells: a mask block,
-// and 1/8 of the blur); else they are measured in pixels.  Their size is the root of twice the
-// area (the edge of a mesh's cell).  Spheres of 20k to 2.6M triangles at 1, 3 and 10 m, three
-// lenses, 360p and 1080p: frames by packets take 0.82 to 1.04 of the other's time where the
-// median triangle is from 0.5 of a packet's width on, 0.93 to 1.1 near 0.35, 1.1 to 1.4 near 0.25 and
-// up to 3.1 below (1M triangles, 35 mm, 1080p: 704 / 401 us, four rays 1355 / 808).  The lawn
-// workloads are far from the line: at most 0.46 of the triangles of their near field are below
-// it (a few spheres behind the lawn), and the rule wants seven in ten.
+// reaches half the mask's threshold (the mask spreads over neighbouring tiles) and measures them
+// against what a packet covers there, a patch of the image and the blur's width (pixel order:
+// 8 x 4 half-resolution pixels; lens cells: a mask block, and 1/8 of the blur); else they are
+// measured in pixels.  Their size is the root of twice the area (the edge of a mesh's cell).
+// Spheres of 20k to 2.6M triangles at 1, 3 and 10 m, three lenses, 360p and 1080p: frames by
+// packets take 0.82 to 1.04 of the other's time where the median triangle is from 0.5 of a packet's
+// width on, 0.93 to 1.1 near 0.35, 1.1 to 1.4 near 0.25 and up to 3.1 below (1M triangles, 35 mm,
+// 1080p: 704 / 401 us, four rays 1355 / 808).  The lawn workloads are far from the line: at most 0.46
+// of the triangles of their near field are below it (a few spheres behind the lawn), and the rule
+// wants seven in ten.
 struct MeshView {
     int seen = 0, fine = 0;
     double area = 0;                         // of the rectangle that holds the small ones, px
@@ -560,7 +561,7 @@ static MeshView mesh_view(const DofScene *s, const DevCam &c, bool near, float m
         const float x = g * (rx * c.R.x + ry * c.R.y + rz * c.R.z), y = g * (rx * c.U.x + ry * c.U.y + rz * c.U.z);
         if (!(std::fabs(x) <= c.halfW && std::fabs(y) <= c.halfH)) continue;
         const float blur = c.cocK * (c.d - z) / z;
-        if (near && !(blur >= 4.f * mask_hpx)) continue;
+        if (near && !(blur >= 2.f * mask_hpx)) continue;
         v.seen++;
         if (!(g * t[4] < (near ? 0.33f * (cells ? 64.f + 0.125f * blur : 16.f + blur) : 8.f))) continue;
         v.fine++;

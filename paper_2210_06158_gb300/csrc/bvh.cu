@@ -4,7 +4,8 @@
 // Both builders start from the triangles sorted by the 63-bit Morton codes of their
 // centroids (21 bits per axis: scenes with a ground plane hundreds of metres wide still
 // resolve centimetre detail; a stable LSD radix sort written here, 8-bit digits,
-// warp-matched ranks).  The default one joins neighbours in one round of PLOC clustering
+// warp-matched ranks), the default one by as many of the upper bits as its triangles' size
+// asks for (cluster_key_from).  The default one joins neighbours in one round of PLOC clustering
 // and splits the clusters top-down by a binned surface-area heuristic.  The other is the
 // LBVH after Karras, "Maximizing Parallelism in the Construction of BVHs, Octrees, and
 // k-d Trees" (HPG 2012): one thread per internal node finds its key range and split

@@ -29,6 +29,8 @@ SPACE = {
     "steps": [8, 16, 32, 64],
     "packets": [0, 1],
 }
+# where a search starts: one setting for all sessions, not what an untouched context runs (which
+# chooses tracer, ray order and main-filter form per step)
 DEFAULT = {"bvh_width": 4, "ray_grid": 4, "stack": 96, "blocks_per_sm": 8, "refill_idle": 16, "steps": 64,
            "packets": 0}
 
@@ -158,9 +160,9 @@ def tune_gathers(ctx, run_frame, frames=4, rounds=2, stream=None):
     return best, seen
 
 
-# PLOC search radii tried per scene: on the grass workloads the tree quality does not
-# follow the radius (node tests per ray vary by up to a third between neighbouring
-# radii), so several are built and the fastest kept
+# Search radii of the clustering round tried per scene.  With the surface-area splits on top the
+# radius moves the tree little (about 70 node tests per packet at 496k grass triangles whatever it
+# is); what is left does not follow the radius, so several are built and the fastest kept
 SCENE_RADII = [8, 12, 16, 24, 32, 40, 48, 56, 64, 96, 128, 192]
 
 
