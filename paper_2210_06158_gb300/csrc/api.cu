@@ -1025,9 +1025,9 @@ static void enqueue_step(DofCtx *ctx, const BatchArgs &A, const AS &as, bool ada
         // 768p, four: 0.443 -> 0.418).  With lens-cell order the mask itself is long, and the
         // prefilter waits as well (4K 3.413 -> 3.383 ms; in pixel order it would leave the SMs idle:
         // 1080p 0.559 -> 0.568).  The rays are those the step may take at most: a frame that then
-        // traces none pays for the wait (1080p, adaptive 227 -> 254 us), so steps of fewer than 400k
-        // and those with one count per pixel in pixel order do not wait (540p without a ray: with
-        // the wait 80 -> 90 us).
+        // traces none pays for the wait (1080p, adaptive 227 -> 254 us), so steps of few rays (900 x 386,
+        // up to six by Eq. 4, 260k: with the wait 326 -> 316 us; 540p by lens cells without a ray, 130k:
+        // 80 -> 90) and those with one count per pixel in pixel order do not wait.
         std::lock_guard<std::mutex> lock(ctx->launch_mu);
         cudaStream_t rs = ctx->ray_stream;
         bool cells = false;
@@ -1036,7 +1036,7 @@ static void enqueue_step(DofCtx *ctx, const BatchArgs &A, const AS &as, bool ada
             cells |= A.s[s].lens_grid > 1;
             rays += step_rays(A.s[s]);
         }
-        const bool hold = (cells || adaptive) && rays >= 400e3;
+        const bool hold = (cells && rays >= 400e3) || (adaptive && rays >= 200e3);
         cudaEventRecord(ctx->ev_fork, st);
         cudaStreamWaitEvent(rs, ctx->ev_fork, 0);
         launch_mask_b(A, as, adaptive, rs, nullptr);
